@@ -166,6 +166,7 @@ struct SmallGroup {  // small runs of one lattice size, annealed by anneal_small
 struct SweepGroup {  // runs of one lattice size among the resident runs
     uint32_t L = 0;
     int any_glass = 0;
+    uint32_t theta_max = 0;
     std::vector<uint32_t> runs;
     uint64_t runs_off = 0;               // in d_meta
     std::vector<uint64_t> tile_map_off;  // per candidate, in d_meta (n + 1 entries)
@@ -782,6 +783,7 @@ pa_status rebuild(pa_engine *e)
         SweepGroup &g = e->groups[it->second];
         g.runs.push_back(s);
         if (e->rd[s].model == PA_EA_PMJ) g.any_glass = 1;
+        g.theta_max = std::max(g.theta_max, e->rd[s].theta);
     }
     for (auto &g : e->groups) {
         const Tuning &t = e->tuning[g.L];
@@ -889,7 +891,7 @@ void launch_group_sweep(pa_engine *e, const SweepGroup &g, uint32_t c)
 {
     const Tuning &t = e->tuning[g.L];
     launch_sweep(e->P, meta(e, g.runs_off), meta(e, g.tile_map_off[c]), (uint32_t)g.runs.size(), g.n_tiles[c],
-                 t.candidates[c], g.any_glass, e->stream);
+                 t.candidates[c], g.any_glass, g.theta_max, e->stream);
 }
 
 // beta_0 draws of the pending runs (Sec. II.B step (i)) and their step-0 measurement.

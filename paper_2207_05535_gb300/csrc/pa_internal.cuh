@@ -113,7 +113,10 @@ struct SweepCfg {
     uint32_t G;      // Philox groups per colour = ceil(N / 8)
     uint32_t PS;     // bytes per colour plane = 4 G (byte planes); the row pitch (padded or compact rows)
     uint32_t smem;   // dynamic shared memory bytes
-    uint32_t WPT;    // fast kernel: plane words per thread
+    uint32_t WPT;    // bit-sliced kernels: plane words per thread
+    uint32_t TH;     // half-sweeps of shared Philox parts held in shared memory (0: none)
+    uint32_t K;      // consecutive tiles one CTA works through (set by launch_sweep)
+    uint32_t Lh, pw; // compact rows: L/2 and words of a stored plane
 };
 
 // Row pitch of a colour plane: L/2 when that is a power of two; else the
@@ -197,7 +200,7 @@ void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_run
 // the bit-sliced kernel applies.
 std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast);
 void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *tile_off, uint32_t n_group_runs,
-                  uint32_t n_tiles, const SweepCfg &cfg, int any_glass, cudaStream_t s);
+                  uint32_t n_tiles, const SweepCfg &cfg, int any_glass, uint32_t theta_max, cudaStream_t s);
 void launch_overlap(const Pool &P, const uint32_t *q_runs, uint32_t n_q_runs, uint32_t max_Rcap, int init,
                     cudaStream_t s);
 // run_ctas(R_cap) CTAs per run (at most run_ctas(max_Rcap)); also prepares the

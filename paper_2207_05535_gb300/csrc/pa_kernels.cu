@@ -1004,17 +1004,23 @@ __global__ void __launch_bounds__(MAXT) sweep_kernel(Pool P, const uint32_t *gro
 // above, row below) from the other plane, the unsatisfied bonds
 // x_d = s ^ n_d ^ J_d, their count with a bit-sliced adder (c0 = count & 1,
 // ge2 = count >= 2), and the acceptance mask
-//      accept = ge2 | (c0 & B1) | B2,   B_m = [u < T_m]  (T_2 <= T_1),
+//      accept = ge2 | [u < T],   T = T_1 where c0, else T_2  (T_2 <= T_1),
 // i.e. dE = 8 - 4 count <= 0, or u < T_1 when dE = 4, or u < T_2 when dE = 8.
 // The 32 uniforms come from 8 Philox calls with the same counters as the
 // generic kernel, so both kernels (and the oracle) flip the same spins.
 // E and M of the child are recomputed from its final planes.
 //
-// Throughput (GB300): Philox4x32-10 dominates.  Each round is two
-// 32x32->64 multiplies (multiplier pipe, half rate, two passes each) and two
-// 3-input XORs (integer pipe); the multiplier bounds the kernel at about
-// 40 multiply-add slots per Philox call.  The round keys are precomputed and
-// the first round's multiply of the temperature counter is hoisted.
+// Throughput (GB300): Philox4x32-10 dominates.  A 32x32->64 multiply holds the multiplier
+// for 4 cycles of an SM sub-partition and, measured beside xors, also the integer ALU for 2; every
+// xor, compare and shift holds the ALU for 2.  So a warp's Philox call costs about
+// 2 (products + ALU instructions) cycles and the way to a faster sweep is fewer of both: the
+// products that do not change from call to call are taken out (SharedPart, ChildPart: 14 of 19
+// left with a table, 16 without) and each uniform is compared once, with the threshold its site's
+// bonds select, instead of with T_1 and T_2 (8 ALU instructions and 4 adds fewer per call, against
+// one byte permute and one 16-byte shared-memory load).  Measured (theta = 10, 40 runs, 4e8 spins):
+// L = 8, 16, 32: 1610 -> 1903, 1608 -> 1877, 1605 -> 1818 updates/ns; L = 64, 128, 256: 1549 ->
+// 1790, 1536 -> 1788, 1455 -> 1665; per warp and call at L = 16: 62 -> 50 instructions, 100 -> 86
+// cycles, of which ALU and products explain 2 (26 + 14) = 80.
 // --------------------------------------------------------------------------
 struct PhiloxKeys {
     uint32_t k0[10], k1[10];
@@ -1071,171 +1077,340 @@ __device__ __forceinline__ uint4 philox_rk(uint32_t c0, uint32_t c1, uint32_t c3
     return make_uint4(x0, x1, x2, x3);
 }
 
-template <bool SG, int WPT>
-__device__ __forceinline__ void sweep_pow2_body(const Pool &P, const uint32_t *group_runs, const uint32_t *tile_off,
-                                                uint32_t n_group_runs, const SweepCfg &cfg)
+// A sweep's Philox calls have counters (g, j, i, tag | h): group g of the colour plane, child
+// j, temperature i, half-sweep h.  Over a launch i is fixed, a thread's j and its word's eight
+// g's are fixed, and h runs.  Word 0 of the second round then depends on j alone and its
+// word 2 on (g, h) alone, so of the first three rounds' six products
+//   M1 i and M0 g are constants,
+//   M0 x0 of round 2 belongs to the child, M1 x2 of round 3 to (child, g): fixed over h,
+//   M1 x2 of round 2 and M0 x0 of round 3 belong to (g, h): the same for every child.
+// SharedPart holds what belongs to (g, h), ChildPart what belongs to (child, g); a call is one
+// xor of each pair and the last seven rounds, 14 products instead of 19.
+struct SharedPart {
+    uint32_t lo1, hi0, lo0;  // lo(M1 x2) of round 2; M0 x0 of round 3
+};
+
+__device__ __forceinline__ SharedPart philox_shared(uint32_t g, uint32_t ctr3, uint32_t lo1_0, const PhiloxKeys &K)
 {
-    extern __shared__ __align__(16) uint32_t smw[];
-    const uint32_t slot = locate_slot(tile_off, n_group_runs, blockIdx.x);
-    const uint32_t run = group_runs[slot];
-    const RunDev rd = P.runs[run];
-    const RunState st = P.st[run];
-    if (st.status) return;
-    const uint32_t i = st.step + 1;
-    if (i >= rd.n_beta) return;
-    const uint32_t Rn = st.R_new;
-    const uint32_t tile0 = (blockIdx.x - tile_off[slot]) * cfg.RPC;
-    if (tile0 >= Rn) return;  // uniform over the CTA
+    const uint32_t x2 = __umulhi(0xD2511F53u, g) ^ ctr3 ^ K.k1[0];
+    const unsigned long long p1 = 0xCD9E8D57ull * x2;
+    const uint32_t y0 = (uint32_t)(p1 >> 32) ^ lo1_0 ^ K.k0[1];
+    const unsigned long long p0 = 0xD2511F53ull * y0;
+    return SharedPart{(uint32_t)p1, (uint32_t)(p0 >> 32), (uint32_t)p0};
+}
 
-    const uint32_t TPR = cfg.TPR, HW = TPR * WPT;  // threads per replica, words per plane
-    const uint32_t Lh = rd.Lh, N = rd.N;
-    const uint32_t rloc = threadIdx.x / TPR, tl = threadIdx.x & (TPR - 1);
-    const uint32_t child = tile0 + rloc;
-    const bool active = child < Rn;
-    uint32_t *pl = smw + rloc * 2 * HW;
-    int32_t *acc = reinterpret_cast<int32_t *>(smw + cfg.RPC * 2 * HW);
-    const bool wide = TPR > 32;
-    if (wide && threadIdx.x < 2 * cfg.RPC) acc[threadIdx.x] = 0;
+struct ChildPart {
+    uint32_t x2;         // lo(M0 x0) of round 2 with the key: xored with SharedPart.hi0
+    uint32_t a[8], b[8]; // per group: hi(M1 x2) of round 3 with the key, and lo
+};
 
-    const uint32_t ob = (i - 1) & 1u, nbuf = i & 1u;
-    uint32_t own[WPT][2];
-    uint32_t parent = 0;
-    if (active) parent = P.parent[rd.rep_off + child];
-    const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent * rd.wstride;
+__device__ __forceinline__ void philox_child(ChildPart &c, uint32_t g0, uint32_t child, uint32_t hi1_0,
+                                             const PhiloxKeys &K)
+{
+    const unsigned long long pc = 0xD2511F53ull * (hi1_0 ^ child ^ K.k0[0]);
+    c.x2 = (uint32_t)pc ^ K.k1[2];
 #pragma unroll
-    for (int q = 0; q < WPT; ++q) {
-        const uint32_t w = tl + q * TPR;
-        own[q][0] = active ? src[w] : 0u;
-        own[q][1] = active ? src[HW + w] : 0u;
-        pl[w] = own[q][0];
-        pl[HW + w] = own[q][1];
+    for (uint32_t q = 0; q < 8; ++q) {
+        const uint32_t y2 = (uint32_t)(pc >> 32) ^ (0xD2511F53u * (g0 + q)) ^ K.k1[1];
+        const unsigned long long p = 0xCD9E8D57ull * y2;
+        c.a[q] = (uint32_t)(p >> 32) ^ K.k0[2];
+        c.b[q] = (uint32_t)p;
     }
-    uint32_t J[WPT][2][4];
+}
+
+// The call of group q of the word: rounds 4 to 10 from the two parts.
+__device__ __forceinline__ uint4 philox_join(const ChildPart &c, uint32_t q, const SharedPart &v, const PhiloxKeys &K)
+{
+    uint32_t x0 = c.a[q] ^ v.lo1, x1 = c.b[q], x2 = v.hi0 ^ c.x2, x3 = v.lo0;
 #pragma unroll
-    for (int q = 0; q < WPT; ++q)
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int d = 0; d < 4; ++d) J[q][c][d] = 0;
-    if (SG) {
+    for (int r = 3; r < 10; ++r) {
+        const unsigned long long p0 = 0xD2511F53ull * x0, p1 = 0xCD9E8D57ull * x2;
+        x0 = (uint32_t)(p1 >> 32) ^ x1 ^ K.k0[r];
+        x1 = (uint32_t)p1;
+        x2 = (uint32_t)(p0 >> 32) ^ x3 ^ K.k1[r];
+        x3 = (uint32_t)p0;
+    }
+    return make_uint4(x0, x1, x2, x3);
+}
+
+// The shared parts of TH half-sweeps from h0 on for groups 0 .. 8 HW - 1, in shared memory as
+// [half-sweep][group in its word][word]: a warp writes and reads consecutive 16-byte entries.
+__device__ __forceinline__ void fill_shared_parts(uint4 *tab, uint32_t HW, uint32_t h0, uint32_t TH, uint32_t lo1_0,
+                                                  const PhiloxKeys &K)
+{
+    const uint32_t n = 8 * HW * TH;
+    uint32_t hq = 0, w = threadIdx.x;  // 8 half-sweep + group in its word; word
+    for (uint32_t e = threadIdx.x; e < n; e += blockDim.x, w += blockDim.x) {
+        while (w >= HW) {
+            w -= HW;
+            ++hq;
+        }
+        const SharedPart v = philox_shared(8 * w + (hq & 7u), (TAG_SWEEP << 24) | (h0 + (hq >> 3)), lo1_0, K);
+        tab[e] = make_uint4(v.lo1, v.hi0, v.lo0, 0u);
+    }
+}
+
+// Metropolis thresholds by site.  A site with an odd number of unsatisfied bonds (bit of c0
+// set) flips when u < T_1, one with none when u < T_2, and the others flip whatever u is: so
+// one comparison per site is enough, against the threshold its bit of c0 selects.  s_thr[n]
+// holds the four thresholds of a Philox group whose bits of c0 are n.
+__device__ __forceinline__ void fill_thresholds(uint4 *s_thr, uint32_t t1, uint32_t t2)
+{
+    if (threadIdx.x < 16) {
+        const uint32_t n = threadIdx.x;
+        s_thr[n] = make_uint4(n & 1u ? t1 : t2, n & 2u ? t1 : t2, n & 4u ? t1 : t2, n & 8u ? t1 : t2);
+    }
+}
+
+// The low and high nibbles of c0's bytes, each times 16: byte offsets into s_thr.
+struct SiteNibbles {
+    uint32_t lo, hi;
+};
+__device__ __forceinline__ SiteNibbles site_nibbles(uint32_t c0)
+{
+    return SiteNibbles{(c0 << 4) & 0xF0F0F0F0u, c0 & 0xF0F0F0F0u};
+}
+
+// Bits 4 q .. 4 q + 3 of B: u below the thresholds of the group's sites.
+__device__ __forceinline__ void accept_group(uint32_t &B, const uint4 &u, uint32_t q, const SiteNibbles &n,
+                                             const uint4 *s_thr)
+{
+    const uint32_t off = __byte_perm(q & 1u ? n.hi : n.lo, 0u, 0x4440u | (q >> 1));
+    const uint4 T = *reinterpret_cast<const uint4 *>(reinterpret_cast<const char *>(s_thr) + off);
+    or_if_below(B, u.x, T.x, 1u << (4 * q));
+    or_if_below(B, u.y, T.y, 2u << (4 * q));
+    or_if_below(B, u.z, T.z, 4u << (4 * q));
+    or_if_below(B, u.w, T.w, 8u << (4 * q));
+}
+
+// Number of unsatisfied bonds of each site, bit-sliced: parity and "at least two".
+__device__ __forceinline__ void count_bonds(uint32_t x1, uint32_t x2, uint32_t x3, uint32_t x4, uint32_t &c0,
+                                            uint32_t &ge2)
+{
+    const uint32_t s = x1 ^ x2 ^ x3, m = (x1 & x2) | (x1 & x3) | (x2 & x3);
+    c0 = s ^ x4;
+    ge2 = m | (s & x4);
+}
+
+// HW: words of a colour plane (L = 8 sqrt(HW)); WPT: plane words per thread.
+// TAB: the shared parts come from a table in shared memory, cfg.TH half-sweeps at a time, that
+// every child of the CTA reads; otherwise each thread forms them, which is faster from L = 64 on:
+// a table of a few children's CTA costs more to fill than it saves (L = 64, 4 children: 1616
+// against 1786 updates/ns; L = 128, 4 children: 1455 against 1788).
+// With one word per thread the word, its bond masks and its child parts stay in registers (128
+// of them, two CTAs of 256 threads per SM; a cap at 80 or 64 for more warps is 3 to 7 % slower);
+// with several (L = 256) they are read from shared memory (bond masks: global) as each word is
+// swept, so that two CTAs share an SM: 1665 updates/ns, against 1605 for one CTA of 1024 threads.
+// MANY: a CTA works through cfg.K tiles (launch_sweep says when).
+// Two children per thread, to share the shared parts in registers, spill at 128 registers: 2 %
+// slower at L = 64 and 128.
+template <bool SG, uint32_t HW, uint32_t WPT, bool TAB, bool MANY, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const uint32_t *group_runs,
+                                                                const uint32_t *tile_off, uint32_t n_group_runs,
+                                                                SweepCfg cfg)
+{
+    constexpr uint32_t Lh = HW == 1 ? 4 : HW == 4 ? 8 : HW == 16 ? 16 : HW == 64 ? 32 : HW == 256 ? 64 : 128;
+    static_assert(Lh * Lh == 16 * HW, "L = 2 Lh, N = 64 HW");
+    constexpr uint32_t N = 64 * HW, TPR = HW / WPT;  // sites; threads per replica
+    constexpr bool WIDE = TPR > 32;                  // a replica spans several warps
+    constexpr bool MULTI = WPT > 1;
+    extern __shared__ __align__(16) uint32_t smw[];  // TAB: the table; MULTI: child parts; planes; sums
+    __shared__ uint4 s_thr[16];
+    const uint32_t rloc = threadIdx.x / TPR, tl = threadIdx.x % TPR;
+    uint4 *tab = reinterpret_cast<uint4 *>(smw);
+    uint2 *ab = reinterpret_cast<uint2 *>(smw) + rloc * 8 * HW;  // MULTI: [group in its word][word]
+    uint32_t *planes = smw + (TAB ? cfg.TH * 32 * HW : MULTI ? cfg.RPC * 16 * HW : 0);
+    uint32_t *pl = planes + rloc * 2 * HW;
+    int32_t *acc = reinterpret_cast<int32_t *>(planes + cfg.RPC * 2 * HW);
+
+    uint32_t tile = MANY ? blockIdx.x * cfg.K : blockIdx.x;
+    const uint32_t tend = MANY ? min(tile + cfg.K, tile_off[n_group_runs]) : tile + 1;
+    uint32_t slot = locate_slot(tile_off, n_group_runs, tile);
+    while (tile < tend) {
+        if (MANY)
+            while (tile_off[slot + 1] <= tile) ++slot;
+        const uint32_t first = tile_off[slot], stop = MANY ? min(tend, tile_off[slot + 1]) : tend;
+        const uint32_t run = group_runs[slot];
+        const RunDev rd = P.runs[run];
+        const RunState st = P.st[run];
+        const uint32_t i = st.step + 1, Rn = st.R_new;
+        if (st.status || i >= rd.n_beta || (tile - first) * cfg.RPC >= Rn) {  // uniform over the CTA
+            if (!MANY) return;
+            tile = stop;
+            continue;
+        }
+        // ---- the run: thresholds, keys, bond masks, the table's first half-sweeps
+        const uint32_t ob = (i - 1) & 1u, nbuf = i & 1u, H = 2 * rd.theta;
         const uint32_t *Jp = P.J + rd.J_off + 2 * rd.wstride;
+        uint32_t J[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
+        auto bonds = [&](uint32_t c, uint32_t w) {
 #pragma unroll
-        for (int q = 0; q < WPT; ++q)
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int d = 0; d < 4; ++d) J[q][c][d] = Jp[(c * 4 + d) * HW + tl + q * TPR];
-    }
-    const unsigned long long T1 = P.thr[rd.thr_off + 2 * i], T2 = P.thr[rd.thr_off + 2 * i + 1];
-    const uint32_t t1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T1;
-    const uint32_t t2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T2;
-    const uint32_t all1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
-    const uint32_t all2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
-    PhiloxKeys K;
-    philox_keys(K, rd.seed, rd.run_id);
-    const uint32_t hi1_0 = __umulhi(0xCD9E8D57u, i), lo1_0 = 0xCD9E8D57u * i;
-    if (TPR <= 32) __syncwarp(); else __syncthreads();
+            for (int d = 0; d < 4; ++d) J[c][d] = Jp[(c * 4 + d) * HW + w];
+        };
+        if (SG && !MULTI) {
+            bonds(0, tl);
+            bonds(1, tl);
+        }
+        const unsigned long long T1 = P.thr[rd.thr_off + 2 * i], T2 = P.thr[rd.thr_off + 2 * i + 1];
+        const uint32_t t1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T1;
+        const uint32_t t2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T2;
+        const uint32_t all1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
+        const uint32_t all2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
+        PhiloxKeys K;
+        philox_keys(K, rd.seed, rd.run_id);
+        const uint32_t hi1_0 = __umulhi(0xCD9E8D57u, i), lo1_0 = 0xCD9E8D57u * i;
+        if (MANY) __syncthreads();  // the tiles of the run before are done with the shared memory
+        fill_thresholds(s_thr, t1, t2);
+        uint32_t in_tab = min(cfg.TH, H);  // half-sweeps in the table, from tab_h on
+        uint32_t tab_h = 0;
+        if (TAB) fill_shared_parts(tab, HW, 0, in_tab, lo1_0, K);
+        const uint4 *tp = tab;
 
-    auto neighbours = [&](uint32_t c, uint32_t w, uint32_t &same, uint32_t &rot, uint32_t &up, uint32_t &dn) {
-        plane_neighbours(pl + (c ^ 1u) * HW, HW, Lh, c, w, same, rot, up, dn);
-    };
-
-    for (uint32_t t = 0; t < rd.theta; ++t) {
+        // Word w of colour c in half-sweep h: the new spins.
+        ChildPart cp;
+        auto sweep_word = [&](uint32_t c, uint32_t w, uint32_t h, uint32_t S) {
+            uint32_t same, rot, up, dn, c0, ge2;
+            plane_neighbours(pl + (c ^ 1u) * HW, HW, Lh, c, w, same, rot, up, dn);
+            count_bonds(S ^ same ^ J[c][0], S ^ rot ^ J[c][1], S ^ up ^ J[c][2], S ^ dn ^ J[c][3], c0, ge2);
+            const SiteNibbles nib = site_nibbles(c0);
+            uint32_t B = 0;
 #pragma unroll
-        for (uint32_t c = 0; c < 2; ++c) {
-            if (active) {
-                const uint32_t ctr3 = (TAG_SWEEP << 24) | (t << 1) | c;
-#pragma unroll
-                for (int q = 0; q < WPT; ++q) {
-                    const uint32_t w = tl + q * TPR;
-                    uint32_t same, rot, up, dn;
-                    neighbours(c, w, same, rot, up, dn);
-                    const uint32_t S = own[q][c];
-                    const uint32_t x1 = S ^ same ^ J[q][c][0], x2 = S ^ rot ^ J[q][c][1];
-                    const uint32_t x3 = S ^ up ^ J[q][c][2], x4 = S ^ dn ^ J[q][c][3];
-                    const uint32_t a = x1 ^ x2, b = x1 & x2, e = x3 ^ x4, f = x3 & x4;
-                    const uint32_t c0 = a ^ e, ge2 = b | f | (a & e);
-                    // bits of distinct sites never collide, so the packing can add or or
-                    uint32_t B1 = 0, B2 = 0;
-#pragma unroll
-                    for (uint32_t g = 0; g < 8; ++g) {
-                        const uint4 u = philox_rk<true>(8 * w + g, child, ctr3, hi1_0, lo1_0, K);
-                        pack_group(B1, B2, u, g, t1, t2);
-                    }
-                    const uint32_t flip = ge2 | (c0 & (B1 | all1)) | B2 | all2;
-                    own[q][c] = S ^ flip;
+            for (uint32_t q = 0; q < 8; ++q) {
+                SharedPart v;
+                if (TAB) {
+                    const uint4 e = tp[q * HW];
+                    v = SharedPart{e.x, e.y, e.z};
+                } else {
+                    v = philox_shared(8 * w + q, (TAG_SWEEP << 24) | h, lo1_0, K);
                 }
-                // all of this colour's words are updated before any is published
-#pragma unroll
-                for (int q = 0; q < WPT; ++q) pl[c * HW + tl + q * TPR] = own[q][c];
+                if (MULTI) {
+                    const uint2 e = ab[q * HW + w];
+                    cp.a[q] = e.x;
+                    cp.b[q] = e.y;
+                }
+                accept_group(B, philox_join(cp, q, v, K), q, nib, s_thr);
             }
-            if (TPR <= 32) __syncwarp(); else __syncthreads();
-        }
-    }
+            return S ^ (ge2 | B | (c0 & all1) | all2);
+        };
 
-    // child: planes, E from the final lattice (every bond touches one colour-0 site), M
-    int32_t unsat = 0, up1 = 0;
-    if (active) {
-        uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)child * rd.wstride;
+        for (; tile < stop; ++tile) {
+            const uint32_t tile0 = (tile - first) * cfg.RPC;
+            if (MANY && tile0 >= Rn) {  // uniform over the CTA
+                tile = stop;
+                break;
+            }
+            const uint32_t child = tile0 + rloc;
+            const bool active = child < Rn;
+            uint32_t own[2] = {0u, 0u}, parent = 0;
+            if (active) parent = P.parent[rd.rep_off + child];
+            const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent * rd.wstride;
+            if (MULTI) {
+                for (uint32_t w = tl; w < HW; w += TPR) {
+                    philox_child(cp, 8 * w, child, hi1_0, K);
 #pragma unroll
-        for (int q = 0; q < WPT; ++q) {
-            const uint32_t w = tl + q * TPR;
-            dst[w] = own[q][0];
-            dst[HW + w] = own[q][1];
-            uint32_t same, rot, up, dn;
-            neighbours(0, w, same, rot, up, dn);
-            const uint32_t S = own[q][0];
-            unsat += __popc(S ^ same ^ J[q][0][0]) + __popc(S ^ rot ^ J[q][0][1]) + __popc(S ^ up ^ J[q][0][2]) +
-                     __popc(S ^ dn ^ J[q][0][3]);
-            up1 += __popc(own[q][0]) + __popc(own[q][1]);
-        }
-    }
-    if (!wide) {
-        for (uint32_t o = 1; o < TPR; o <<= 1) {
-            unsat += __shfl_xor_sync(FULL, unsat, o);
-            up1 += __shfl_xor_sync(FULL, up1, o);
-        }
-    } else {
-        if (active) {
-            atomicAdd(&acc[2 * rloc], unsat);
-            atomicAdd(&acc[2 * rloc + 1], up1);
-        }
-        __syncthreads();
-        unsat = acc[2 * rloc];
-        up1 = acc[2 * rloc + 1];
-    }
-    if (active && tl == 0) {
-        const uint64_t pc = rd.rep_off + parent, cc = rd.rep_off + child;
-        P.E[nbuf][cc] = 2 * unsat - 2 * (int32_t)N;
-        P.M[nbuf][cc] = 2 * up1 - (int32_t)N;
-        P.fam[nbuf][cc] = P.fam[ob][pc];
-    }
-}
+                    for (uint32_t q = 0; q < 8; ++q) ab[q * HW + w] = make_uint2(cp.a[q], cp.b[q]);
+                }
+            } else {
+                philox_child(cp, 8 * tl, child, hi1_0, K);
+            }
+            if (WIDE && tl == 0) acc[2 * rloc] = acc[2 * rloc + 1] = 0;
+#pragma unroll
+            for (uint32_t q = 0; q < 2 * WPT; ++q) {
+                const uint32_t v = active ? src[q * TPR + tl] : 0u;
+                if (!MULTI) own[q & 1u] = v;  // one word per thread: q is the colour
+                pl[q * TPR + tl] = v;
+            }
+            if (MANY && TAB && tab_h != 0) {  // a schedule longer than the table: back to its start
+                __syncthreads();
+                fill_shared_parts(tab, HW, 0, in_tab = min(cfg.TH, H), lo1_0, K);
+                tab_h = 0;
+            }
+            tp = tab + tl;
+            // the thresholds, the table and, where a replica spans warps, its planes
+            __syncthreads();
 
-// The kernels: the compiler's own register choice for 256 and 1024 threads
-// (78 and 40 registers; an explicit bound of one CTA per SM let it take 150 at
-// 256 threads and run 19 % slower at L = 128), two CTAs per SM for 512 threads
-// (L = 256: +5 % against one, measured).
-template <bool SG, int WPT, int MAXT>
-__global__ void __launch_bounds__(MAXT) sweep_pow2_kernel(Pool P, const uint32_t *group_runs, const uint32_t *tile_off,
-                                                          uint32_t n_group_runs, SweepCfg cfg)
-{
-    sweep_pow2_body<SG, WPT>(P, group_runs, tile_off, n_group_runs, cfg);
-}
+            for (uint32_t t = 0; t < rd.theta; ++t) {
+#pragma unroll
+                for (uint32_t c = 0; c < 2; ++c) {
+                    const uint32_t h = 2 * t + c;
+                    if (TAB && h - tab_h == in_tab) {  // uniform over the CTA
+                        __syncthreads();
+                        tab_h = h;
+                        in_tab = min(cfg.TH, H - h);
+                        fill_shared_parts(tab, HW, h, in_tab, lo1_0, K);
+                        tp = tab + tl;
+                        __syncthreads();
+                    }
+                    // replicas beyond the population (zero planes) are swept along and not stored
+                    if (MULTI) {  // a half-sweep reads only the other plane: words are published as they are done
+#pragma unroll 1
+                        for (uint32_t w = tl; w < HW; w += TPR) {
+                            if (SG) bonds(c, w);
+                            pl[c * HW + w] = sweep_word(c, w, h, pl[c * HW + w]);
+                        }
+                    } else {
+                        own[c] = sweep_word(c, tl, h, own[c]);
+                        pl[c * HW + tl] = own[c];
+                    }
+                    if (TAB) tp += 8 * HW;
+                    if (WIDE)
+                        __syncthreads();
+                    else
+                        __syncwarp();
+                }
+            }
 
-template <bool SG, int WPT>
-__global__ void __launch_bounds__(512, 2) sweep_pow2_kernel_2cta(Pool P, const uint32_t *group_runs,
-                                                                 const uint32_t *tile_off, uint32_t n_group_runs,
-                                                                 SweepCfg cfg)
-{
-    sweep_pow2_body<SG, WPT>(P, group_runs, tile_off, n_group_runs, cfg);
+            // child: planes, E from the final lattice (every bond touches one colour-0 site), M
+            int32_t unsat = 0, up1 = 0;
+            if (active) {
+                uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)child * rd.wstride;
+#pragma unroll
+                for (uint32_t q = 0; q < WPT; ++q) {
+                    const uint32_t w = q * TPR + tl;
+                    const uint32_t S = MULTI ? pl[w] : own[0], S1 = MULTI ? pl[HW + w] : own[1];
+                    dst[w] = S;
+                    dst[HW + w] = S1;
+                    if (SG && MULTI) bonds(0, w);
+                    uint32_t same, rot, up, dn;
+                    plane_neighbours(pl + HW, HW, Lh, 0, w, same, rot, up, dn);
+                    unsat += __popc(S ^ same ^ J[0][0]) + __popc(S ^ rot ^ J[0][1]) + __popc(S ^ up ^ J[0][2]) +
+                             __popc(S ^ dn ^ J[0][3]);
+                    up1 += __popc(S) + __popc(S1);
+                }
+            }
+            if (!WIDE) {
+#pragma unroll
+                for (uint32_t o = 1; o < TPR; o <<= 1) {
+                    unsat += __shfl_xor_sync(FULL, unsat, o);
+                    up1 += __shfl_xor_sync(FULL, up1, o);
+                }
+            } else {
+                if (active) {
+                    atomicAdd(&acc[2 * rloc], unsat);
+                    atomicAdd(&acc[2 * rloc + 1], up1);
+                }
+                __syncthreads();
+                if (tl == 0) {
+                    unsat = acc[2 * rloc];
+                    up1 = acc[2 * rloc + 1];
+                }
+            }
+            if (active && tl == 0) {
+                const uint64_t pc = rd.rep_off + parent, cc = rd.rep_off + child;
+                P.E[nbuf][cc] = 2 * unsat - 2 * (int32_t)N;
+                P.M[nbuf][cc] = 2 * up1 - (int32_t)N;
+                P.fam[nbuf][cc] = P.fam[ob][pc];
+            }
+            if (!MANY) return;
+            if (!WIDE) __syncwarp();  // the planes are read before the next tile's are stored
+        }
+    }
 }
 
 // --------------------------------------------------------------------------
-// Bit-sliced sweep for even L whose half-width L/2 is not a power of two but
-// at most 31 (Sec. V.A.1): rows of a colour plane are padded to a pitch P in
-// {4, 8, 16, 32} with L P a multiple of 32, so rows tile 32-bit words exactly
-// as in the power-of-two kernel; padding bits are masked out of every flip
+// Bit-sliced sweep with padded rows, used for L = 12 (Sec. V.A.1): rows of a
+// colour plane are padded to a pitch P in {8, 16, 32} with L P a multiple of 32,
+// so rows tile 32-bit words exactly as in the power-of-two kernel; padding bits are masked out of every flip
 // and popcount and stay 0.  Each thread owns one plane word (32 / P rows); its
 // sites are the compact sublattice indices [kb, kb + (32 / P) L/2), drawn from
 // the same Philox counters as every other path (the groups at either end of
@@ -1436,14 +1611,17 @@ __global__ void __launch_bounds__(256, PA_PAD_MIN_BLOCKS) sweep_pad_kernel(Pool 
 // in the words of the first and last rows only, at the wrapped positions.  A
 // plane's string starts after FP = ceil(L/64) words and is followed by
 // L/64 + 2 words, so every window stays inside the array; bits read from those
-// margins are always masked out.  Both this kernel and the padded-row kernel
-// are launch-shape candidates for L <= 64 (the padded rows are faster for some
-// small L, whose compact planes end in a mostly empty word).
+// margins are always masked out.  The geometry and the bond masks of every word
+// are formed once per CTA in shared memory; a word's flips are formed as in the
+// power-of-two kernel, each thread with its own shared parts (a table of them is
+// slower here, 1367 against 1415 updates/ns at L = 30).  A barrier ends every
+// half-sweep; the block sizes tried are those that fill whole groups of four warps
+// best, as an SM's four sub-partitions share a CTA's warps evenly then (L = 100: 471
+// threads 1357 updates/ns, 157 threads 1160 at 2 CTAs' worth of registers).  Four
+// CTAs of 256 threads per SM (64 registers): 128 registers are 1 to 9 % slower.
+// Measured (theta = 10, as above): L = 20 glass 1146 -> 1324 updates/ns, L = 30
+// 1293 -> 1422, L = 46 1256 -> 1435, L = 100 1247 -> 1345.
 // --------------------------------------------------------------------------
-#ifndef PA_COMPACT_WIDE
-#define PA_COMPACT_WIDE true
-#endif
-
 __device__ __forceinline__ uint32_t low_bits(uint32_t n) { return n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u; }
 
 // 32 bits of the bit string s from bit p on (words p >> 5 and p >> 5 + 1 exist).
@@ -1482,8 +1660,8 @@ __device__ uint32_t padded_from_compact(const uint32_t *O, uint32_t base, uint32
     return x0 < Lh ? bits_at(O, base + y * Lh + x0) & low_bits(Lh - x0) : 0u;
 }
 
-// Per-thread geometry of compact word w.
-struct CompactWord {
+// Geometry of compact word w.
+struct __align__(16) CompactWord {
     uint32_t RS, RE, EV, VM;  // row starts, row ends, even rows, sites of the plane
     uint32_t mU, mD;          // bits whose row above (below) is the lattice's last (first) row
     uint32_t pU, pD;          // window positions of the wrapped rows (the plain ones where none wraps)
@@ -1561,121 +1739,152 @@ __device__ __forceinline__ void compact_neighbours(const uint32_t *O, const uint
     const uint32_t left = (l1 & ~g.RS) | (lw & g.RS);   // x' - 1 within the row
     const uint32_t right = (r1 & ~g.RE) | (rw & g.RE);  // x' + 1 within the row
     rot = c == 0 ? ((left & g.EV) | (right & ~g.EV)) : ((right & g.EV) | (left & ~g.EV));
-    if (g.mU) up = (up & ~g.mU) | (bits_at(O, g.pU) & g.mU);  // the first row's row above: the last row
-    if (g.mD) dn = (dn & ~g.mD) | (bits_at(O, g.pD) & g.mD);  // the last row's row below: the first row
+    // without branches: a divergent branch here would keep the compiler from drawing the first
+    // Philox groups while these loads are in flight
+    up = (up & ~g.mU) | (bits_at(O, g.pU) & g.mU);  // the first row's row above: the last row
+    dn = (dn & ~g.mD) | (bits_at(O, g.pD) & g.mD);  // the last row's row below: the first row
 }
 
-#ifndef PA_COMPACT_MIN_BLOCKS
-#define PA_COMPACT_MIN_BLOCKS 4  // caps registers at 64 (no spills); 1-8 % faster than 3 or 2 CTAs of 256 (measured)
-#endif
-
-template <bool SG, int MAXT, bool NARROW>
-__global__ void __launch_bounds__(MAXT, MAXT <= 256 ? PA_COMPACT_MIN_BLOCKS : 1)
+template <bool SG, int MAXT, int MINB, bool NARROW>
+__global__ void __launch_bounds__(MAXT, MINB)
     sweep_compact_kernel(Pool P, const uint32_t *group_runs, const uint32_t *tile_off, uint32_t n_group_runs,
                          SweepCfg cfg)
 {
-    extern __shared__ __align__(16) uint32_t smw[];
-    const uint32_t slot = locate_slot(tile_off, n_group_runs, blockIdx.x);
-    const uint32_t run = group_runs[slot];
-    const RunDev rd = P.runs[run];
-    const RunState st = P.st[run];
-    if (st.status) return;
-    const uint32_t i = st.step + 1;
-    if (i >= rd.n_beta) return;
-    const uint32_t Rn = st.R_new;
-    const uint32_t tile0 = (blockIdx.x - tile_off[slot]) * cfg.RPC;
-    if (tile0 >= Rn) return;  // uniform over the CTA
+    extern __shared__ __align__(16) uint32_t smw[];  // geometry, bond masks (SG), planes, sums
+    __shared__ uint4 s_thr[16];
+    uint32_t tile = blockIdx.x * cfg.K;
+    const uint32_t tend = min(tile + cfg.K, tile_off[n_group_runs]);
+    uint32_t slot = locate_slot(tile_off, n_group_runs, tile);
 
     const uint32_t CW = cfg.TPR;  // compact words per plane = threads per replica
-    const uint32_t Lh = rd.Lh, N = rd.N, NB = N / 2, pitch = rd.pitch, PW = rd.pw;
+    const uint32_t Lh = cfg.Lh, N = 4 * Lh * Lh, NB = N / 2, pitch = cfg.PS, PW = cfg.pw;
     const uint32_t FP = (Lh + 31) >> 5, AW = FP + CW + (Lh >> 5) + 2, base = 32 * FP;
     const uint32_t rloc = threadIdx.x / CW, w = threadIdx.x - rloc * CW;
-    const uint32_t child = tile0 + rloc;
-    const bool active = child < Rn;
-    uint32_t *pl = smw + rloc * 2 * AW;
-    int32_t *acc = reinterpret_cast<int32_t *>(smw + cfg.RPC * 2 * AW);
-    for (uint32_t q = threadIdx.x; q < 2 * cfg.RPC; q += blockDim.x) acc[q] = 0;  // one thread per replica at L <= 6
-
-    const uint32_t ob = (i - 1) & 1u, nbuf = i & 1u;
-    uint32_t own[2] = {0u, 0u}, parent = 0;
-    if (active) {
-        parent = P.parent[rd.rep_off + child];
-        const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent * rd.wstride;
-        own[0] = compact_from_padded(src, pitch, Lh, NB, w);
-        own[1] = compact_from_padded(src + PW, pitch, Lh, NB, w);
-    }
-    pl[FP + w] = own[0];
-    pl[AW + FP + w] = own[1];
-    uint32_t J[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};
-    if (SG) {
-        const uint32_t *Jp = P.J + rd.J_off + 2 * rd.wstride;
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int d = 0; d < 4; ++d) J[c][d] = compact_from_padded(Jp + (c * 4 + d) * PW, pitch, Lh, NB, w);
-    }
-    const CompactWord g = compact_word(w, Lh, NB, base);
+    CompactWord *geo = reinterpret_cast<CompactWord *>(smw);
+    uint32_t *Jw = reinterpret_cast<uint32_t *>(geo + CW);  // [colour][neighbour][word]
+    uint32_t *planes = Jw + (SG ? 8 * CW : 0);
+    uint32_t *pl = planes + rloc * 2 * AW;
+    int32_t *acc = reinterpret_cast<int32_t *>(planes + cfg.RPC * 2 * AW);
+    if (threadIdx.x < CW) geo[w] = compact_word(w, Lh, NB, base);  // rloc = 0
     const CompactShifts z = compact_shifts(Lh);
 
-    const unsigned long long T1 = P.thr[rd.thr_off + 2 * i], T2 = P.thr[rd.thr_off + 2 * i + 1];
-    const uint32_t t1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T1;
-    const uint32_t t2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T2;
-    const uint32_t all1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
-    const uint32_t all2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
-    PhiloxKeys K;
-    philox_keys(K, rd.seed, rd.run_id);
-    const uint32_t hi1_0 = __umulhi(0xCD9E8D57u, i), lo1_0 = 0xCD9E8D57u * i;
-    __syncthreads();
-
-    for (uint32_t t = 0; t < rd.theta; ++t) {
-#pragma unroll
-        for (uint32_t c = 0; c < 2; ++c) {
-            if (active) {
-                uint32_t same, rot, up, dn;
-                compact_neighbours<NARROW>(pl + (c ^ 1u) * AW, pl + (c ^ 1u) * AW + FP + w, z, g, c, same, rot, up,
-                                           dn);
-                const uint32_t S = own[c];
-                const uint32_t x1 = S ^ same ^ J[c][0], x2 = S ^ rot ^ J[c][1];
-                const uint32_t x3 = S ^ up ^ J[c][2], x4 = S ^ dn ^ J[c][3];
-                const uint32_t a = x1 ^ x2, b = x1 & x2, e = x3 ^ x4, f = x3 & x4;
-                const uint32_t c0 = a ^ e, ge2 = b | f | (a & e);
-                const uint32_t ctr3 = (TAG_SWEEP << 24) | (t << 1) | c;
-                uint32_t B1 = 0, B2 = 0;
-#pragma unroll
-                for (uint32_t q = 0; q < 8; ++q) {
-                    const uint4 u = philox_rk<PA_COMPACT_WIDE>(8 * w + q, child, ctr3, hi1_0, lo1_0, K);
-                    pack_group(B1, B2, u, q, t1, t2);
+    while (tile < tend) {
+        while (tile_off[slot + 1] <= tile) ++slot;
+        const uint32_t first = tile_off[slot], stop = min(tend, tile_off[slot + 1]);
+        const uint32_t run = group_runs[slot];
+        const RunDev rd = P.runs[run];
+        const RunState st = P.st[run];
+        const uint32_t i = st.step + 1, Rn = st.R_new;
+        if (st.status || i >= rd.n_beta || (tile - first) * cfg.RPC >= Rn) {  // uniform over the CTA
+            tile = stop;
+            continue;
+        }
+        // ---- the run: thresholds, keys, bond masks
+        const uint32_t ob = (i - 1) & 1u, nbuf = i & 1u;
+        const unsigned long long T1 = P.thr[rd.thr_off + 2 * i], T2 = P.thr[rd.thr_off + 2 * i + 1];
+        const uint32_t t1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T1;
+        const uint32_t t2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T2;
+        const uint32_t all1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
+        const uint32_t all2 = T2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : 0u;
+        PhiloxKeys K;
+        philox_keys(K, rd.seed, rd.run_id);
+        const uint32_t hi1_0 = __umulhi(0xCD9E8D57u, i), lo1_0 = 0xCD9E8D57u * i;
+        __syncthreads();  // the tiles of the run before are done with the shared memory
+        fill_thresholds(s_thr, t1, t2);
+        if (SG) {
+            const uint32_t *Jp = P.J + rd.J_off + 2 * rd.wstride;
+            for (uint32_t e = threadIdx.x, cd = 0, v = threadIdx.x; e < 8 * CW; e += blockDim.x, v += blockDim.x) {
+                while (v >= CW) {
+                    v -= CW;
+                    ++cd;
                 }
-                const uint32_t flip = (ge2 | (c0 & (B1 | all1)) | B2 | all2) & g.VM;
-                own[c] = S ^ flip;
-                pl[c * AW + FP + w] = own[c];
+                Jw[e] = compact_from_padded(Jp + cd * PW, pitch, Lh, NB, v);
+            }
+        }
+
+        for (; tile < stop; ++tile) {
+            const uint32_t tile0 = (tile - first) * cfg.RPC;
+            if (tile0 >= Rn) {  // uniform over the CTA
+                tile = stop;
+                break;
+            }
+            const uint32_t child = tile0 + rloc;
+            const bool active = child < Rn;
+            uint32_t own[2] = {0u, 0u}, parent = 0;
+            if (active) {
+                parent = P.parent[rd.rep_off + child];
+                const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent * rd.wstride;
+                own[0] = compact_from_padded(src, pitch, Lh, NB, w);
+                own[1] = compact_from_padded(src + PW, pitch, Lh, NB, w);
+            }
+            pl[FP + w] = own[0];
+            pl[AW + FP + w] = own[1];
+            if (w == 0) acc[2 * rloc] = acc[2 * rloc + 1] = 0;
+            ChildPart cp;
+            philox_child(cp, 8 * w, child, hi1_0, K);
+            __syncthreads();
+
+            for (uint32_t t = 0; t < rd.theta; ++t) {
+#pragma unroll
+                for (uint32_t c = 0; c < 2; ++c) {
+                    const uint32_t h = 2 * t + c;
+                    const CompactWord g = geo[w];
+                    uint32_t same, rot, up, dn, c0, ge2;
+                    compact_neighbours<NARROW>(pl + (c ^ 1u) * AW, pl + (c ^ 1u) * AW + FP + w, z, g, c, same, rot,
+                                               up, dn);
+                    const uint32_t S = own[c];
+                    if (SG) {
+                        same ^= Jw[4 * c * CW + w];
+                        rot ^= Jw[(4 * c + 1) * CW + w];
+                        up ^= Jw[(4 * c + 2) * CW + w];
+                        dn ^= Jw[(4 * c + 3) * CW + w];
+                    }
+                    count_bonds(S ^ same, S ^ rot, S ^ up, S ^ dn, c0, ge2);
+                    const SiteNibbles nib = site_nibbles(c0);
+                    uint32_t B = 0;
+#pragma unroll
+                    for (uint32_t q = 0; q < 8; ++q) {
+                        const SharedPart v = philox_shared(8 * w + q, (TAG_SWEEP << 24) | h, lo1_0, K);
+                        accept_group(B, philox_join(cp, q, v, K), q, nib, s_thr);
+                    }
+                    const uint32_t flip = (ge2 | B | (c0 & all1) | all2) & g.VM;
+                    own[c] = S ^ flip;
+                    pl[c * AW + FP + w] = own[c];
+                    __syncthreads();
+                }
+            }
+
+            // child: planes back in their padded rows, E from the final lattice (every bond
+            // touches one colour-0 site), M
+            if (active) {
+                uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)child * rd.wstride;
+                for (uint32_t p = w; p < PW; p += CW) {
+                    dst[p] = padded_from_compact(pl, base, pitch, Lh, p);
+                    dst[PW + p] = padded_from_compact(pl + AW, base, pitch, Lh, p);
+                }
+                const CompactWord g = geo[w];
+                uint32_t same, rot, up, dn;
+                compact_neighbours<NARROW>(pl + AW, pl + AW + FP + w, z, g, 0, same, rot, up, dn);
+                if (SG) {
+                    same ^= Jw[w];
+                    rot ^= Jw[CW + w];
+                    up ^= Jw[2 * CW + w];
+                    dn ^= Jw[3 * CW + w];
+                }
+                const uint32_t S = own[0];
+                const int32_t unsat = __popc((S ^ same) & g.VM) + __popc((S ^ rot) & g.VM) + __popc((S ^ up) & g.VM) +
+                                      __popc((S ^ dn) & g.VM);
+                atomicAdd(&acc[2 * rloc], unsat);
+                atomicAdd(&acc[2 * rloc + 1], __popc(own[0]) + __popc(own[1]));
             }
             __syncthreads();
+            if (active && w == 0) {
+                const uint64_t pc = rd.rep_off + parent, cc = rd.rep_off + child;
+                P.E[nbuf][cc] = 2 * acc[2 * rloc] - 2 * (int32_t)N;
+                P.M[nbuf][cc] = 2 * acc[2 * rloc + 1] - (int32_t)N;
+                P.fam[nbuf][cc] = P.fam[ob][pc];
+            }
         }
-    }
-
-    // child: planes back in their padded rows, E from the final lattice (every bond
-    // touches one colour-0 site), M
-    if (active) {
-        uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)child * rd.wstride;
-        for (uint32_t p = w; p < PW; p += CW) {
-            dst[p] = padded_from_compact(pl, base, pitch, Lh, p);
-            dst[PW + p] = padded_from_compact(pl + AW, base, pitch, Lh, p);
-        }
-        uint32_t same, rot, up, dn;
-        compact_neighbours<NARROW>(pl + AW, pl + AW + FP + w, z, g, 0, same, rot, up, dn);
-        const uint32_t S = own[0];
-        const int32_t unsat = __popc((S ^ same ^ J[0][0]) & g.VM) + __popc((S ^ rot ^ J[0][1]) & g.VM) +
-                              __popc((S ^ up ^ J[0][2]) & g.VM) + __popc((S ^ dn ^ J[0][3]) & g.VM);
-        atomicAdd(&acc[2 * rloc], unsat);
-        atomicAdd(&acc[2 * rloc + 1], __popc(own[0]) + __popc(own[1]));
-    }
-    __syncthreads();
-    if (active && w == 0) {
-        const uint64_t pc = rd.rep_off + parent, cc = rd.rep_off + child;
-        P.E[nbuf][cc] = 2 * acc[2 * rloc] - 2 * (int32_t)N;
-        P.M[nbuf][cc] = 2 * acc[2 * rloc + 1] - (int32_t)N;
-        P.fam[nbuf][cc] = P.fam[ob][pc];
     }
 }
 
@@ -3489,6 +3698,14 @@ cudaError_t prepare_kernels()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(resample_multinomial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  RESAMPLE_STAGE_MAX * sizeof(int32_t));
+    for (void *k : {(void *)sweep_pow2_kernel<true, 1024, 4, false, true, 256, 2>,
+                    (void *)sweep_pow2_kernel<false, 1024, 4, false, true, 256, 2>,
+                    (void *)sweep_pow2_kernel<true, 1024, 4, false, false, 256, 2>,
+                    (void *)sweep_pow2_kernel<false, 1024, 4, false, false, 256, 2>})  // planes, child parts: 72 KB
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+    for (void *k : {(void *)sweep_compact_kernel<true, 1024, 1, false>, (void *)sweep_compact_kernel<false, 1024, 1, false>})
+        if (e == cudaSuccess)  // geometry, bond masks and planes of up to 1009 words: 73 KB
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
     if (e == cudaSuccess)  // Wang pairing with R_cap up to 8192: 144 KB
         e = cudaFuncSetAttribute(wang_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     return e;
@@ -3533,20 +3750,23 @@ void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_run
     resample_parents_kernel<<<grid, RESAMPLE_THREADS, 0, s>>>(P, runs);
 }
 
-// Launch shapes of the bit-sliced kernel: WPT plane words per thread and
-// `block` threads per CTA (a multiple of the threads per replica, HW / WPT).
-SweepCfg sweep_fast_config(uint32_t L, uint32_t WPT, uint32_t block)
+// Launch shapes of the bit-sliced power-of-two kernel: WPT plane words per thread, `block`
+// threads per CTA (a multiple of the HW / WPT threads of a replica) and TH half-sweeps of
+// shared Philox parts in the table (0: no table).
+SweepCfg sweep_fast_config(uint32_t L, uint32_t WPT, uint32_t block, uint32_t TH)
 {
     SweepCfg c{};
-    const uint32_t N = L * L, HW = N / 64;
+    const uint32_t HW = L * L / 64;
+    c.K = 1;
     c.fast = 1;
     c.WPT = WPT;
     c.TPR = HW / WPT;
     c.block = block;
     c.RPC = block / c.TPR;
-    c.G = N / 8;
+    c.G = 8 * HW;
     c.PS = 0;
-    c.smem = c.RPC * 2 * HW * 4 + 8 * c.RPC;
+    c.TH = TH;
+    c.smem = TH * c.G * 16 + (WPT > 1 ? c.RPC * c.G * 8 : 0) + c.RPC * 2 * HW * 4 + 8 * c.RPC;
     return c;
 }
 
@@ -3556,52 +3776,75 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
     const uint32_t N = L * L;
     const bool pow2 = L >= 8 && L <= 256 && (L & (L - 1)) == 0;
     if (pow2 && allow_fast) {
-        const uint32_t HW = N / 64;
-        if (HW <= 128) {
-            v.push_back(sweep_fast_config(L, 1, 128));
-            v.push_back(sweep_fast_config(L, 1, 256));
-        } else if (HW == 256) {
-            v.push_back(sweep_fast_config(L, 1, 256));
-            v.push_back(sweep_fast_config(L, 2, 128));
-        } else {  // L = 256
-            v.push_back(sweep_fast_config(L, 4, 256));
-            v.push_back(sweep_fast_config(L, 2, 512));
-            v.push_back(sweep_fast_config(L, 1, 1024));
+        // Updates/ns of each shape (40 ferromagnet runs, 4e8 spins, theta = 10); the tuner picks.
+        if (L <= 32) {  // tables of 5 to 16 KB; L = 32: 1790, without a table 1654
+            const uint32_t TH = L == 8 ? 40 : L == 16 ? 20 : 8;
+            v.push_back(sweep_fast_config(L, 1, 256, TH));  // L = 8, 16, 32: 1875, 1859, 1790
+            v.push_back(sweep_fast_config(L, 1, 128, TH));  // 1882, 1849, 1776
+        } else if (L == 64) {  // a table of two half-sweeps, filled by 4 replicas: 1616
+            v.push_back(sweep_fast_config(L, 1, 128, 0));  // 1786
+            v.push_back(sweep_fast_config(L, 1, 256, 0));  // 1760
+        } else if (L == 128) {  // with a table for 2 or 4 replicas: 1418, 1455
+            v.push_back(sweep_fast_config(L, 1, 256, 0));  // 1788
+        } else {  // L = 256: one replica per CTA
+            v.push_back(sweep_fast_config(L, 4, 256, 0));   // 1668
+            v.push_back(sweep_fast_config(L, 1, 1024, 0));  // 1605; the faster one for few replicas
         }
         return v;
     }
     const uint32_t Pt = row_pitch(L), Lh = L / 2, CW = (L * Lh + 31) / 32;
     if (allow_fast && CW <= 1024) {  // compact rows
-        for (uint32_t target : {256u, 128u}) {
+        // The replicas of a CTA of at most `target` threads that leave the fewest lanes idle in
+        // whole groups of four warps (one per SM sub-partition).
+        auto shape = [&](uint32_t target) {
             SweepCfg c{};
+            c.K = 1;
             c.fast = 3;
             c.WPT = 1;
             c.TPR = CW;
-            c.RPC = target / CW > 0 ? target / CW : 1;
+            c.RPC = 1;
+            double best = 0.0;
+            for (uint32_t r = 1; r * CW <= target; ++r) {
+                const double used = (double)(r * CW) / ((r * CW + 127) / 128 * 128);
+                if (used >= best) {
+                    best = used;
+                    c.RPC = r;
+                }
+            }
             c.block = c.RPC * CW;
-            c.G = (N + 7) / 8;
+            c.G = 8 * CW;
             c.PS = Pt;
-            c.smem = c.RPC * 2 * ((Lh + 31) / 32 + CW + Lh / 32 + 2) * 4 + 8 * c.RPC;
+            c.Lh = Lh;
+            c.pw = plane_words_of(L);
+            // geometry, bond masks, planes, sums
+            c.smem = CW * 32 + CW * 32 + c.RPC * 2 * ((Lh + 31) / 32 + CW + Lh / 32 + 2) * 4 + 8 * c.RPC;
             if (v.empty() || v.back().block != c.block) v.push_back(c);
-        }
+        };
+        shape(256);
+        shape(512);
     }
-    if (allow_fast && L >= 6 && Pt <= 32 && Pt != L / 2) {  // padded rows
-        const uint32_t HW = L * Pt / 32;
+    // Padded rows draw only the 6 Philox groups that a word of 4 rows holds at L = 12, where the
+    // compact planes end in a word three quarters empty: 1218 against 1138 updates/ns there; at
+    // every other size tried (6 to 62) the compact rows are 10 to 55 % faster.
+    if (allow_fast && L == 12) {
         for (uint32_t target : {128u, 256u}) {
             SweepCfg c{};
+            const uint32_t HW = L * Pt / 32;
+            c.K = 1;
             c.fast = 2;
             c.WPT = 1;
             c.TPR = HW;
-            c.RPC = target / HW > 0 ? target / HW : 1;
+            c.RPC = target / HW;
             c.block = c.RPC * HW;
             c.G = (N + 7) / 8;
-            c.PS = Pt;  // the row pitch selects the kernel instantiation
+            c.PS = Pt;
             c.smem = c.RPC * 2 * HW * 4 + 8 * c.RPC;
             v.push_back(c);
         }
     }
     if (!v.empty()) return v;
     SweepCfg c{};
+    c.K = 1;
     c.fast = 0;
     c.WPT = 1;
     c.G = (N + 7) / 8;
@@ -3623,53 +3866,68 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
 }
 
 void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *tile_off, uint32_t n_group_runs,
-                  uint32_t n_tiles, const SweepCfg &cfg, int any_glass, cudaStream_t s)
+                  uint32_t n_tiles, const SweepCfg &shape, int any_glass, uint32_t theta_max, cudaStream_t s)
 {
-    const dim3 grid(n_tiles);
-#define PA_SWEEP_FAST(SG, WPT, MAXT) \
-    sweep_pow2_kernel<SG, WPT, MAXT><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg)
-#define PA_SWEEP_FAST2(SG, WPT) \
-    sweep_pow2_kernel_2cta<SG, WPT><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg)
+    SweepCfg cfg = shape;
+    // Consecutive tiles per CTA.  With few sweeps per launch, finding the run, its thresholds, keys
+    // and table are a third of a tile's time, and one CTA pays them once for K tiles (theta = 1,
+    // 40 runs of 1.6e6 replicas in all: L = 16 1077 -> 1219 updates/ns, L = 64 1042 -> 1342, L = 256
+    // 1358 -> 1441).  At theta = 10 they are 3 % and the loop over tiles costs the power-of-two
+    // kernel as much in registers (L = 16: 1877 one tile, 1818 four), so it is compiled both ways
+    // and theta > 4 takes one tile.  K leaves at least 4 (compact rows: 16) CTAs per SM slot, for
+    // a last wave that is short beside the launch.
+    const bool many = cfg.fast == 1 && theta_max <= 4;
+    if (many) cfg.K = std::min(8u, std::max(1u, n_tiles / (152 * 4 * 4)));
+    if (cfg.fast == 3) cfg.K = std::min(4u, std::max(1u, n_tiles / (152 * 2 * 16)));
+    const dim3 grid((n_tiles + cfg.K - 1) / cfg.K);
+#define PA_SWEEP_FAST_(SG, HW, WPT, TAB, MANY, MAXT, MINB)                                                          \
+    sweep_pow2_kernel<SG, HW, WPT, TAB, MANY, MAXT, MINB><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, \
+                                                                                            n_group_runs, cfg)
+#define PA_SWEEP_FAST(HW, WPT, TAB, MAXT, MINB)                                                              \
+    (any_glass ? (many ? PA_SWEEP_FAST_(true, HW, WPT, TAB, true, MAXT, MINB)                                \
+                       : PA_SWEEP_FAST_(true, HW, WPT, TAB, false, MAXT, MINB))                              \
+               : (many ? PA_SWEEP_FAST_(false, HW, WPT, TAB, true, MAXT, MINB)                               \
+                       : PA_SWEEP_FAST_(false, HW, WPT, TAB, false, MAXT, MINB)))
     if (cfg.fast == 3) {  // compact rows; the row pitch is at most 32 exactly when L/2 <= 31
-#define PA_SWEEP_COMPACT(MAXT, NARROW)                                                                            \
-    (any_glass ? sweep_compact_kernel<true, MAXT, NARROW><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, \
-                                                                                          n_group_runs, cfg)      \
-               : sweep_compact_kernel<false, MAXT, NARROW><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs,         \
-                                                                                           tile_off, n_group_runs, cfg))
+#define PA_SWEEP_COMPACT(MAXT, MINB, NARROW)                                                                       \
+    (any_glass ? sweep_compact_kernel<true, MAXT, MINB, NARROW><<<grid, cfg.block, cfg.smem, s>>>(                 \
+                     P, group_runs, tile_off, n_group_runs, cfg)                                                   \
+               : sweep_compact_kernel<false, MAXT, MINB, NARROW><<<grid, cfg.block, cfg.smem, s>>>(                \
+                     P, group_runs, tile_off, n_group_runs, cfg))
         if (cfg.block <= 256 && cfg.PS <= 32)
-            PA_SWEEP_COMPACT(256, true);
+            PA_SWEEP_COMPACT(256, 4, true);
         else if (cfg.block <= 256)
-            PA_SWEEP_COMPACT(256, false);
+            PA_SWEEP_COMPACT(256, 4, false);
+        else if (cfg.block <= 512 && cfg.PS <= 32)
+            PA_SWEEP_COMPACT(512, 2, true);
+        else if (cfg.block <= 512)
+            PA_SWEEP_COMPACT(512, 2, false);
         else
-            PA_SWEEP_COMPACT(1024, false);
+            PA_SWEEP_COMPACT(1024, 1, false);
 #undef PA_SWEEP_COMPACT
-    } else if (cfg.fast == 2) {  // padded rows: cfg.PS holds the row pitch
-#define PA_SWEEP_PAD(PT)                                                                                 \
-    (any_glass ? sweep_pad_kernel<true, PT><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, \
-                                                                               n_group_runs, cfg)      \
-               : sweep_pad_kernel<false, PT><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, \
-                                                                                n_group_runs, cfg))
-        if (cfg.PS == 8)
-            PA_SWEEP_PAD(8);
-        else if (cfg.PS == 16)
-            PA_SWEEP_PAD(16);
-        else
-            PA_SWEEP_PAD(32);
-#undef PA_SWEEP_PAD
+    } else if (cfg.fast == 2) {  // padded rows of pitch 8
+        any_glass ? sweep_pad_kernel<true, 8><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg)
+                  : sweep_pad_kernel<false, 8><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg);
     } else if (!cfg.fast && cfg.G <= cfg.TPR && cfg.block <= 512)
         sweep_kernel<true, 512><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg);
     else if (!cfg.fast)
         sweep_kernel<false, 1024><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg);
-    else if (cfg.WPT == 1 && cfg.block <= 256)
-        any_glass ? PA_SWEEP_FAST(true, 1, 256) : PA_SWEEP_FAST(false, 1, 256);
-    else if (cfg.WPT == 1)
-        any_glass ? PA_SWEEP_FAST(true, 1, 1024) : PA_SWEEP_FAST(false, 1, 1024);
-    else if (cfg.WPT == 2)
-        any_glass ? PA_SWEEP_FAST2(true, 2) : PA_SWEEP_FAST2(false, 2);
+    else if (cfg.G == 8)
+        PA_SWEEP_FAST(1, 1, true, 256, 2);
+    else if (cfg.G == 8 * 4)
+        PA_SWEEP_FAST(4, 1, true, 256, 2);
+    else if (cfg.G == 8 * 16)
+        PA_SWEEP_FAST(16, 1, true, 256, 2);
+    else if (cfg.G == 8 * 64)
+        PA_SWEEP_FAST(64, 1, false, 256, 2);
+    else if (cfg.G == 8 * 256)
+        PA_SWEEP_FAST(256, 1, false, 256, 2);
+    else if (cfg.WPT == 4)
+        PA_SWEEP_FAST(1024, 4, false, 256, 2);
     else
-        any_glass ? PA_SWEEP_FAST(true, 4, 256) : PA_SWEEP_FAST(false, 4, 256);
+        PA_SWEEP_FAST(1024, 1, false, 1024, 1);
 #undef PA_SWEEP_FAST
-#undef PA_SWEEP_FAST2
+#undef PA_SWEEP_FAST_
 }
 
 void launch_overlap(const Pool &P, const uint32_t *q_runs, uint32_t n_q_runs, uint32_t max_Rcap, int init,
