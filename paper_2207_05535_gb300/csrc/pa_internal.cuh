@@ -226,6 +226,10 @@ void launch_wavg(const pa_step_record *recs, const unsigned long long *rec_off, 
 // Copies the record of each listed run at the temperature it has reached to out[k].
 void launch_gather_records(const Pool &P, const uint32_t *runs, uint32_t n_runs, pa_step_record *out,
                            cudaStream_t s);
+// Groups t0 .. t0 + count - 1 of four consecutive sites of the replicas at `words` (one run's
+// packed planes, counted from the first replica) as int8 +-1 into out (4 count bytes).
+void launch_unpack_spins(const uint32_t *words, const RunDev &rd, uint32_t t0, uint32_t count, int8_t *out,
+                         cudaStream_t s);
 // n_steps temperatures of the small runs `runs` (all of lattice size L), cs
 // CTAs (a cluster) per run.
 // Launch shape of the small-run kernel: CTAs per cluster (one cluster per run),

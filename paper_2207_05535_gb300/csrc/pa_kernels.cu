@@ -3530,6 +3530,29 @@ __global__ void __launch_bounds__(128) philox_calibration_kernel(uint32_t *out, 
     out[t] = acc;
 }
 
+// Sites 4 (t0 + t) .. 4 (t0 + t) + 3 of a run of replicas (numbered replica by replica) as int8
+// +-1.  Site n of a replica has sublattice index k = n / 2 in row y = k / (L/2); on an even row
+// its even columns lie in plane 0, on an odd row in plane 1.
+__global__ void __launch_bounds__(256) unpack_spins_kernel(const uint32_t *words, uint32_t wstride, uint32_t pw,
+                                                           uint32_t Lh, uint32_t pitch, uint32_t t0, uint32_t count,
+                                                           char4 *out)
+{
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= count) return;
+    const uint32_t Q = Lh * Lh;  // groups of four sites per replica
+    const uint32_t j = (t0 + t) / Q, k = 2 * (t0 + t - j * Q);
+    const uint32_t *s = words + (uint64_t)j * wstride;
+    signed char v[4];
+#pragma unroll
+    for (uint32_t q = 0; q < 2; ++q) {
+        const uint32_t y = (k + q) / Lh, pos = y * pitch + (k + q - y * Lh);
+        const uint32_t *even = s + (y & 1u ? pw : 0u), *odd = s + (y & 1u ? 0u : pw);
+        v[2 * q] = (even[pos >> 5] >> (pos & 31)) & 1u ? 1 : -1;
+        v[2 * q + 1] = (odd[pos >> 5] >> (pos & 31)) & 1u ? 1 : -1;
+    }
+    out[t] = make_char4(v[0], v[1], v[2], v[3]);
+}
+
 // The record of each listed run at the temperature it has reached (a gather
 // for pa_step_records: one copy back to the host for a whole batch).
 __global__ void gather_records_kernel(Pool P, const uint32_t *runs, uint32_t n, pa_step_record *out)
@@ -3674,6 +3697,14 @@ void launch_anneal_small(const Pool &P, const uint32_t *runs, uint32_t n_runs, u
     uint32_t H = sh.H;
     void *args[] = {(void *)&P, (void *)&runs, (void *)&n_steps, (void *)&H};
     cudaLaunchKernelExC(&cfg, small_kernel(L, any_glass, sh.variant), args);
+}
+
+void launch_unpack_spins(const uint32_t *words, const RunDev &rd, uint32_t t0, uint32_t count, int8_t *out,
+                         cudaStream_t s)
+{
+    if (count == 0) return;
+    unpack_spins_kernel<<<(count + 255) / 256, 256, 0, s>>>(words, rd.wstride, rd.pw, rd.Lh, rd.pitch, t0, count,
+                                                            reinterpret_cast<char4 *>(out));
 }
 
 void launch_gather_records(const Pool &P, const uint32_t *runs, uint32_t n_runs, pa_step_record *out, cudaStream_t s)
