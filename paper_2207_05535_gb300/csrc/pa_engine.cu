@@ -1360,37 +1360,18 @@ pa_status pa_finished(const pa_engine *e, uint32_t *slots_out, uint32_t cap, uin
 pa_status pa_reset(pa_engine *e)
 {
     if (!e) return PA_ERR_INVALID_ARG;
-    PA_CUDA(cudaStreamSynchronize(e->stream));
-    std::vector<RunState> st(e->active.size());
-    for (size_t k = 0; k < e->active.size(); ++k) {
-        const uint32_t s = e->active[k];
-        const RunDev &x = e->rd[s];
-        st[k].step = 0;
-        st[k].R_cur = x.R;
-        st[k].R_new = x.R;
-        st[k].status = 0;
-        st[k].lnQ = 0.0;
-        st[k].ticket = 0;
-        st[k].Emin = 0;
-        st[k].n_levels = 0;
-        st[k].pad = 0;
-        PA_CUDA(cudaMemcpyAsync(e->P.st + s, &st[k], sizeof(RunState), cudaMemcpyHostToDevice, e->stream));
-        PA_CUDA(cudaMemsetAsync(e->P.rec + x.rec_off, 0, sizeof(pa_step_record) * x.n_beta, e->stream));
-        PA_CUDA(cudaMemsetAsync(e->P.scratch + x.scr_off, 0, 8 * scr_table_off(x.N), e->stream));
-        if (x.overlap) {
-            const uint64_t nq = (uint64_t)x.n_beta * (x.N + 1);
-            PA_CUDA(cudaMemsetAsync(e->P.qh + x.qh_off, 0, sizeof(uint32_t) * nq, e->stream));
-            PA_CUDA(cudaMemsetAsync(e->P.qhp + x.qh_off, 0, sizeof(uint32_t) * nq, e->stream));
-            PA_CUDA(cudaMemsetAsync(e->P.qhw + x.qh_off, 0, sizeof(uint32_t) * nq, e->stream));
-        }
+    std::vector<char> waiting(e->rh.size(), 0);
+    for (uint32_t s : e->pending) waiting[s] = 1;
+    for (uint32_t s : e->active) {
         e->rh[s].steps_done = 0;
-        if (std::find(e->pending.begin(), e->pending.end(), s) == e->pending.end()) e->pending.push_back(s);
+        if (!waiting[s]) e->pending.push_back(s);
     }
+    PA_TRY(rebuild(e));  // the pending list holds every resident run now
+    if (e->init_n)
+        timed_launch(e, PA_K_INIT, [&] { launch_reset_runs(e->P, meta(e, e->init_runs_off), e->init_n, e->stream); });
+    PA_CUDA(cudaGetLastError());
     PA_CUDA(cudaMemsetAsync(e->P.status, 0, sizeof(uint32_t), e->stream));
-    PA_CUDA(cudaStreamSynchronize(e->stream));  // st must outlive the copies
     e->latched = PA_OK;
-    e->h2d += sizeof(RunState) * e->active.size();
-    e->dirty = true;
     return prepare(e);
 }
 
