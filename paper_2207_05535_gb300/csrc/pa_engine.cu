@@ -1519,6 +1519,19 @@ pa_status pa_calibrate_philox(uint32_t wide, uint32_t reps, void *cuda_stream, d
     return PA_OK;
 }
 
+// Enqueues the copy of a result into the caller's memory, whose pages are first touched from the
+// host (they are overwritten anyway), while the device still works on the result.  A copy into
+// pages that have never been touched takes their faults one by one from the device: 20.8 MB into
+// fresh pages 17 ms, 0.8 ms with the touching (0.13 ms into pages in use).
+static cudaError_t copy_out(void *host, const void *dev, size_t bytes, cudaStream_t s)
+{
+    volatile char *p = static_cast<volatile char *>(host);
+    if (bytes >= (64u << 10))
+        for (size_t o = 0; o < bytes; o += 4096) p[o] = 0;
+    if (bytes) p[bytes - 1] = 0;
+    return cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, s);
+}
+
 pa_status pa_records(pa_engine *e, uint32_t run, pa_step_record *host_out, uint32_t *host_qhist,
                      uint32_t *host_qhist_pair, uint32_t *host_qhist_wang)
 {
@@ -1526,19 +1539,16 @@ pa_status pa_records(pa_engine *e, uint32_t run, pa_step_record *host_out, uint3
     const RunDev &x = e->rd[run];
     if ((host_qhist || host_qhist_pair || host_qhist_wang) && !x.overlap) return PA_ERR_INVALID_ARG;
     PA_TRY(prepare(e));
-    PA_CUDA(cudaMemcpyAsync(host_out, e->P.rec + x.rec_off, sizeof(pa_step_record) * x.n_beta,
-                            cudaMemcpyDeviceToHost, e->stream));
+    PA_CUDA(copy_out(host_out, e->P.rec + x.rec_off, sizeof(pa_step_record) * x.n_beta, e->stream));
     const size_t nq = (size_t)x.n_beta * (x.N + 1);
     e->d2h += sizeof(pa_step_record) * x.n_beta +
               sizeof(uint32_t) * nq * ((host_qhist ? 1 : 0) + (host_qhist_pair ? 1 : 0) + (host_qhist_wang ? 1 : 0));
     if (host_qhist)
-        PA_CUDA(cudaMemcpyAsync(host_qhist, e->P.qh + x.qh_off, sizeof(uint32_t) * nq, cudaMemcpyDeviceToHost, e->stream));
+        PA_CUDA(copy_out(host_qhist, e->P.qh + x.qh_off, sizeof(uint32_t) * nq, e->stream));
     if (host_qhist_pair)
-        PA_CUDA(cudaMemcpyAsync(host_qhist_pair, e->P.qhp + x.qh_off, sizeof(uint32_t) * nq, cudaMemcpyDeviceToHost,
-                                e->stream));
+        PA_CUDA(copy_out(host_qhist_pair, e->P.qhp + x.qh_off, sizeof(uint32_t) * nq, e->stream));
     if (host_qhist_wang)
-        PA_CUDA(cudaMemcpyAsync(host_qhist_wang, e->P.qhw + x.qh_off, sizeof(uint32_t) * nq, cudaMemcpyDeviceToHost,
-                                e->stream));
+        PA_CUDA(copy_out(host_qhist_wang, e->P.qhw + x.qh_off, sizeof(uint32_t) * nq, e->stream));
     return sync_read(e);
 }
 
@@ -1594,7 +1604,7 @@ pa_status pa_population_slice(pa_engine *e, uint32_t run, uint32_t first, uint32
                                 (uint32_t)(len / 4), stage, e->stream);
             e->launches += 1;
             PA_CUDA(cudaGetLastError());
-            PA_CUDA(cudaMemcpyAsync(host_spins + o, stage, len, cudaMemcpyDeviceToHost, e->stream));
+            PA_CUDA(copy_out(host_spins + o, stage, len, e->stream));
         }
         PA_CUDA(cudaMemsetAsync(stage, 0, std::min(cap, bytes), e->stream));
         e->d2h += bytes;
@@ -1698,12 +1708,10 @@ pa_status pa_weighted_average_runs(pa_engine *e, const uint32_t *run_idx, uint32
     e->d2h += sizeof(pa_wavg) * n_groups * n_steps +
               sizeof(double) * nP * ((host_Pq ? 1 : 0) + (host_Pq_pair ? 1 : 0) + (host_Pq_wang ? 1 : 0));
     PA_CUDA(cudaGetLastError());
-    PA_CUDA(cudaMemcpyAsync(host_out, d_out, sizeof(pa_wavg) * n_groups * n_steps, cudaMemcpyDeviceToHost, e->stream));
-    if (host_Pq) PA_CUDA(cudaMemcpyAsync(host_Pq, d_pq, sizeof(double) * nP, cudaMemcpyDeviceToHost, e->stream));
-    if (host_Pq_pair)
-        PA_CUDA(cudaMemcpyAsync(host_Pq_pair, d_pqp, sizeof(double) * nP, cudaMemcpyDeviceToHost, e->stream));
-    if (host_Pq_wang)
-        PA_CUDA(cudaMemcpyAsync(host_Pq_wang, d_pqw, sizeof(double) * nP, cudaMemcpyDeviceToHost, e->stream));
+    PA_CUDA(copy_out(host_out, d_out, sizeof(pa_wavg) * n_groups * n_steps, e->stream));
+    if (host_Pq) PA_CUDA(copy_out(host_Pq, d_pq, sizeof(double) * nP, e->stream));
+    if (host_Pq_pair) PA_CUDA(copy_out(host_Pq_pair, d_pqp, sizeof(double) * nP, e->stream));
+    if (host_Pq_wang) PA_CUDA(copy_out(host_Pq_wang, d_pqw, sizeof(double) * nP, e->stream));
     return pa_sync(e);
 }
 
@@ -1760,10 +1768,10 @@ pa_status pa_weighted_average(const pa_step_record *recs, const uint32_t *qhist,
         launch_wavg_wang(d_rec, d_roff, d_qh, d_qhp, d_qhw, d_qoff, 1, M, n_steps, N, weight_kind, d_out, d_w, d_pq,
                          d_pqp, d_pqw, st);
         if ((err = cudaGetLastError())) break;
-        if ((err = cudaMemcpyAsync(out, d_out, sizeof(pa_wavg) * n_steps, cudaMemcpyDeviceToHost, st))) break;
-        if (Pq && (err = cudaMemcpyAsync(Pq, d_pq, sizeof(double) * nP, cudaMemcpyDeviceToHost, st))) break;
-        if (Pq_pair && (err = cudaMemcpyAsync(Pq_pair, d_pqp, sizeof(double) * nP, cudaMemcpyDeviceToHost, st))) break;
-        if (Pq_wang && (err = cudaMemcpyAsync(Pq_wang, d_pqw, sizeof(double) * nP, cudaMemcpyDeviceToHost, st))) break;
+        if ((err = copy_out(out, d_out, sizeof(pa_wavg) * n_steps, st))) break;
+        if (Pq && (err = copy_out(Pq, d_pq, sizeof(double) * nP, st))) break;
+        if (Pq_pair && (err = copy_out(Pq_pair, d_pqp, sizeof(double) * nP, st))) break;
+        if (Pq_wang && (err = copy_out(Pq_wang, d_pqw, sizeof(double) * nP, st))) break;
         err = cudaStreamSynchronize(st);
     } while (0);
     if (err != cudaSuccess) s = cuda_fail(err, "pa_weighted_average");
