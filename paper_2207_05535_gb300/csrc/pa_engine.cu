@@ -241,7 +241,7 @@ struct pa_engine {
     std::vector<uint32_t> big;         // the other resident runs (per-stage kernels)
     uint64_t big_off = 0;
     std::map<uint32_t, Tuning> tuning;  // per lattice size
-    uint32_t max_Rcap_active = 0, max_pw = 1;
+    uint32_t max_Rcap_active = 0, max_N_active = 0, max_pw = 1;
     // execution
     uint64_t launches = 0;
     cudaGraph_t graph = nullptr;
@@ -720,9 +720,11 @@ pa_status rebuild(pa_engine *e)
     m.insert(m.end(), e->big.begin(), e->big.end());
     e->q_runs.clear();
     e->max_Rcap_active = 0;
+    e->max_N_active = 0;
     for (uint32_t s : e->active) {
         if (e->rd[s].overlap) e->q_runs.push_back(s);  // small runs have none
         e->max_Rcap_active = std::max(e->max_Rcap_active, e->rd[s].R_cap);
+        e->max_N_active = std::max(e->max_N_active, e->rd[s].N);
     }
     e->q_off = m.size();
     m.insert(m.end(), e->q_runs.begin(), e->q_runs.end());
@@ -918,7 +920,7 @@ pa_status enqueue_pending(pa_engine *e)
             launch_wang(e->P, meta(e, e->init_wang_off), e->init_wang_n, e->init_wang_maxcap, 1, e->stream);
         });
     timed_launch(e, PA_K_MEASURE,
-                 [&] { launch_measure(e->P, runs, e->init_n, e->max_Rcap_active, 1, e->stream); });
+                 [&] { launch_measure(e->P, runs, e->init_n, e->max_Rcap_active, e->max_N_active, 1, e->stream); });
     e->pending.clear();
     e->dirty = true;  // the pending list is consumed
     PA_CUDA(cudaGetLastError());
@@ -987,7 +989,7 @@ void enqueue_tick(pa_engine *e)
             launch_overlap(e->P, meta(e, e->q_off), (uint32_t)e->q_runs.size(), e->max_Rcap_active, 0, e->stream);
         });
     enqueue_wang(e);
-    timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->max_Rcap_active, 0, e->stream); });
+    timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->max_Rcap_active, e->max_N_active, 0, e->stream); });
 }
 
 // One eager step of tuning.  A lattice size whose sweep shape is not chosen yet
@@ -1039,7 +1041,7 @@ pa_status enqueue_tuning_tick(pa_engine *e)
             launch_overlap(e->P, meta(e, e->q_off), (uint32_t)e->q_runs.size(), e->max_Rcap_active, 0, e->stream);
         });
     enqueue_wang(e);
-    if (na) timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->max_Rcap_active, 0, e->stream); });
+    if (na) timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->max_Rcap_active, e->max_N_active, 0, e->stream); });
     PA_CUDA(cudaGetLastError());
     if (timing.empty()) return PA_OK;
     PA_CUDA(cudaStreamSynchronize(e->stream));

@@ -206,7 +206,7 @@ void launch_overlap(const Pool &P, const uint32_t *q_runs, uint32_t n_q_runs, ui
                     cudaStream_t s);
 // run_ctas(R_cap) CTAs per run (at most run_ctas(max_Rcap)); also prepares the
 // next nearest-integer resampling of each run.
-void launch_measure(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap, int init,
+void launch_measure(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap, uint32_t max_N, int init,
                     cudaStream_t s);
 // theta = PA_THETA_INF runs: fresh energies from the exact distribution for
 // the population of the step in flight (init: the beta_0 population).

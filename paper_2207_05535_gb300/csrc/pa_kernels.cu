@@ -591,6 +591,11 @@ __global__ void __launch_bounds__(512) resample_multinomial_kernel(Pool P, const
 //   resample_parents_kernel  offsets (earlier CTAs' totals plus a scan inside
 //                            the CTA) and the parent map
 constexpr uint32_t RESAMPLE_THREADS = 512;
+// Launches whose populations all have at most this many replicas resample and measure with 128
+// threads per run: a run's time is a chain of dependent steps that more threads do not shorten,
+// and four times the runs share an SM (2048 runs of R = 100, L = 16: measurement
+// 89 -> 37 us a step, resampling 36 -> 15 us).
+constexpr uint32_t FEW_REPLICAS = 1024;
 constexpr uint32_t COUNTS_SMEM_LEVELS = 2048;  // level tables staged in shared memory (L <= 45)
 constexpr uint32_t COUNTS_BATCH = 4;           // replicas per thread in flight
 constexpr uint32_t PARENT_BATCH = 8;           // rows of 32 copy numbers a warp loads at once
@@ -2502,7 +2507,6 @@ struct Moments {
 #endif
 constexpr uint32_t MEASURE_SMEM_BINS = 4097;  // L <= 64: counts in shared memory
 constexpr uint32_t MEASURE_BATCH = 4;         // rows of 32 replicas a warp loads at once
-constexpr uint32_t MEASURE_SMEM_TERMS = MEASURE_SMEM_BINS;  // doubles that fit in the counters' space
 
 // The shared memory of a run's measurement tail (CTAs of up to 1024 threads).
 struct TailSmem {
@@ -2665,9 +2669,9 @@ __device__ void run_tail(const Pool &P, const RunDev &rd, RunState *st, uint32_t
 }
 
 __global__ void __launch_bounds__(PA_MEASURE_THREADS, PA_MEASURE_MIN_BLOCKS) measure_kernel(Pool P, const uint32_t *runs,
-                                                                                           int init)
+                                                                                           int init, uint32_t bins)
 {
-    __shared__ __align__(16) uint32_t sh_h[2][MEASURE_SMEM_BINS];
+    extern __shared__ __align__(16) uint32_t sh_h[];  // [2][bins]: energy and magnetisation counts; the terms
     __shared__ FamPart part[32];
     __shared__ TailSmem ts;
     __shared__ uint32_t sh_last;
@@ -2691,12 +2695,12 @@ __global__ void __launch_bounds__(PA_MEASURE_THREADS, PA_MEASURE_MIN_BLOCKS) mea
     unsigned long long *scr = P.scratch + rd.scr_off;
     uint32_t *gE = reinterpret_cast<uint32_t *>(scr);
     uint32_t *gM = reinterpret_cast<uint32_t *>(scr + scr_mhist_off(N));
-    const bool smem = n1 <= MEASURE_SMEM_BINS;
-    uint32_t *hE = smem ? sh_h[0] : gE, *hM = smem ? sh_h[1] : gM;
+    const bool smem = n1 <= bins;
+    uint32_t *hE = smem ? sh_h : gE, *hM = smem ? sh_h + bins : gM;
     if (smem) {
         for (uint32_t n = tid; n < n1; n += nt) {
-            sh_h[0][n] = 0u;
-            sh_h[1][n] = 0u;
+            hE[n] = 0u;
+            hM[n] = 0u;
         }
         __syncthreads();
     }
@@ -2791,8 +2795,8 @@ __global__ void __launch_bounds__(PA_MEASURE_THREADS, PA_MEASURE_MIN_BLOCKS) mea
     __syncthreads();
     if (smem)  // this CTA's counts into the run's histograms
         for (uint32_t n = tid; n < n1; n += nt) {
-            if (sh_h[0][n]) atomicAdd(&gE[n], sh_h[0][n]);
-            if (sh_h[1][n]) atomicAdd(&gM[n], sh_h[1][n]);
+            if (hE[n]) atomicAdd(&gE[n], hE[n]);
+            if (hM[n]) atomicAdd(&gM[n], hM[n]);
         }
     FamPart *gp = reinterpret_cast<FamPart *>(scr + scr_tail_off(N));
     if (tid == 0) {
@@ -2826,8 +2830,7 @@ __global__ void __launch_bounds__(PA_MEASURE_THREADS, PA_MEASURE_MIN_BLOCKS) mea
     }
     __syncthreads();
 
-    run_tail(P, rd, st, i, init, R, eb, gE, gM, scr, &part[0], reinterpret_cast<double *>(&sh_h[0][0]),
-             MEASURE_SMEM_TERMS, ts);
+    run_tail(P, rd, st, i, init, R, eb, gE, gM, scr, &part[0], reinterpret_cast<double *>(sh_h), bins, ts);
 }
 
 // A record's 128-bit sum as a double: sign and magnitude, then hi 2^64 + lo
@@ -3836,7 +3839,7 @@ void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_run
     if (n_runs == 0) return;
     const dim3 grid(n_runs, run_ctas(max_Rcap));
     if (grid.y == 1) {  // every population in one CTA: one launch
-        resample_counts_kernel<true><<<grid, RESAMPLE_THREADS, 0, s>>>(P, runs);
+        resample_counts_kernel<true><<<grid, max_Rcap <= FEW_REPLICAS ? 128 : RESAMPLE_THREADS, 0, s>>>(P, runs);
         return;
     }
     resample_counts_kernel<false><<<grid, RESAMPLE_THREADS, 0, s>>>(P, runs);
@@ -4030,11 +4033,13 @@ void launch_overlap(const Pool &P, const uint32_t *q_runs, uint32_t n_q_runs, ui
     overlap_kernel<<<grid, 256, 0, s>>>(P, q_runs, init);
 }
 
-void launch_measure(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap, int init,
+void launch_measure(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap, uint32_t max_N, int init,
                     cudaStream_t s)
 {
     if (n_runs == 0) return;
-    measure_kernel<<<dim3(n_runs, run_ctas(max_Rcap)), PA_MEASURE_THREADS, 0, s>>>(P, runs, init);
+    const uint32_t bins = std::min(max_N + 1, MEASURE_SMEM_BINS);
+    const uint32_t threads = max_Rcap <= FEW_REPLICAS ? 128 : PA_MEASURE_THREADS;
+    measure_kernel<<<dim3(n_runs, run_ctas(max_Rcap)), threads, 2 * bins * sizeof(uint32_t), s>>>(P, runs, init, bins);
 }
 
 void launch_philox_calibration(uint32_t *out, uint32_t blocks, uint32_t threads, uint32_t iters, bool wide,

@@ -1,0 +1,67 @@
+"""Resampling, measurement and Wang pairing at the sizes where their launches
+change: against the oracle, bit for bit (ln Q and -beta F to 1e-12 relative, a few
+ulp of the device's log)."""
+import numpy as np
+import pytest
+
+import oracle as O
+from paper_2207_05535_gb300 import _lib
+from paper_2207_05535_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _against_oracle(descs, flags=0):
+    n = max(d.n_beta for d in descs)
+    with _lib.Engine(descs, flags=flags) as eng:
+        eng.run_to_end(use_graph=False)
+        for k, d in enumerate(descs):
+            o = O.OracleRun.from_desc(d)
+            for _ in range(1, d.n_beta):
+                assert o.step() == 0
+            g, r = eng.records(k), o.records()
+            for f in g.dtype.names:
+                if f in ("lnQ", "minus_betaF"):
+                    assert np.allclose(g[f], r[f], rtol=1e-12, atol=1e-12), (k, f)
+                elif f in r.dtype.names:
+                    assert np.array_equal(g[f], r[f]), (k, f)
+            _, E, M, fam, _ = eng.population(k)
+            _, oE, oM, ofam = o.population()
+            assert np.array_equal(E, oE) and np.array_equal(M, oM) and np.array_equal(fam, ofam)
+    assert n > 1
+
+
+def _multi(L, R, run=0, beta_f=0.4, model=W.FERRO):
+    return W.RunDesc(L, model, R, 1, W.schedule(beta_f, 4), seed=3, run_id=run, disorder_id=run, resample=W.MULTINOMIAL)
+
+
+# one replica, fewer than a warp, chunks that do not divide, the block sizes' edge, more levels
+# than shared memory holds (L = 64: up to 4097, of which a population at beta = 0 takes few; a
+# second run of another size sets the launch's shared memory), more replicas than it stages
+@pytest.mark.parametrize("sizes", [[(8, 1)], [(8, 31), (16, 33)], [(16, 1000), (6, 2048)], [(16, 2049), (8, 5)],
+                                   [(30, 3001)], [(64, 700), (8, 400)], [(4, 25000)], [(8, 24576), (8, 24577)]])
+def test_multinomial(sizes):
+    _against_oracle([_multi(L, R, k) for k, (L, R) in enumerate(sizes)])
+
+
+# levels far apart: a glass population quenched in one step spreads over many levels
+def test_multinomial_many_levels():
+    _against_oracle([W.RunDesc(64, W.EA_PMJ, 3000, 1, np.array([0.0, 0.02, 0.7, 0.72]), seed=4, run_id=1,
+                               resample=W.MULTINOMIAL)])
+
+
+# 128-thread and 512-thread launches (capacity up to 1024 and above), with lattice sizes on both
+# sides of the counters' shared memory in one launch
+@pytest.mark.parametrize("R", [1, 2, 31, 127, 128, 129, 500, 700, 1100])
+def test_small_population_launches(R):
+    b = W.schedule(0.6, 4)
+    _against_oracle([W.RunDesc(L, W.EA_PMJ if L % 4 else W.FERRO, R, 1, b, seed=6, run_id=L) for L in (6, 16, 30, 66)],
+                    flags=4)
+
+
+# pairings whose families near R / 2, so that searches go to the whole block
+@pytest.mark.parametrize("R", [40, 200, 1000, 1500])
+def test_wang_large_families(R):
+    b = np.array([0.0, 0.3, 0.9, 1.2, 1.4])
+    _against_oracle([W.RunDesc(8, W.EA_PMJ, R, 1, b, seed=7, run_id=k, disorder_id=k, overlap=W.Q_WANG)
+                     for k in range(6)])
