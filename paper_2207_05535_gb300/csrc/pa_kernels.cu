@@ -2083,6 +2083,7 @@ __global__ void __launch_bounds__(256) overlap_kernel(Pool P, const uint32_t *q_
 //   3. every thread takes pairs (k, pi*_k): Hamming distance of the colour
 //      planes, histogram, sum |N - 2d|.
 // --------------------------------------------------------------------------
+constexpr uint32_t WARP_TRIES = 4;  // rounds of 32 positions before a search goes to the whole block
 constexpr uint32_t WANG_BUCKET_BITS = 12, WANG_BUCKETS = 1u << WANG_BUCKET_BITS;
 
 // Replica indices 0..R-1 in ascending order of their (distinct) 64-bit keys,
@@ -2135,6 +2136,7 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
     __shared__ long long sh_l[32];
     __shared__ uint32_t sh_scan[33];
     __shared__ uint32_t s_ok, s_swaps;
+    __shared__ uint32_t s_i0, s_l0, s_fk, s_fpk, s_found;  // a search handed to the block; s_l0 = 0: no more
     const uint32_t run = runs[blockIdx.x];
     const RunDev rd = P.runs[run];
     const RunState st = P.st[run];
@@ -2161,7 +2163,32 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
     }
     for (uint32_t j = tid; j < R; j += nt) fam[j] = P.fam[b][rd.rep_off + j];
     __syncthreads();
-    if (tid < 32) {
+    // The pass is one warp's: it visits the positions in sigma order and searches a swap partner
+    // 32 positions at a time.  Once a family nears R / 2 a search goes through most of the
+    // permutation, and there are up to R / 2 of them; so after WARP_TRIES
+    // rounds the block's 32 warps take the rest at once, the smallest l found being the one the warp
+    // would have reached.  The warps meet at barrier 1 only, twice per search.
+    auto meet = [&] { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); };
+    auto block_search = [&] {
+        const uint32_t i0 = s_i0, fk = s_fk, fpk = s_fpk;
+        for (uint32_t l = s_l0 + tid; l < R; l += nt) {
+            uint32_t q = i0 + l;
+            if (q >= R) q -= R;
+            const uint32_t p = sg[q];
+            if (fam[pi[p]] != fk && fpk != fam[p]) {
+                atomicMin(&s_found, l);
+                break;
+            }
+        }
+    };
+    if (tid >= 32) {
+        for (;;) {
+            meet();
+            if (s_l0 == 0) break;
+            block_search();
+            meet();
+        }
+    } else {
         uint32_t swaps = 0;
         bool ok = true;
         for (uint32_t base = 0; base < R && ok; base += 32) {
@@ -2178,8 +2205,8 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
                 const int t = __ffs(bal) - 1;
                 const uint32_t i0 = base + t, k = sg[i0];
                 const uint32_t fk = fam[k], fpk = fam[pi[k]];
-                uint32_t found = 0xFFFFFFFFu;
-                for (uint32_t l0 = 1; l0 < R; l0 += 32) {  // at most R - 1 positions
+                uint32_t found = 0xFFFFFFFFu, l0 = 1;
+                for (; l0 < min(R, 1 + 32 * WARP_TRIES); l0 += 32) {  // at most R - 1 positions in all
                     const uint32_t l = l0 + lane;
                     bool c = false;
                     uint32_t p = 0;
@@ -2193,6 +2220,24 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
                     if (bc) {
                         found = __shfl_sync(FULL, p, __ffs(bc) - 1);
                         break;
+                    }
+                }
+                if (found == 0xFFFFFFFFu && l0 < R) {
+                    if (lane == 0) {
+                        s_i0 = i0;
+                        s_l0 = l0;
+                        s_fk = fk;
+                        s_fpk = fpk;
+                        s_found = 0xFFFFFFFFu;
+                    }
+                    __syncwarp();
+                    meet();
+                    block_search();
+                    meet();
+                    if (s_found != 0xFFFFFFFFu) {
+                        uint32_t q = i0 + s_found;
+                        if (q >= R) q -= R;
+                        found = sg[q];
                     }
                 }
                 if (found == 0xFFFFFFFFu) {
@@ -2212,7 +2257,10 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
         if (lane == 0) {
             s_ok = ok ? 1u : 0u;
             s_swaps = swaps;
+            s_l0 = 0;
         }
+        __syncwarp();
+        meet();
     }
     __syncthreads();
     pa_step_record *rec = P.rec + rd.rec_off + i;
