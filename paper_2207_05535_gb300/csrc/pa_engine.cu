@@ -951,7 +951,7 @@ void enqueue_resample(pa_engine *e)
     if (!e->multi_runs.empty())
         timed_launch(e, PA_K_RESAMPLE, [&] {
             launch_resample_multinomial(e->P, meta(e, e->multi_off), (uint32_t)e->multi_runs.size(),
-                                        e->multi_maxcap, e->stream);
+                                        e->multi_maxcap, e->max_N_active, e->stream);
         });
 }
 

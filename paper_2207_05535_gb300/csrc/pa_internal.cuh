@@ -190,7 +190,7 @@ void launch_init_population(const Pool &P, const uint32_t *tile_off, const uint3
 // Resampling of runs with PA_MULTINOMIAL, one CTA per run.  max_Rcap: the
 // largest R_cap among the runs (sets the energies staged in shared memory).
 void launch_resample_multinomial(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap,
-                                 cudaStream_t s);
+                                 uint32_t max_N, cudaStream_t s);
 // Nearest-integer resampling (PA_NEAREST) from the tables the measurement of
 // the previous step prepared, run_ctas(R_cap) CTAs per run, in
 // resample_nearest_launches(max_Rcap) kernel launches (one when every

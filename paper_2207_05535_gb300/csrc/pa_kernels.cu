@@ -411,13 +411,28 @@ __global__ void init_couplings_kernel(Pool P, const uint32_t *runs)
 // --------------------------------------------------------------------------
 // Populations of up to this many replicas have their energies staged in shared memory.
 constexpr uint32_t RESAMPLE_STAGE_MAX = 24576;  // 96 KB
+constexpr uint32_t MULTI_THREADS = 1024, MULTI_LEVELS = 512;  // multinomial kernel: threads, levels in shared memory
 
 // Multinomial resampling (PA_MULTINOMIAL), one CTA per run: R draws, each
 // picking a level from the cumulative weights and a member of that level
 // uniformly; then the copy numbers' scan and the parent map as below.
-__global__ void __launch_bounds__(512) resample_multinomial_kernel(Pool P, const uint32_t *runs, uint32_t stage)
+// Dynamic shared memory of a launch that stages R <= stage replicas and up to `levels` energy
+// levels: cumulative weights, per-warp level counts, level starts, energies (then copy numbers),
+// members.
+__host__ __device__ inline uint32_t multinomial_smem(uint32_t stage, uint32_t levels)
 {
-    extern __shared__ int32_t sE[];  // [stage]
+    return levels * (8 + 2 * (MULTI_THREADS / 32) + 4) + stage * 6 + 16;
+}
+
+__global__ void __launch_bounds__(MULTI_THREADS) resample_multinomial_kernel(Pool P, const uint32_t *runs,
+                                                                             uint32_t stage, uint32_t levels)
+{
+    extern __shared__ __align__(16) unsigned char msm[];
+    double *s_cdf = reinterpret_cast<double *>(msm);                              // [levels]
+    int32_t *sE = reinterpret_cast<int32_t *>(s_cdf + levels);                    // [stage], then the copy numbers
+    uint32_t *s_first = reinterpret_cast<uint32_t *>(sE + stage);                 // [levels]
+    uint16_t *s_wcnt = reinterpret_cast<uint16_t *>(s_first + levels);            // [warp][levels]
+    uint16_t *s_mem = s_wcnt + (MULTI_THREADS / 32) * levels;                     // [stage]
     __shared__ uint32_t sh_hist[SMEM_BINS];
     __shared__ int32_t sh_i[32];
     __shared__ uint32_t sh_u[33];
@@ -454,88 +469,173 @@ __global__ void __launch_bounds__(512) resample_multinomial_kernel(Pool P, const
     double *cdf = reinterpret_cast<double *>(scr + scr_table_off(rd.N));
     uint32_t *fill = reinterpret_cast<uint32_t *>(scr + scr_level_off(rd.N));
     uint32_t *members = reinterpret_cast<uint32_t *>(scr + scr_tail_off(rd.N));
-    uint32_t *h = nb <= SMEM_BINS ? sh_hist : g_hist;
-    for (uint32_t n = tid; n < nb; n += nt) h[n] = 0;
-    __syncthreads();
-    for (uint32_t j = tid; j < Rprev; j += nt) atomicAdd(&h[(uint32_t)(Ev[j] - Emin) >> 2], 1u);
-    __syncthreads();
-
     const double dbeta = P.beta[rd.beta_off + i] - P.beta[rd.beta_off + i - 1];
     const double *w = P.wt + P.wtoff[rd.wt_off + i];  // w[n] = exp(-4 n dbeta_i), shared table
-    if (tid == 0) {
-        double S = 0.0;
-        for (uint32_t n = 0; n < nb; ++n) {
-            S = __dadd_rn(S, __dmul_rn((double)h[n], w[n]));
-            cdf[n] = S;
-        }
-        sh_S = S;
-        st->lnQ = (-dbeta) * (double)Emin + log(S) - log((double)Rprev);
-    }
-    __syncthreads();
-    const double S = sh_S;
+    const uint32_t lane = tid & 31u, wid = tid >> 5, nwarp = nt >> 5;
+    const uint32_t chunk = (Rprev + nwarp - 1) / nwarp;  // each warp's contiguous replicas
+    const uint32_t c_lo = min(Rprev, wid * chunk), c_hi = min(Rprev, c_lo + chunk);
     uint32_t *cnt = P.cnt + rd.rep_off;
-
-    // stable list of replicas by level: members[first(n) + rank]
-    if (tid < 32) {
-        uint32_t acc = 0;
-        for (uint32_t base = 0; base < nb; base += 32) {  // fill[n] = first(n)
-            const uint32_t n = base + tid;
-            const uint32_t v = n < nb ? h[n] : 0u;
-            uint32_t x = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                uint32_t y = __shfl_up_sync(FULL, x, o);
-                if ((int)tid >= o) x += y;
-            }
-            if (n < nb) fill[n] = acc + x - v;
-            acc += __shfl_sync(FULL, x, 31);
-        }
+    if (staged && nb <= levels) {
+        // Everything in shared memory.  Each warp counts the levels of its replicas; a level's
+        // members then start at the counts of the lower levels and of the earlier warps, so every
+        // warp places its own, in replica order.  (20 runs of R = 10,000, L = 16, one CTA each: 144 us a step with
+        // one warp building the list and levels, members and copy numbers in global memory, 61 us now.)
+        uint32_t *h = sh_hist;
+        uint16_t *wc = s_wcnt + wid * levels;
+        for (uint32_t n = lane; n < nb; n += 32) wc[n] = 0;
         __syncwarp();
-        for (uint32_t base = 0; base < Rprev; base += 32) {
-            const uint32_t j = base + tid;
-            const bool ok = j < Rprev;
-            const uint32_t n = ok ? (uint32_t)(Ev[j] - Emin) >> 2 : 0xffffffffu;
+        for (uint32_t base = c_lo; base < c_hi; base += 32) {
+            const uint32_t j = base + lane, n = j < c_hi ? (uint32_t)(sE[j] - Emin) >> 2 : 0xffffffffu;
             const unsigned peers = __match_any_sync(FULL, n);
-            const uint32_t rank = __popc(peers & ((1u << tid) - 1u));
-            uint32_t pos = 0;
-            if (ok) pos = fill[n] + rank;
+            if (j < c_hi && lane == (uint32_t)__ffs(peers) - 1u) wc[n] = (uint16_t)(wc[n] + __popc(peers));
             __syncwarp();
-            if (ok) {
-                members[pos] = j;
-                if (rank == 0) fill[n] += __popc(peers);
+        }
+        __syncthreads();
+        for (uint32_t n = tid; n < nb; n += nt) {
+            uint32_t acc = 0;
+            for (uint32_t k = 0; k < nwarp; ++k) {
+                const uint32_t v = s_wcnt[k * levels + n];
+                s_wcnt[k * levels + n] = (uint16_t)acc;
+                acc += v;
+            }
+            h[n] = acc;
+            s_cdf[n] = __dmul_rn((double)acc, w[n]);
+        }
+        __syncthreads();
+        if (wid == 0) {  // the sum in ascending level order
+            if (lane == 0) {
+                double S = 0.0;
+                for (uint32_t n = 0; n < nb; ++n) {
+                    S = __dadd_rn(S, s_cdf[n]);
+                    s_cdf[n] = S;
+                }
+                sh_S = S;
+                st->lnQ = (-dbeta) * (double)Emin + log(S) - log((double)Rprev);
+            }
+        } else if (wid == 1) {
+            uint32_t acc = 0;
+            for (uint32_t base = 0; base < nb; base += 32) {
+                const uint32_t n = base + lane;
+                const uint32_t v = n < nb ? h[n] : 0u;
+                uint32_t x = v;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(FULL, x, o);
+                    if ((int)lane >= o) x += y;
+                }
+                if (n < nb) s_first[n] = acc + x - v;
+                acc += __shfl_sync(FULL, x, 31);
+            }
+        }
+        __syncthreads();
+        for (uint32_t base = c_lo; base < c_hi; base += 32) {
+            const uint32_t j = base + lane, n = j < c_hi ? (uint32_t)(sE[j] - Emin) >> 2 : 0xffffffffu;
+            const unsigned peers = __match_any_sync(FULL, n);
+            const uint32_t rank = __popc(peers & ((1u << lane) - 1u));
+            if (j < c_hi) s_mem[s_first[n] + wc[n] + rank] = (uint16_t)j;
+            __syncwarp();
+            if (j < c_hi && rank == 0) wc[n] = (uint16_t)(wc[n] + __popc(peers));
+            __syncwarp();
+        }
+        __syncthreads();  // the energies are done with: their space takes the copy numbers
+        cnt = reinterpret_cast<uint32_t *>(sE);
+        for (uint32_t j = tid; j < Rprev; j += nt) cnt[j] = 0;
+        __syncthreads();
+        const double S = sh_S;
+        for (uint32_t d = tid; d < rd.R; d += nt) {
+            const uint4 o = philox4x32_10(d, 0, i, TAG_MULTINOMIAL << 24, rd.seed, rd.run_id);
+            const unsigned long long u53 = ((unsigned long long)(o.x >> 5) << 26) | (unsigned long long)(o.y >> 6);
+            const double x = __dmul_rn(__dmul_rn((double)u53, 1.0 / 9007199254740992.0), S);
+            uint32_t a = 0, b = nb;  // first n with cdf[n] > x
+            while (a < b) {
+                const uint32_t m = (a + b) >> 1;
+                if (s_cdf[m] > x)
+                    b = m;
+                else
+                    a = m + 1;
+            }
+            const uint32_t lev = a < nb ? a : nb - 1;
+            const uint32_t idx = (uint32_t)(((unsigned long long)o.z * (unsigned long long)h[lev]) >> 32);
+            atomicAdd(&cnt[s_mem[s_first[lev] + idx]], 1u);
+        }
+        __syncthreads();
+    } else {
+        uint32_t *h = nb <= SMEM_BINS ? sh_hist : g_hist;
+        for (uint32_t n = tid; n < nb; n += nt) h[n] = 0;
+        __syncthreads();
+        for (uint32_t j = tid; j < Rprev; j += nt) atomicAdd(&h[(uint32_t)(Ev[j] - Emin) >> 2], 1u);
+        __syncthreads();
+
+        if (tid == 0) {
+            double S = 0.0;
+            for (uint32_t n = 0; n < nb; ++n) {
+                S = __dadd_rn(S, __dmul_rn((double)h[n], w[n]));
+                cdf[n] = S;
+            }
+            sh_S = S;
+            st->lnQ = (-dbeta) * (double)Emin + log(S) - log((double)Rprev);
+        }
+        __syncthreads();
+        const double S = sh_S;
+
+        // stable list of replicas by level: members[first(n) + rank]
+        if (tid < 32) {
+            uint32_t acc = 0;
+            for (uint32_t base = 0; base < nb; base += 32) {  // fill[n] = first(n)
+                const uint32_t n = base + tid;
+                const uint32_t v = n < nb ? h[n] : 0u;
+                uint32_t x = v;
+                for (int o = 1; o < 32; o <<= 1) {
+                    uint32_t y = __shfl_up_sync(FULL, x, o);
+                    if ((int)tid >= o) x += y;
+                }
+                if (n < nb) fill[n] = acc + x - v;
+                acc += __shfl_sync(FULL, x, 31);
             }
             __syncwarp();
+            for (uint32_t base = 0; base < Rprev; base += 32) {
+                const uint32_t j = base + tid;
+                const bool ok = j < Rprev;
+                const uint32_t n = ok ? (uint32_t)(Ev[j] - Emin) >> 2 : 0xffffffffu;
+                const unsigned peers = __match_any_sync(FULL, n);
+                const uint32_t rank = __popc(peers & ((1u << tid) - 1u));
+                uint32_t pos = 0;
+                if (ok) pos = fill[n] + rank;
+                __syncwarp();
+                if (ok) {
+                    members[pos] = j;
+                    if (rank == 0) fill[n] += __popc(peers);
+                }
+                __syncwarp();
+            }
         }
-    }
-    for (uint32_t j = tid; j < Rprev; j += nt) cnt[j] = 0;
-    __syncthreads();
-    const uint32_t last = nb - 1;
-    for (uint32_t d = tid; d < rd.R; d += nt) {
-        const uint4 o = philox4x32_10(d, 0, i, TAG_MULTINOMIAL << 24, rd.seed, rd.run_id);
-        const unsigned long long u53 = ((unsigned long long)(o.x >> 5) << 26) | (unsigned long long)(o.y >> 6);
-        const double x = __dmul_rn(__dmul_rn((double)u53, 1.0 / 9007199254740992.0), S);
-        uint32_t a = 0, b = nb;  // first n with cdf[n] > x
-        while (a < b) {
-            const uint32_t m = (a + b) >> 1;
-            if (cdf[m] > x)
-                b = m;
-            else
-                a = m + 1;
+        for (uint32_t j = tid; j < Rprev; j += nt) cnt[j] = 0;
+        __syncthreads();
+        const uint32_t last = nb - 1;
+        for (uint32_t d = tid; d < rd.R; d += nt) {
+            const uint4 o = philox4x32_10(d, 0, i, TAG_MULTINOMIAL << 24, rd.seed, rd.run_id);
+            const unsigned long long u53 = ((unsigned long long)(o.x >> 5) << 26) | (unsigned long long)(o.y >> 6);
+            const double x = __dmul_rn(__dmul_rn((double)u53, 1.0 / 9007199254740992.0), S);
+            uint32_t a = 0, b = nb;  // first n with cdf[n] > x
+            while (a < b) {
+                const uint32_t m = (a + b) >> 1;
+                if (cdf[m] > x)
+                    b = m;
+                else
+                    a = m + 1;
+            }
+            const uint32_t lev = a < nb ? a : last;
+            const uint32_t idx = (uint32_t)(((unsigned long long)o.z * (unsigned long long)h[lev]) >> 32);
+            const uint32_t first = fill[lev] - h[lev];
+            atomicAdd(&cnt[members[first + idx]], 1u);
         }
-        const uint32_t lev = a < nb ? a : last;
-        const uint32_t idx = (uint32_t)(((unsigned long long)o.z * (unsigned long long)h[lev]) >> 32);
-        const uint32_t first = fill[lev] - h[lev];
-        atomicAdd(&cnt[members[first + idx]], 1u);
+        __syncthreads();
+        if (h == g_hist)  // leave the measurement's histogram cleared
+            for (uint32_t n = tid; n < nb; n += nt) g_hist[n] = 0u;
     }
-    __syncthreads();
-    if (h == g_hist)  // leave the measurement's histogram cleared
-        for (uint32_t n = tid; n < nb; n += nt) g_hist[n] = 0u;
 
     // the copy numbers' exclusive scan and the parent map (contiguous families).
     // Each warp takes a contiguous chunk of the replicas; one barrier joins the chunks.
     uint32_t *parent = P.parent + rd.rep_off;
-    const uint32_t lane = tid & 31u, wid = tid >> 5, nwarp = nt >> 5;
-    const uint32_t chunk = (Rprev + nwarp - 1) / nwarp;
-    const uint32_t c_lo = min(Rprev, wid * chunk), c_hi = min(Rprev, c_lo + chunk);
     uint32_t wsum = 0;
     for (uint32_t j = c_lo + lane; j < c_hi; j += 32) wsum += cnt[j];
     wsum = warp_sum(wsum);
@@ -3833,7 +3933,7 @@ cudaError_t prepare_kernels()
         e = cudaFuncSetAttribute(sweep_kernel<true, 512>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(resample_multinomial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 RESAMPLE_STAGE_MAX * sizeof(int32_t));
+                                 multinomial_smem(RESAMPLE_STAGE_MAX, MULTI_LEVELS));
     for (void *k : {(void *)sweep_pow2_kernel<true, 1024, 4, false, true, 256, 2>,
                     (void *)sweep_pow2_kernel<false, 1024, 4, false, true, 256, 2>,
                     (void *)sweep_pow2_kernel<true, 1024, 4, false, false, 256, 2>,
@@ -3875,11 +3975,14 @@ void launch_dos_sample(const Pool &P, const uint32_t *runs, uint32_t n_runs, uin
 }
 
 void launch_resample_multinomial(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap,
-                                 cudaStream_t s)
+                                 uint32_t max_N, cudaStream_t s)
 {
     if (n_runs == 0) return;
-    const uint32_t stage = max_Rcap < RESAMPLE_STAGE_MAX ? max_Rcap : RESAMPLE_STAGE_MAX;
-    resample_multinomial_kernel<<<n_runs, 512, stage * sizeof(int32_t), s>>>(P, runs, stage);
+    const uint32_t stage = (std::min(max_Rcap, RESAMPLE_STAGE_MAX) + 1) / 2 * 2;
+    const uint32_t levels = (std::min(max_N + 1, MULTI_LEVELS) + 1) / 2 * 2;
+    // small populations: four CTAs share an SM (a block of MULTI_THREADS takes one to itself)
+    const uint32_t threads = max_Rcap <= 2048 ? 256 : MULTI_THREADS;
+    resample_multinomial_kernel<<<n_runs, threads, multinomial_smem(stage, levels), s>>>(P, runs, stage, levels);
 }
 
 void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap, cudaStream_t s)
