@@ -1173,18 +1173,21 @@ __device__ __forceinline__ SharedPart philox_shared(uint32_t g, uint32_t ctr3, u
     return SharedPart{(uint32_t)p1, (uint32_t)(p0 >> 32), (uint32_t)p0};
 }
 
-struct ChildPart {
-    uint32_t x2;         // lo(M0 x0) of round 2 with the key: xored with SharedPart.hi0
-    uint32_t a[8], b[8]; // per group: hi(M1 x2) of round 3 with the key, and lo
+template <uint32_t NG>
+struct ChildPartN {        // of NG consecutive groups
+    uint32_t x2;           // lo(M0 x0) of round 2 with the key: xored with SharedPart.hi0
+    uint32_t a[NG], b[NG]; // per group: hi(M1 x2) of round 3 with the key, and lo
 };
+using ChildPart = ChildPartN<8>;
 
-__device__ __forceinline__ void philox_child(ChildPart &c, uint32_t g0, uint32_t child, uint32_t hi1_0,
+template <uint32_t NG>
+__device__ __forceinline__ void philox_child(ChildPartN<NG> &c, uint32_t g0, uint32_t child, uint32_t hi1_0,
                                              const PhiloxKeys &K)
 {
     const unsigned long long pc = 0xD2511F53ull * (hi1_0 ^ child ^ K.k0[0]);
     c.x2 = (uint32_t)pc ^ K.k1[2];
 #pragma unroll
-    for (uint32_t q = 0; q < 8; ++q) {
+    for (uint32_t q = 0; q < NG; ++q) {
         const uint32_t y2 = (uint32_t)(pc >> 32) ^ (0xD2511F53u * (g0 + q)) ^ K.k1[1];
         const unsigned long long p = 0xCD9E8D57ull * y2;
         c.a[q] = (uint32_t)(p >> 32) ^ K.k0[2];
@@ -1193,7 +1196,8 @@ __device__ __forceinline__ void philox_child(ChildPart &c, uint32_t g0, uint32_t
 }
 
 // The call of group q of the word: rounds 4 to 10 from the two parts.
-__device__ __forceinline__ uint4 philox_join(const ChildPart &c, uint32_t q, const SharedPart &v, const PhiloxKeys &K)
+template <uint32_t NG>
+__device__ __forceinline__ uint4 philox_join(const ChildPartN<NG> &c, uint32_t q, const SharedPart &v, const PhiloxKeys &K)
 {
     uint32_t x0 = c.a[q] ^ v.lo1, x1 = c.b[q], x2 = v.hi0 ^ c.x2, x3 = v.lo0;
 #pragma unroll
@@ -3231,6 +3235,7 @@ __global__ void wavg_q_kernel(const pa_step_record *recs, const unsigned long lo
 // path, so a run can move between the two paths at any step.
 // --------------------------------------------------------------------------
 constexpr uint32_t SMALL_MAX_N = 1024;  // L <= 32
+constexpr uint32_t SMALL_MAX_CTAS = 16;  // largest cluster (above 8 by the non-portable opt-in)
 
 // HW: words of a colour plane (L = 8: 1, 16: 4, 32: 16); LPW lanes per word; NT the
 // largest block (a multiple of 32, at least 128) and MINB the CTAs per SM it is
@@ -3258,7 +3263,7 @@ __global__ void __launch_bounds__(NT, MINB) anneal_small_kernel(Pool P, const ui
     __shared__ uint32_t sh_lvl[2];  // the lowest and highest occupied energy level
     __shared__ double sh_S, sh_logS, sh_logR;
     __shared__ uint32_t sh_carry, sh_first;
-    __shared__ FamPart s_part[8];  // CTA 0: the family statistics of each CTA's chunk of children
+    __shared__ FamPart s_part[SMALL_MAX_CTAS];  // CTA 0: the family statistics of each CTA's chunk of children
     __shared__ int32_t sh_eb;      // CTA 0: base of the energy levels of the new population
     __shared__ uint32_t sh_pre_step;  // the temperature whose comparison bits s_pre holds
     extern __shared__ uint2 s_pre[];  // H > 0: [half-sweep][replica of the tile][word] (B1, B2)
@@ -3393,6 +3398,8 @@ __global__ void __launch_bounds__(NT, MINB) anneal_small_kernel(Pool P, const ui
                 // the first tile of a slice may find its bits drawn already
                 const bool pre = AHEAD && H && tile0 == c_lo && rank != 0 && sh_pre_step == i;
                 const uint32_t Hh = min(H, 2 * rd.theta);
+                ChildPartN<GPL> cp;
+                philox_child(cp, 8 * w + sub * GPL, child, hi1_0, K);
                 auto draw = [&](uint32_t h, uint32_t &B1, uint32_t &B2) {
                     if (AHEAD && pre && h < Hh) {
                         const uint2 v = s_pre[(h * (nt / LPR) + rl) * HW + w];
@@ -3406,7 +3413,7 @@ __global__ void __launch_bounds__(NT, MINB) anneal_small_kernel(Pool P, const ui
 #pragma unroll
                     for (uint32_t q = 0; q < GPL; ++q) {
                         const uint32_t g = sub * GPL + q;
-                        const uint4 u = philox_rk<true>(8 * w + g, child, ctr3, hi1_0, lo1_0, K);
+                        const uint4 u = philox_join(cp, q, philox_shared(8 * w + g, ctr3, lo1_0, K), K);
                         pack_group(B1, B2, u, g, t1, t2);
                     }
 #pragma unroll
@@ -3542,6 +3549,8 @@ __global__ void __launch_bounds__(NT, MINB) anneal_small_kernel(Pool P, const ui
             const uint32_t u2 = U2 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)U2;
             const uint32_t g1 = __umulhi(0xCD9E8D57u, i2), g0 = 0xCD9E8D57u * i2;
             const uint32_t child = lo_k + rl, Hh = min(H, 2 * rd.theta), tr = nt / LPR;
+            ChildPartN<GPL> cp;
+            philox_child(cp, 8 * w + sub * GPL, child, g1, K);
 #pragma unroll AHEAD_UNROLL
             for (uint32_t h = 0; h < Hh; ++h) {
                 const uint32_t ctr3 = (TAG_SWEEP << 24) | h;
@@ -3549,7 +3558,7 @@ __global__ void __launch_bounds__(NT, MINB) anneal_small_kernel(Pool P, const ui
 #pragma unroll
                 for (uint32_t q = 0; q < GPL; ++q) {
                     const uint32_t g = sub * GPL + q;
-                    const uint4 u = philox_rk<true>(8 * w + g, child, ctr3, g1, g0, K);
+                    const uint4 u = philox_join(cp, q, philox_shared(8 * w + g, ctr3, g0, K), K);
                     pack_group(B1, B2, u, g, u1, u2);
                 }
 #pragma unroll
@@ -3814,6 +3823,8 @@ static cudaLaunchConfig_t small_launch_config(uint32_t n_clusters, const SmallSh
     return cfg;
 }
 
+constexpr uint32_t SMS = 152;  // of a GB300
+
 static int small_fit(uint32_t L, int any_glass, const SmallShape &sh)
 {
     cudaLaunchAttribute at[1];
@@ -3835,11 +3846,18 @@ static uint32_t isqrt_u32(uint32_t R)
     return q;
 }
 
+// The largest cluster to try, from the threads that 8 CTAs would sweep with: more than 8 CTAs
+// (the non-portable sizes) pay where those are bound by their throughput, not by the chain of a
+// temperature's steps.  Per temperature, 8 against 16 CTAs: L = 16, R = 1000 (628 threads) 45.3
+// against 28.6 us; L = 16, R = 500 (324 threads) 28.8 against 29.7; L = 8, R = 500 (328) 12.7
+// against 13.4.
+static uint32_t small_largest_cluster(uint32_t threads_of_8) { return threads_of_8 > 384 ? SMALL_MAX_CTAS : 8u; }
+
 // Launch shapes of the small-run kernel for n runs of lattice size L.  A run's
 // steps are a chain of cluster barriers, so a run whose CTAs share SMs with
 // another run's is slower by the sharing, and the launch lasts as long as its
 // slowest run: every shape here keeps all clusters on SMs of their own (asked
-// of the occupancy calculator), the largest cluster first (at most 8 CTAs).
+// of the occupancy calculator), the largest cluster first.
 // small_shape: a block covering a CTA's equal share of R + 3 sqrt(R) + 1
 // children (beyond the nearest-integer resampling's spread); without one,
 // 512-thread CTAs two per SM, about two CTAs per SM over all the runs, the
@@ -3849,7 +3867,8 @@ SmallShape small_shape(uint32_t L, int any_glass, uint32_t n_runs, uint32_t R_ma
     const uint32_t hw = L * L / 64;
     const uint32_t lpr = hw * (L == 8 ? SMALL_LPW_L8 : L == 16 ? SMALL_LPW_L16 : SMALL_LPW_L32);
     const uint32_t R_est = R_max + 3 * isqrt_u32(R_max) + 1;
-    for (uint32_t cs = 8; cs >= 1; --cs) {
+    for (uint32_t cs = L == 32 ? 8 : small_largest_cluster((R_est + 7) / 8 * lpr); cs >= 1; --cs) {
+        if (cs > 1 && cs * n_runs > SMS) continue;  // cannot have an SM per CTA
         const uint32_t chunk = (R_est + cs - 1) / cs;
         uint32_t block = (chunk * lpr + 31) / 32 * 32;
         block = block < 128 ? 128 : block;
@@ -3879,7 +3898,8 @@ SmallShape small_shape_ahead(uint32_t L, int any_glass, uint32_t n_runs, uint32_
     if ((L != 8 && L != 16) || theta_max == 0) return none;
     const uint32_t hw = L * L / 64, lpr4 = 4;
     const uint32_t R_est = R_max + 3 * isqrt_u32(R_max) + 1;
-    for (uint32_t cs = 8; cs >= 2; --cs) {
+    for (uint32_t cs = small_largest_cluster((R_est + 6) / 7 * lpr4); cs >= 2; --cs) {
+        if (cs * n_runs > SMS) continue;
         const uint32_t Wc = (R_est + cs - 2) / (cs - 1);
         uint32_t block = (Wc * lpr4 + 31) / 32 * 32;
         block = block < 128 ? 128 : block;
@@ -3925,6 +3945,13 @@ cudaError_t prepare_kernels()
                 const cudaError_t e = cudaFuncSetAttribute(small_kernel(L, sg, v),
                                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                            (int)SMALL_PRE_BYTES);
+                if (e != cudaSuccess) return e;
+            }
+    for (uint32_t L : {8u, 16u, 32u})
+        for (int sg = 0; sg < 2; ++sg)
+            for (uint32_t v = 0; v <= (L == 32 ? 2u : 4u); ++v) {
+                const cudaError_t e =
+                    cudaFuncSetAttribute(small_kernel(L, sg, v), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
                 if (e != cudaSuccess) return e;
             }
     cudaError_t e = cudaFuncSetAttribute(sweep_kernel<false, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
