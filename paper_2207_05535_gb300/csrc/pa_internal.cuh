@@ -114,6 +114,7 @@ struct SweepCfg {
     uint32_t PS;     // bytes per colour plane = 4 G (byte planes); the row pitch (padded or compact rows)
     uint32_t smem;   // dynamic shared memory bytes
     uint32_t WPT;    // bit-sliced kernels: plane words per thread
+    uint32_t NR;     // power-of-two kernel: children per thread, at the same word
     uint32_t TH;     // half-sweeps of shared Philox parts held in shared memory (0: none)
     uint32_t K;      // consecutive tiles one CTA works through (set by launch_sweep)
     uint32_t Lh, pw; // compact rows: L/2 and words of a stored plane

@@ -1092,8 +1092,8 @@ __global__ void __launch_bounds__(MAXT) sweep_kernel(Pool P, const uint32_t *gro
 // left with a table, 16 without) and each uniform is compared once, with the threshold its site's
 // bonds select, instead of with T_1 and T_2 (8 ALU instructions and 4 adds fewer per call, against
 // one byte permute and one 16-byte shared-memory load).  Measured (theta = 10, 40 runs, 4e8 spins):
-// L = 8, 16, 32: 1610 -> 1903, 1608 -> 1877, 1605 -> 1818 updates/ns; L = 64, 128, 256: 1549 ->
-// 1790, 1536 -> 1788, 1455 -> 1665; per warp and call at L = 16: 62 -> 50 instructions, 100 -> 86
+// L = 8, 16, 32: 1610 -> 1903, 1608 -> 1877, 1605 -> 1875 updates/ns; L = 64, 128, 256: 1549 ->
+// 1875, 1536 -> 1854, 1455 -> 1781; per warp and call at L = 16: 62 -> 50 instructions, 100 -> 86
 // cycles, of which ALU and products explain 2 (26 + 14) = 80.
 // --------------------------------------------------------------------------
 struct PhiloxKeys {
@@ -1275,14 +1275,14 @@ __device__ __forceinline__ void count_bonds(uint32_t x1, uint32_t x2, uint32_t x
 // every child of the CTA reads; otherwise each thread forms them, which is faster from L = 64 on:
 // a table of a few children's CTA costs more to fill than it saves (L = 64, 4 children: 1616
 // against 1786 updates/ns; L = 128, 4 children: 1455 against 1788).
-// With one word per thread the word, its bond masks and its child parts stay in registers (128
-// of them, two CTAs of 256 threads per SM; a cap at 80 or 64 for more warps is 3 to 7 % slower);
-// with several (L = 256) they are read from shared memory (bond masks: global) as each word is
-// swept, so that two CTAs share an SM: 1665 updates/ns, against 1605 for one CTA of 1024 threads.
+// NR: children per thread, at the same word: one of them forms (or reads) a group's shared part
+// for all.  With one word of one child per thread the word, its bond masks and its child parts
+// stay in registers (128 of them, two CTAs of 256 threads per SM; a cap at 80 or 64 for more
+// warps is 3 to 7 % slower); otherwise (MULTI) child parts and spins are read from shared memory
+// as each word is swept, which leaves the registers to the chains of both children (with their
+// parts in registers too they spill, and are slower than one child).
 // MANY: a CTA works through cfg.K tiles (launch_sweep says when).
-// Two children per thread, to share the shared parts in registers, spill at 128 registers: 2 %
-// slower at L = 64 and 128.
-template <bool SG, uint32_t HW, uint32_t WPT, bool TAB, bool MANY, int MAXT, int MINB>
+template <bool SG, uint32_t HW, uint32_t WPT, uint32_t NR, bool TAB, bool MANY, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const uint32_t *group_runs,
                                                                 const uint32_t *tile_off, uint32_t n_group_runs,
                                                                 SweepCfg cfg)
@@ -1291,14 +1291,14 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const ui
     static_assert(Lh * Lh == 16 * HW, "L = 2 Lh, N = 64 HW");
     constexpr uint32_t N = 64 * HW, TPR = HW / WPT;  // sites; threads per replica
     constexpr bool WIDE = TPR > 32;                  // a replica spans several warps
-    constexpr bool MULTI = WPT > 1;
+    constexpr bool MULTI = WPT * NR > 1;
     extern __shared__ __align__(16) uint32_t smw[];  // TAB: the table; MULTI: child parts; planes; sums
     __shared__ uint4 s_thr[16];
     const uint32_t rloc = threadIdx.x / TPR, tl = threadIdx.x % TPR;
     uint4 *tab = reinterpret_cast<uint4 *>(smw);
-    uint2 *ab = reinterpret_cast<uint2 *>(smw) + rloc * 8 * HW;  // MULTI: [group in its word][word]
-    uint32_t *planes = smw + (TAB ? cfg.TH * 32 * HW : MULTI ? cfg.RPC * 16 * HW : 0);
-    uint32_t *pl = planes + rloc * 2 * HW;
+    uint2 *ab = reinterpret_cast<uint2 *>(smw + (TAB ? cfg.TH * 32 * HW : 0)) + rloc * 8 * HW * NR;  // MULTI: [child][group in its word][word]
+    uint32_t *planes = smw + (TAB ? cfg.TH * 32 * HW : 0) + (MULTI ? cfg.RPC * 16 * HW : 0);
+    uint32_t *pl = planes + NR * rloc * 2 * HW;  // child n: pl + 2 n HW
     int32_t *acc = reinterpret_cast<int32_t *>(planes + cfg.RPC * 2 * HW);
 
     uint32_t tile = MANY ? blockIdx.x * cfg.K : blockIdx.x;
@@ -1344,14 +1344,21 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const ui
         if (TAB) fill_shared_parts(tab, HW, 0, in_tab, lo1_0, K);
         const uint4 *tp = tab;
 
-        // Word w of colour c in half-sweep h: the new spins.
+        // Word w of colour c in half-sweep h: the children's spins S become the new ones.
         ChildPart cp;
-        auto sweep_word = [&](uint32_t c, uint32_t w, uint32_t h, uint32_t S) {
-            uint32_t same, rot, up, dn, c0, ge2;
-            plane_neighbours(pl + (c ^ 1u) * HW, HW, Lh, c, w, same, rot, up, dn);
-            count_bonds(S ^ same ^ J[c][0], S ^ rot ^ J[c][1], S ^ up ^ J[c][2], S ^ dn ^ J[c][3], c0, ge2);
-            const SiteNibbles nib = site_nibbles(c0);
-            uint32_t B = 0;
+        uint32_t x2[NR];  // MULTI: the children's own part
+        auto sweep_word = [&](uint32_t c, uint32_t w, uint32_t h, uint32_t (&S)[NR]) {
+            uint32_t c0[NR], ge2[NR], B[NR];
+            SiteNibbles nib[NR];
+#pragma unroll
+            for (uint32_t n = 0; n < NR; ++n) {
+                uint32_t same, rot, up, dn;
+                plane_neighbours(pl + (2 * n + (c ^ 1u)) * HW, HW, Lh, c, w, same, rot, up, dn);
+                count_bonds(S[n] ^ same ^ J[c][0], S[n] ^ rot ^ J[c][1], S[n] ^ up ^ J[c][2], S[n] ^ dn ^ J[c][3],
+                            c0[n], ge2[n]);
+                nib[n] = site_nibbles(c0[n]);
+                B[n] = 0;
+            }
 #pragma unroll
             for (uint32_t q = 0; q < 8; ++q) {
                 SharedPart v;
@@ -1361,14 +1368,19 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const ui
                 } else {
                     v = philox_shared(8 * w + q, (TAG_SWEEP << 24) | h, lo1_0, K);
                 }
-                if (MULTI) {
-                    const uint2 e = ab[q * HW + w];
-                    cp.a[q] = e.x;
-                    cp.b[q] = e.y;
+#pragma unroll
+                for (uint32_t n = 0; n < NR; ++n) {
+                    if (MULTI) {
+                        const uint2 e = ab[(8 * n + q) * HW + w];
+                        cp.x2 = x2[n];
+                        cp.a[q] = e.x;
+                        cp.b[q] = e.y;
+                    }
+                    accept_group(B[n], philox_join(cp, q, v, K), q, nib[n], s_thr);
                 }
-                accept_group(B, philox_join(cp, q, v, K), q, nib, s_thr);
             }
-            return S ^ (ge2 | B | (c0 & all1) | all2);
+#pragma unroll
+            for (uint32_t n = 0; n < NR; ++n) S[n] ^= ge2[n] | B[n] | (c0[n] & all1) | all2;
         };
 
         for (; tile < stop; ++tile) {
@@ -1377,26 +1389,34 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const ui
                 tile = stop;
                 break;
             }
-            const uint32_t child = tile0 + rloc;
-            const bool active = child < Rn;
-            uint32_t own[2] = {0u, 0u}, parent = 0;
-            if (active) parent = P.parent[rd.rep_off + child];
-            const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent * rd.wstride;
-            if (MULTI) {
-                for (uint32_t w = tl; w < HW; w += TPR) {
-                    philox_child(cp, 8 * w, child, hi1_0, K);
+            const uint32_t child = tile0 + NR * rloc;  // the thread's children: child .. child + NR - 1
+            uint32_t own[2] = {0u, 0u}, parent[NR];
 #pragma unroll
-                    for (uint32_t q = 0; q < 8; ++q) ab[q * HW + w] = make_uint2(cp.a[q], cp.b[q]);
-                }
+            for (uint32_t n = 0; n < NR; ++n) parent[n] = child + n < Rn ? P.parent[rd.rep_off + child + n] : 0u;
+            if (MULTI) {
+#pragma unroll
+                for (uint32_t n = 0; n < NR; ++n)
+                    for (uint32_t w = tl; w < HW; w += TPR) {
+                        philox_child(cp, 8 * w, child + n, hi1_0, K);
+                        x2[n] = cp.x2;
+#pragma unroll
+                        for (uint32_t q = 0; q < 8; ++q) ab[(8 * n + q) * HW + w] = make_uint2(cp.a[q], cp.b[q]);
+                    }
             } else {
                 philox_child(cp, 8 * tl, child, hi1_0, K);
             }
-            if (WIDE && tl == 0) acc[2 * rloc] = acc[2 * rloc + 1] = 0;
+            if (WIDE && tl == 0)
 #pragma unroll
-            for (uint32_t q = 0; q < 2 * WPT; ++q) {
-                const uint32_t v = active ? src[q * TPR + tl] : 0u;
-                if (!MULTI) own[q & 1u] = v;  // one word per thread: q is the colour
-                pl[q * TPR + tl] = v;
+                for (uint32_t n = 0; n < 2 * NR; ++n) acc[2 * NR * rloc + n] = 0;
+#pragma unroll
+            for (uint32_t n = 0; n < NR; ++n) {
+                const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent[n] * rd.wstride;
+#pragma unroll
+                for (uint32_t q = 0; q < 2 * WPT; ++q) {
+                    const uint32_t v = child + n < Rn ? src[q * TPR + tl] : 0u;
+                    if (!MULTI) own[q & 1u] = v;  // one word per thread: q is the colour
+                    pl[2 * n * HW + q * TPR + tl] = v;
+                }
             }
             if (MANY && TAB && tab_h != 0) {  // a schedule longer than the table: back to its start
                 __syncthreads();
@@ -1424,11 +1444,17 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const ui
 #pragma unroll 1
                         for (uint32_t w = tl; w < HW; w += TPR) {
                             if (SG) bonds(c, w);
-                            pl[c * HW + w] = sweep_word(c, w, h, pl[c * HW + w]);
+                            uint32_t S[NR];
+#pragma unroll
+                            for (uint32_t n = 0; n < NR; ++n) S[n] = pl[(2 * n + c) * HW + w];
+                            sweep_word(c, w, h, S);
+#pragma unroll
+                            for (uint32_t n = 0; n < NR; ++n) pl[(2 * n + c) * HW + w] = S[n];
                         }
                     } else {
-                        own[c] = sweep_word(c, tl, h, own[c]);
-                        pl[c * HW + tl] = own[c];
+                        uint32_t S[NR] = {own[c]};
+                        sweep_word(c, tl, h, S);
+                        pl[c * HW + tl] = own[c] = S[0];
                     }
                     if (TAB) tp += 8 * HW;
                     if (WIDE)
@@ -1438,47 +1464,55 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const ui
                 }
             }
 
-            // child: planes, E from the final lattice (every bond touches one colour-0 site), M
-            int32_t unsat = 0, up1 = 0;
-            if (active) {
-                uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)child * rd.wstride;
+            // children: planes, E from the final lattice (every bond touches one colour-0 site), M
 #pragma unroll
-                for (uint32_t q = 0; q < WPT; ++q) {
-                    const uint32_t w = q * TPR + tl;
-                    const uint32_t S = MULTI ? pl[w] : own[0], S1 = MULTI ? pl[HW + w] : own[1];
-                    dst[w] = S;
-                    dst[HW + w] = S1;
-                    if (SG && MULTI) bonds(0, w);
-                    uint32_t same, rot, up, dn;
-                    plane_neighbours(pl + HW, HW, Lh, 0, w, same, rot, up, dn);
-                    unsat += __popc(S ^ same ^ J[0][0]) + __popc(S ^ rot ^ J[0][1]) + __popc(S ^ up ^ J[0][2]) +
-                             __popc(S ^ dn ^ J[0][3]);
-                    up1 += __popc(S) + __popc(S1);
-                }
-            }
-            if (!WIDE) {
+            for (uint32_t n = 0; n < NR; ++n) {
+                const bool here = child + n < Rn;
+                int32_t unsat = 0, up1 = 0;
+                if (here) {
+                    uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)(child + n) * rd.wstride;
+                    const uint32_t *pn = pl + 2 * n * HW;
 #pragma unroll
-                for (uint32_t o = 1; o < TPR; o <<= 1) {
-                    unsat += __shfl_xor_sync(FULL, unsat, o);
-                    up1 += __shfl_xor_sync(FULL, up1, o);
+                    for (uint32_t q = 0; q < WPT; ++q) {
+                        const uint32_t w = q * TPR + tl;
+                        const uint32_t S = MULTI ? pn[w] : own[0], S1 = MULTI ? pn[HW + w] : own[1];
+                        dst[w] = S;
+                        dst[HW + w] = S1;
+                        if (SG && MULTI) bonds(0, w);
+                        uint32_t same, rot, up, dn;
+                        plane_neighbours(pn + HW, HW, Lh, 0, w, same, rot, up, dn);
+                        unsat += __popc(S ^ same ^ J[0][0]) + __popc(S ^ rot ^ J[0][1]) + __popc(S ^ up ^ J[0][2]) +
+                                 __popc(S ^ dn ^ J[0][3]);
+                        up1 += __popc(S) + __popc(S1);
+                    }
                 }
-            } else {
-                if (active) {
-                    atomicAdd(&acc[2 * rloc], unsat);
-                    atomicAdd(&acc[2 * rloc + 1], up1);
+                int32_t *sums = acc + 2 * (NR * rloc + n);
+                if (!WIDE) {
+#pragma unroll
+                    for (uint32_t o = 1; o < TPR; o <<= 1) {
+                        unsat += __shfl_xor_sync(FULL, unsat, o);
+                        up1 += __shfl_xor_sync(FULL, up1, o);
+                    }
+                } else if (here) {
+                    atomicAdd(&sums[0], unsat);
+                    atomicAdd(&sums[1], up1);
                 }
-                __syncthreads();
-                if (tl == 0) {
-                    unsat = acc[2 * rloc];
-                    up1 = acc[2 * rloc + 1];
+                if (!WIDE && here && tl == 0) {
+                    sums[0] = unsat;
+                    sums[1] = up1;
                 }
             }
-            if (active && tl == 0) {
-                const uint64_t pc = rd.rep_off + parent, cc = rd.rep_off + child;
-                P.E[nbuf][cc] = 2 * unsat - 2 * (int32_t)N;
-                P.M[nbuf][cc] = 2 * up1 - (int32_t)N;
-                P.fam[nbuf][cc] = P.fam[ob][pc];
-            }
+            if (WIDE) __syncthreads();
+            if (tl == 0)
+#pragma unroll
+                for (uint32_t n = 0; n < NR; ++n)
+                    if (child + n < Rn) {
+                        const int32_t *sums = acc + 2 * (NR * rloc + n);
+                        const uint64_t pc = rd.rep_off + parent[n], cc = rd.rep_off + child + n;
+                        P.E[nbuf][cc] = 2 * sums[0] - 2 * (int32_t)N;
+                        P.M[nbuf][cc] = 2 * sums[1] - (int32_t)N;
+                        P.fam[nbuf][cc] = P.fam[ob][pc];
+                    }
             if (!MANY) return;
             if (!WIDE) __syncwarp();  // the planes are read before the next tile's are stored
         }
@@ -1695,10 +1729,11 @@ __global__ void __launch_bounds__(256, PA_PAD_MIN_BLOCKS) sweep_pad_kernel(Pool 
 // slower here, 1367 against 1415 updates/ns at L = 30).  A barrier ends every
 // half-sweep; the block sizes tried are those that fill whole groups of four warps
 // best, as an SM's four sub-partitions share a CTA's warps evenly then (L = 100: 471
-// threads 1357 updates/ns, 157 threads 1160 at 2 CTAs' worth of registers).  Four
-// CTAs of 256 threads per SM (64 registers): 128 registers are 1 to 9 % slower.
-// Measured (theta = 10, as above): L = 20 glass 1146 -> 1324 updates/ns, L = 30
-// 1293 -> 1422, L = 46 1256 -> 1435, L = 100 1247 -> 1345.
+// threads 1357 updates/ns, 157 threads 1160 at 2 CTAs' worth of registers).  NR
+// children per thread share a group's shared part, their child parts in shared memory,
+// at three CTAs of 256 threads per SM (80 registers; two or four: 6 or 1 % slower).
+// Measured (theta = 10, as above): L = 20 glass 1146 -> 1375 updates/ns, L = 30
+// 1293 -> 1488, L = 46 1256 -> 1468, L = 100 1247 -> 1380.
 // --------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t low_bits(uint32_t n) { return n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u; }
 
@@ -1908,12 +1943,13 @@ __global__ void __launch_bounds__(128)
     }
 }
 
-template <bool SG, int MAXT, int MINB, bool NARROW>
+template <bool SG, int MAXT, int MINB, bool NARROW, uint32_t NR>
 __global__ void __launch_bounds__(MAXT, MINB)
     sweep_compact_kernel(Pool P, const uint32_t *group_runs, const uint32_t *tile_off, uint32_t n_group_runs,
                          SweepCfg cfg)
 {
-    extern __shared__ __align__(16) uint32_t smw[];  // geometry, bond masks (SG), planes, sums
+    // shared memory: geometry, child parts (NR > 1), bond masks (SG), planes, sums
+    extern __shared__ __align__(16) uint32_t smw[];
     __shared__ uint4 s_thr[16];
     uint32_t tile = blockIdx.x * cfg.K;
     const uint32_t tend = min(tile + cfg.K, tile_off[n_group_runs]);
@@ -1924,9 +1960,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const uint32_t FP = (Lh + 31) >> 5, AW = FP + CW + (Lh >> 5) + 2, base = 32 * FP;
     const uint32_t rloc = threadIdx.x / CW, w = threadIdx.x - rloc * CW;
     CompactWord *geo = reinterpret_cast<CompactWord *>(smw);
-    uint32_t *Jw = reinterpret_cast<uint32_t *>(geo + CW);  // [colour][neighbour][word]
+    uint2 *ab = reinterpret_cast<uint2 *>(geo + CW) + rloc * 8 * NR * CW;  // [child][group in its word][word]
+    uint32_t *Jw = reinterpret_cast<uint32_t *>(geo + CW) + (NR > 1 ? cfg.RPC * 16 * CW : 0);  // [colour][neighbour][word]
     uint32_t *planes = Jw + (SG ? 8 * CW : 0);
-    uint32_t *pl = planes + rloc * 2 * AW;
+    uint32_t *pl = planes + NR * rloc * 2 * AW;  // child n: pl + 2 n AW
     int32_t *acc = reinterpret_cast<int32_t *>(planes + cfg.RPC * 2 * AW);
     if (threadIdx.x < CW) geo[w] = compact_word(w, Lh, NB, base);  // rloc = 0
     const CompactShifts z = compact_shifts(Lh);
@@ -1971,20 +2008,29 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 tile = stop;
                 break;
             }
-            const uint32_t child = tile0 + rloc;
-            const bool active = child < Rn;
-            uint32_t own[2] = {0u, 0u}, parent = 0;
-            if (active) {
-                parent = P.parent[rd.rep_off + child];
-                const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent * rd.wstride;
-                own[0] = compact_from_padded(src, pitch, Lh, NB, w);
-                own[1] = compact_from_padded(src + PW, pitch, Lh, NB, w);
-            }
-            pl[FP + w] = own[0];
-            pl[AW + FP + w] = own[1];
-            if (w == 0) acc[2 * rloc] = acc[2 * rloc + 1] = 0;
+            const uint32_t child = tile0 + NR * rloc;  // the thread's children: child .. child + NR - 1
+            uint32_t own[NR][2], parent[NR], x2[NR];
             ChildPart cp;
-            philox_child(cp, 8 * w, child, hi1_0, K);
+#pragma unroll
+            for (uint32_t n = 0; n < NR; ++n) {
+                own[n][0] = own[n][1] = parent[n] = 0;
+                if (child + n < Rn) {
+                    parent[n] = P.parent[rd.rep_off + child + n];
+                    const uint32_t *src = P.spins[ob] + rd.spin_off + (uint64_t)parent[n] * rd.wstride;
+                    own[n][0] = compact_from_padded(src, pitch, Lh, NB, w);
+                    own[n][1] = compact_from_padded(src + PW, pitch, Lh, NB, w);
+                }
+                pl[2 * n * AW + FP + w] = own[n][0];
+                pl[(2 * n + 1) * AW + FP + w] = own[n][1];
+                philox_child(cp, 8 * w, child + n, hi1_0, K);
+                x2[n] = cp.x2;
+                if (NR > 1)
+#pragma unroll
+                    for (uint32_t q = 0; q < 8; ++q) ab[(8 * n + q) * CW + w] = make_uint2(cp.a[q], cp.b[q]);
+            }
+            if (w == 0)
+#pragma unroll
+                for (uint32_t n = 0; n < 2 * NR; ++n) acc[2 * NR * rloc + n] = 0;
             __syncthreads();
 
             for (uint32_t t = 0; t < rd.theta; ++t) {
@@ -1992,61 +2038,85 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 for (uint32_t c = 0; c < 2; ++c) {
                     const uint32_t h = 2 * t + c;
                     const CompactWord g = geo[w];
-                    uint32_t same, rot, up, dn, c0, ge2;
-                    compact_neighbours<NARROW>(pl + (c ^ 1u) * AW, pl + (c ^ 1u) * AW + FP + w, z, g, c, same, rot,
-                                               up, dn);
-                    const uint32_t S = own[c];
-                    if (SG) {
-                        same ^= Jw[4 * c * CW + w];
-                        rot ^= Jw[(4 * c + 1) * CW + w];
-                        up ^= Jw[(4 * c + 2) * CW + w];
-                        dn ^= Jw[(4 * c + 3) * CW + w];
+                    uint32_t c0[NR], ge2[NR], B[NR];
+                    SiteNibbles nib[NR];
+#pragma unroll
+                    for (uint32_t n = 0; n < NR; ++n) {
+                        const uint32_t *O = pl + (2 * n + (c ^ 1u)) * AW;
+                        uint32_t same, rot, up, dn;
+                        compact_neighbours<NARROW>(O, O + FP + w, z, g, c, same, rot, up, dn);
+                        const uint32_t S = own[n][c];
+                        if (SG) {
+                            same ^= Jw[4 * c * CW + w];
+                            rot ^= Jw[(4 * c + 1) * CW + w];
+                            up ^= Jw[(4 * c + 2) * CW + w];
+                            dn ^= Jw[(4 * c + 3) * CW + w];
+                        }
+                        count_bonds(S ^ same, S ^ rot, S ^ up, S ^ dn, c0[n], ge2[n]);
+                        nib[n] = site_nibbles(c0[n]);
+                        B[n] = 0;
                     }
-                    count_bonds(S ^ same, S ^ rot, S ^ up, S ^ dn, c0, ge2);
-                    const SiteNibbles nib = site_nibbles(c0);
-                    uint32_t B = 0;
 #pragma unroll
                     for (uint32_t q = 0; q < 8; ++q) {
                         const SharedPart v = philox_shared(8 * w + q, (TAG_SWEEP << 24) | h, lo1_0, K);
-                        accept_group(B, philox_join(cp, q, v, K), q, nib, s_thr);
+#pragma unroll
+                        for (uint32_t n = 0; n < NR; ++n) {
+                            if (NR > 1) {
+                                const uint2 e = ab[(8 * n + q) * CW + w];
+                                cp.x2 = x2[n];
+                                cp.a[q] = e.x;
+                                cp.b[q] = e.y;
+                            }
+                            accept_group(B[n], philox_join(cp, q, v, K), q, nib[n], s_thr);
+                        }
                     }
-                    const uint32_t flip = (ge2 | B | (c0 & all1) | all2) & g.VM;
-                    own[c] = S ^ flip;
-                    pl[c * AW + FP + w] = own[c];
+#pragma unroll
+                    for (uint32_t n = 0; n < NR; ++n) {
+                        own[n][c] ^= (ge2[n] | B[n] | (c0[n] & all1) | all2) & g.VM;
+                        pl[(2 * n + c) * AW + FP + w] = own[n][c];
+                    }
                     __syncthreads();
                 }
             }
 
-            // child: planes back in their padded rows, E from the final lattice (every bond
+            // children: planes back in their padded rows, E from the final lattice (every bond
             // touches one colour-0 site), M
-            if (active) {
-                uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)child * rd.wstride;
-                for (uint32_t p = w; p < PW; p += CW) {
-                    dst[p] = padded_from_compact(pl, base, pitch, Lh, p);
-                    dst[PW + p] = padded_from_compact(pl + AW, base, pitch, Lh, p);
+#pragma unroll
+            for (uint32_t n = 0; n < NR; ++n)
+                if (child + n < Rn) {
+                    const uint32_t *pn = pl + 2 * n * AW;
+                    int32_t *sums = acc + 2 * (NR * rloc + n);
+                    uint32_t *dst = P.spins[nbuf] + rd.spin_off + (uint64_t)(child + n) * rd.wstride;
+                    for (uint32_t p = w; p < PW; p += CW) {
+                        dst[p] = padded_from_compact(pn, base, pitch, Lh, p);
+                        dst[PW + p] = padded_from_compact(pn + AW, base, pitch, Lh, p);
+                    }
+                    const CompactWord g = geo[w];
+                    uint32_t same, rot, up, dn;
+                    compact_neighbours<NARROW>(pn + AW, pn + AW + FP + w, z, g, 0, same, rot, up, dn);
+                    if (SG) {
+                        same ^= Jw[w];
+                        rot ^= Jw[CW + w];
+                        up ^= Jw[2 * CW + w];
+                        dn ^= Jw[3 * CW + w];
+                    }
+                    const uint32_t S = own[n][0];
+                    const int32_t unsat = __popc((S ^ same) & g.VM) + __popc((S ^ rot) & g.VM) +
+                                          __popc((S ^ up) & g.VM) + __popc((S ^ dn) & g.VM);
+                    atomicAdd(&sums[0], unsat);
+                    atomicAdd(&sums[1], __popc(own[n][0]) + __popc(own[n][1]));
                 }
-                const CompactWord g = geo[w];
-                uint32_t same, rot, up, dn;
-                compact_neighbours<NARROW>(pl + AW, pl + AW + FP + w, z, g, 0, same, rot, up, dn);
-                if (SG) {
-                    same ^= Jw[w];
-                    rot ^= Jw[CW + w];
-                    up ^= Jw[2 * CW + w];
-                    dn ^= Jw[3 * CW + w];
-                }
-                const uint32_t S = own[0];
-                const int32_t unsat = __popc((S ^ same) & g.VM) + __popc((S ^ rot) & g.VM) + __popc((S ^ up) & g.VM) +
-                                      __popc((S ^ dn) & g.VM);
-                atomicAdd(&acc[2 * rloc], unsat);
-                atomicAdd(&acc[2 * rloc + 1], __popc(own[0]) + __popc(own[1]));
-            }
             __syncthreads();
-            if (active && w == 0) {
-                const uint64_t pc = rd.rep_off + parent, cc = rd.rep_off + child;
-                P.E[nbuf][cc] = 2 * acc[2 * rloc] - 2 * (int32_t)N;
-                P.M[nbuf][cc] = 2 * acc[2 * rloc + 1] - (int32_t)N;
-                P.fam[nbuf][cc] = P.fam[ob][pc];
-            }
+            if (w == 0)
+#pragma unroll
+                for (uint32_t n = 0; n < NR; ++n)
+                    if (child + n < Rn) {
+                        const int32_t *sums = acc + 2 * (NR * rloc + n);
+                        const uint64_t pc = rd.rep_off + parent[n], cc = rd.rep_off + child + n;
+                        P.E[nbuf][cc] = 2 * sums[0] - 2 * (int32_t)N;
+                        P.M[nbuf][cc] = 2 * sums[1] - (int32_t)N;
+                        P.fam[nbuf][cc] = P.fam[ob][pc];
+                    }
         }
     }
 }
@@ -3961,14 +4031,23 @@ cudaError_t prepare_kernels()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(resample_multinomial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  multinomial_smem(RESAMPLE_STAGE_MAX, MULTI_LEVELS));
-    for (void *k : {(void *)sweep_pow2_kernel<true, 1024, 4, false, true, 256, 2>,
-                    (void *)sweep_pow2_kernel<false, 1024, 4, false, true, 256, 2>,
-                    (void *)sweep_pow2_kernel<true, 1024, 4, false, false, 256, 2>,
-                    (void *)sweep_pow2_kernel<false, 1024, 4, false, false, 256, 2>})  // planes, child parts: 72 KB
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
-    for (void *k : {(void *)sweep_compact_kernel<true, 1024, 1, false>, (void *)sweep_compact_kernel<false, 1024, 1, false>})
-        if (e == cudaSuccess)  // geometry, bond masks and planes of up to 1009 words: 73 KB
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 80 * 1024);
+    for (void *k : {(void *)sweep_pow2_kernel<true, 1024, 2, 2, false, true, 512, 1>,
+                    (void *)sweep_pow2_kernel<true, 1024, 2, 2, false, false, 512, 1>,
+                    (void *)sweep_pow2_kernel<false, 1024, 2, 2, false, true, 512, 1>,
+                    (void *)sweep_pow2_kernel<false, 1024, 2, 2, false, false, 512, 1>,
+                    (void *)sweep_pow2_kernel<true, 16, 1, 2, true, true, 256, 2>,
+                    (void *)sweep_pow2_kernel<true, 16, 1, 2, true, false, 256, 2>,
+                    (void *)sweep_pow2_kernel<false, 16, 1, 2, true, true, 256, 2>,
+                    (void *)sweep_pow2_kernel<false, 16, 1, 2, true, false, 256, 2>})  // 144 and 52 KB
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
+    for (void *k : {(void *)sweep_compact_kernel<true, 1024, 1, false, 1>,
+                    (void *)sweep_compact_kernel<false, 1024, 1, false, 1>,
+                    (void *)sweep_compact_kernel<true, 256, 3, true, 2>, (void *)sweep_compact_kernel<false, 256, 3, true, 2>,
+                    (void *)sweep_compact_kernel<true, 256, 3, false, 2>, (void *)sweep_compact_kernel<false, 256, 3, false, 2>,
+                    (void *)sweep_compact_kernel<true, 512, 2, true, 2>, (void *)sweep_compact_kernel<false, 512, 2, true, 2>,
+                    (void *)sweep_compact_kernel<true, 512, 2, false, 2>, (void *)sweep_compact_kernel<false, 512, 2, false, 2>})
+        if (e == cudaSuccess)  // geometry and bond masks of up to 1009 words, child parts of up to 512
+            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
     if (e == cudaSuccess)  // Wang pairing with R_cap up to 8192: 144 KB
         e = cudaFuncSetAttribute(wang_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     return e;
@@ -4027,7 +4106,7 @@ void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_run
 // Launch shapes of the bit-sliced power-of-two kernel: WPT plane words per thread, `block`
 // threads per CTA (a multiple of the HW / WPT threads of a replica) and TH half-sweeps of
 // shared Philox parts in the table (0: no table).
-SweepCfg sweep_fast_config(uint32_t L, uint32_t WPT, uint32_t block, uint32_t TH)
+SweepCfg sweep_fast_config(uint32_t L, uint32_t WPT, uint32_t NR, uint32_t block, uint32_t TH)
 {
     SweepCfg c{};
     const uint32_t HW = L * L / 64;
@@ -4036,11 +4115,12 @@ SweepCfg sweep_fast_config(uint32_t L, uint32_t WPT, uint32_t block, uint32_t TH
     c.WPT = WPT;
     c.TPR = HW / WPT;
     c.block = block;
-    c.RPC = block / c.TPR;
+    c.NR = NR;
+    c.RPC = NR * (block / c.TPR);
     c.G = 8 * HW;
     c.PS = 0;
     c.TH = TH;
-    c.smem = TH * c.G * 16 + (WPT > 1 ? c.RPC * c.G * 8 : 0) + c.RPC * 2 * HW * 4 + 8 * c.RPC;
+    c.smem = TH * c.G * 16 + (WPT * NR > 1 ? c.RPC * c.G * 8 : 0) + c.RPC * 2 * HW * 4 + 8 * c.RPC;
     return c;
 }
 
@@ -4050,19 +4130,25 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
     const uint32_t N = L * L;
     const bool pow2 = L >= 8 && L <= 256 && (L & (L - 1)) == 0;
     if (pow2 && allow_fast) {
-        // Updates/ns of each shape (40 ferromagnet runs, 4e8 spins, theta = 10); the tuner picks.
-        if (L <= 32) {  // tables of 5 to 16 KB; L = 32: 1790, without a table 1654
-            const uint32_t TH = L == 8 ? 40 : L == 16 ? 20 : 8;
-            v.push_back(sweep_fast_config(L, 1, 256, TH));  // L = 8, 16, 32: 1875, 1859, 1790
-            v.push_back(sweep_fast_config(L, 1, 128, TH));  // 1882, 1849, 1776
-        } else if (L == 64) {  // a table of two half-sweeps, filled by 4 replicas: 1616
-            v.push_back(sweep_fast_config(L, 1, 128, 0));  // 1786
-            v.push_back(sweep_fast_config(L, 1, 256, 0));  // 1760
-        } else if (L == 128) {  // with a table for 2 or 4 replicas: 1418, 1455
-            v.push_back(sweep_fast_config(L, 1, 256, 0));  // 1788
-        } else {  // L = 256: one replica per CTA
-            v.push_back(sweep_fast_config(L, 4, 256, 0));   // 1668
-            v.push_back(sweep_fast_config(L, 1, 1024, 0));  // 1605; the faster one for few replicas
+        // Updates/ns of each shape (40 ferromagnet runs, 4e8 spins, theta = 10); the tuner picks.  The
+        // second one of L >= 32 takes one child per thread, for populations too small to fill the
+        // GPU with two.
+        if (L <= 16) {  // tables of 5 and 10 KB; two children per thread: 1501, 1865
+            const uint32_t TH = L == 8 ? 40 : 20;
+            v.push_back(sweep_fast_config(L, 1, 1, 256, TH));  // L = 8, 16: 1902, 1868
+            v.push_back(sweep_fast_config(L, 1, 1, 128, TH));  // 1901, 1868
+        } else if (L == 32) {  // a table of 16 KB; two children without it: 1850
+            v.push_back(sweep_fast_config(L, 1, 2, 256, 8));  // 1875
+            v.push_back(sweep_fast_config(L, 1, 1, 128, 8));  // 1794
+        } else if (L == 64) {  // a table of two half-sweeps: 1616; four children: 1825
+            v.push_back(sweep_fast_config(L, 1, 2, 128, 0));  // 1875
+            v.push_back(sweep_fast_config(L, 1, 1, 128, 0));  // 1792
+        } else if (L == 128) {  // with a table: 1455; four children: 1810
+            v.push_back(sweep_fast_config(L, 1, 2, 256, 0));  // 1854
+            v.push_back(sweep_fast_config(L, 1, 1, 256, 0));  // 1789
+        } else {  // L = 256: 4 words of one child by 256 threads: 1664
+            v.push_back(sweep_fast_config(L, 2, 2, 512, 0));   // 1781
+            v.push_back(sweep_fast_config(L, 1, 1, 1024, 0));  // 1648
         }
         return v;
     }
@@ -4070,32 +4156,46 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
     if (allow_fast && CW <= 1024) {  // compact rows
         // The replicas of a CTA of at most `target` threads that leave the fewest lanes idle in
         // whole groups of four warps (one per SM sub-partition).
-        auto shape = [&](uint32_t target) {
+        auto shape = [&](uint32_t target, uint32_t NR) {
             SweepCfg c{};
             c.K = 1;
             c.fast = 3;
             c.WPT = 1;
             c.TPR = CW;
-            c.RPC = 1;
+            c.NR = NR;
+            uint32_t at_once = 1;
             double best = 0.0;
             for (uint32_t r = 1; r * CW <= target; ++r) {
                 const double used = (double)(r * CW) / ((r * CW + 127) / 128 * 128);
                 if (used >= best) {
                     best = used;
-                    c.RPC = r;
+                    at_once = r;
                 }
             }
-            c.block = c.RPC * CW;
+            c.RPC = NR * at_once;
+            c.block = at_once * CW;
             c.G = 8 * CW;
             c.PS = Pt;
             c.Lh = Lh;
             c.pw = plane_words_of(L);
-            // geometry, bond masks, planes, sums
-            c.smem = CW * 32 + CW * 32 + c.RPC * 2 * ((Lh + 31) / 32 + CW + Lh / 32 + 2) * 4 + 8 * c.RPC;
-            if (v.empty() || v.back().block != c.block) v.push_back(c);
+            // geometry, child parts, bond masks, planes, sums
+            c.smem = CW * 32 + (NR > 1 ? c.RPC * c.G * 8 : 0) + CW * 32 +
+                     c.RPC * 2 * ((Lh + 31) / 32 + CW + Lh / 32 + 2) * 4 + 8 * c.RPC;
+            if (v.empty() || v.back().block != c.block || v.back().NR != NR) v.push_back(c);
         };
-        shape(256);
-        shape(512);
+        // Updates/ns (40 runs, 4e8 spins, theta = 10) of 256 threads with one child each, 256 and 512
+        // with two: L = 6 816, 356, 347; L = 10 1170, 1083, 1039; L = 30 1415, 1488, 1404; L = 46 1374,
+        // 1451, 1468; L = 100 1305, 1374, 1380.
+        if (CW <= 4) {
+            shape(256, 1);
+            shape(256, 2);
+        } else if (CW <= 256) {
+            shape(256, 2);
+            shape(512, 2);
+            shape(256, 1);
+        } else {
+            shape(CW, 1);
+        }
     }
     // Padded rows draw only the 6 Philox groups that a word of 4 rows holds at L = 12, where the
     // compact planes end in a word three quarters empty: 1218 against 1138 updates/ns there; at
@@ -4154,30 +4254,34 @@ void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *til
     if (many) cfg.K = std::min(8u, std::max(1u, n_tiles / (152 * 4 * 4)));
     if (cfg.fast == 3) cfg.K = std::min(4u, std::max(1u, n_tiles / (152 * 2 * 16)));
     const dim3 grid((n_tiles + cfg.K - 1) / cfg.K);
-#define PA_SWEEP_FAST_(SG, HW, WPT, TAB, MANY, MAXT, MINB)                                                          \
-    sweep_pow2_kernel<SG, HW, WPT, TAB, MANY, MAXT, MINB><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, \
+#define PA_SWEEP_FAST_(SG, HW, WPT, NR, TAB, MANY, MAXT, MINB)                                                        \
+    sweep_pow2_kernel<SG, HW, WPT, NR, TAB, MANY, MAXT, MINB><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, \
                                                                                             n_group_runs, cfg)
-#define PA_SWEEP_FAST(HW, WPT, TAB, MAXT, MINB)                                                              \
-    (any_glass ? (many ? PA_SWEEP_FAST_(true, HW, WPT, TAB, true, MAXT, MINB)                                \
-                       : PA_SWEEP_FAST_(true, HW, WPT, TAB, false, MAXT, MINB))                              \
-               : (many ? PA_SWEEP_FAST_(false, HW, WPT, TAB, true, MAXT, MINB)                               \
-                       : PA_SWEEP_FAST_(false, HW, WPT, TAB, false, MAXT, MINB)))
+#define PA_SWEEP_FAST(HW, WPT, NR, TAB, MAXT, MINB)                                                            \
+    (any_glass ? (many ? PA_SWEEP_FAST_(true, HW, WPT, NR, TAB, true, MAXT, MINB)                                \
+                       : PA_SWEEP_FAST_(true, HW, WPT, NR, TAB, false, MAXT, MINB))                              \
+               : (many ? PA_SWEEP_FAST_(false, HW, WPT, NR, TAB, true, MAXT, MINB)                               \
+                       : PA_SWEEP_FAST_(false, HW, WPT, NR, TAB, false, MAXT, MINB)))
     if (cfg.fast == 3) {  // compact rows; the row pitch is at most 32 exactly when L/2 <= 31
-#define PA_SWEEP_COMPACT(MAXT, MINB, NARROW)                                                                       \
-    (any_glass ? sweep_compact_kernel<true, MAXT, MINB, NARROW><<<grid, cfg.block, cfg.smem, s>>>(                 \
+#define PA_SWEEP_COMPACT(MAXT, MINB, NARROW, NR)                                                                   \
+    (any_glass ? sweep_compact_kernel<true, MAXT, MINB, NARROW, NR><<<grid, cfg.block, cfg.smem, s>>>(             \
                      P, group_runs, tile_off, n_group_runs, cfg)                                                   \
-               : sweep_compact_kernel<false, MAXT, MINB, NARROW><<<grid, cfg.block, cfg.smem, s>>>(                \
+               : sweep_compact_kernel<false, MAXT, MINB, NARROW, NR><<<grid, cfg.block, cfg.smem, s>>>(            \
                      P, group_runs, tile_off, n_group_runs, cfg))
-        if (cfg.block <= 256 && cfg.PS <= 32)
-            PA_SWEEP_COMPACT(256, 4, true);
+        if (cfg.NR == 2 && cfg.block <= 256 && cfg.PS <= 32)
+            PA_SWEEP_COMPACT(256, 3, true, 2);
+        else if (cfg.NR == 2 && cfg.block <= 256)
+            PA_SWEEP_COMPACT(256, 3, false, 2);
+        else if (cfg.NR == 2 && cfg.PS <= 32)
+            PA_SWEEP_COMPACT(512, 2, true, 2);
+        else if (cfg.NR == 2)
+            PA_SWEEP_COMPACT(512, 2, false, 2);
+        else if (cfg.block <= 256 && cfg.PS <= 32)
+            PA_SWEEP_COMPACT(256, 4, true, 1);
         else if (cfg.block <= 256)
-            PA_SWEEP_COMPACT(256, 4, false);
-        else if (cfg.block <= 512 && cfg.PS <= 32)
-            PA_SWEEP_COMPACT(512, 2, true);
-        else if (cfg.block <= 512)
-            PA_SWEEP_COMPACT(512, 2, false);
+            PA_SWEEP_COMPACT(256, 4, false, 1);
         else
-            PA_SWEEP_COMPACT(1024, 1, false);
+            PA_SWEEP_COMPACT(1024, 1, false, 1);
 #undef PA_SWEEP_COMPACT
     } else if (cfg.fast == 2) {  // padded rows of pitch 8
         any_glass ? sweep_pad_kernel<true, 8><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg)
@@ -4187,19 +4291,25 @@ void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *til
     else if (!cfg.fast)
         sweep_kernel<false, 1024><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg);
     else if (cfg.G == 8)
-        PA_SWEEP_FAST(1, 1, true, 256, 2);
+        PA_SWEEP_FAST(1, 1, 1, true, 256, 2);
     else if (cfg.G == 8 * 4)
-        PA_SWEEP_FAST(4, 1, true, 256, 2);
+        PA_SWEEP_FAST(4, 1, 1, true, 256, 2);
+    else if (cfg.G == 8 * 16 && cfg.NR == 2)
+        PA_SWEEP_FAST(16, 1, 2, true, 256, 2);
     else if (cfg.G == 8 * 16)
-        PA_SWEEP_FAST(16, 1, true, 256, 2);
+        PA_SWEEP_FAST(16, 1, 1, true, 256, 2);
+    else if (cfg.G == 8 * 64 && cfg.NR == 2)
+        PA_SWEEP_FAST(64, 1, 2, false, 256, 2);
     else if (cfg.G == 8 * 64)
-        PA_SWEEP_FAST(64, 1, false, 256, 2);
+        PA_SWEEP_FAST(64, 1, 1, false, 256, 2);
+    else if (cfg.G == 8 * 256 && cfg.NR == 2)
+        PA_SWEEP_FAST(256, 1, 2, false, 256, 2);
     else if (cfg.G == 8 * 256)
-        PA_SWEEP_FAST(256, 1, false, 256, 2);
-    else if (cfg.WPT == 4)
-        PA_SWEEP_FAST(1024, 4, false, 256, 2);
+        PA_SWEEP_FAST(256, 1, 1, false, 256, 2);
+    else if (cfg.NR == 2)
+        PA_SWEEP_FAST(1024, 2, 2, false, 512, 1);
     else
-        PA_SWEEP_FAST(1024, 1, false, 1024, 1);
+        PA_SWEEP_FAST(1024, 1, 1, false, 1024, 1);
 #undef PA_SWEEP_FAST
 #undef PA_SWEEP_FAST_
 }
