@@ -163,10 +163,13 @@ struct SmallGroup {  // small runs of one lattice size, annealed by anneal_small
     SmallShape ahead = {0, 0, 0, 0, 0};     // several temperatures per launch (cs = 0: none)
 };
 
+constexpr uint32_t SIDE_STREAMS = 3;  // beside the engine's own
+
 struct SweepGroup {  // runs of one lattice size among the resident runs
     uint32_t L = 0;
     int any_glass = 0;
     uint32_t theta_max = 0;
+    double updates = 0;  // per temperature
     std::vector<uint32_t> runs;
     uint64_t runs_off = 0;               // in d_meta
     std::vector<uint64_t> tile_map_off;  // per candidate, in d_meta (n + 1 entries)
@@ -241,6 +244,14 @@ struct pa_engine {
     std::vector<uint32_t> big;         // the other resident runs (per-stage kernels)
     uint64_t big_off = 0;
     std::map<uint32_t, Tuning> tuning;  // per lattice size
+    struct Side {
+        cudaStream_t stream;
+        cudaEvent_t join;
+    };
+    std::vector<Side> side;             // streams the sweeps of several lattice sizes are spread over
+    cudaEvent_t fork = nullptr;
+    bool side_failed = false;
+    std::vector<uint32_t> sweep_order;  // indices of `groups`, most spins to update first
     uint32_t max_Rcap_active = 0, max_N_active = 0, max_pw = 1;
     // execution
     uint64_t launches = 0;
@@ -667,6 +678,8 @@ pa_status admit(pa_engine *e, const pa_run_desc *runs, uint32_t n, uint32_t *slo
     return PA_OK;
 }
 
+void make_side_streams(pa_engine *e);
+
 // Rebuild the device lists (resident runs, overlap runs, per-size work lists,
 // the pending-draw list) after the resident set changed.
 pa_status rebuild(pa_engine *e)
@@ -786,7 +799,13 @@ pa_status rebuild(pa_engine *e)
         g.runs.push_back(s);
         if (e->rd[s].model == PA_EA_PMJ) g.any_glass = 1;
         g.theta_max = std::max(g.theta_max, e->rd[s].theta);
+        g.updates += (double)e->rd[s].theta * e->rd[s].N * e->rd[s].R;
     }
+    e->sweep_order.resize(e->groups.size());
+    for (uint32_t k = 0; k < e->sweep_order.size(); ++k) e->sweep_order[k] = k;
+    std::stable_sort(e->sweep_order.begin(), e->sweep_order.end(),
+                     [&](uint32_t a, uint32_t b) { return e->groups[a].updates > e->groups[b].updates; });
+    make_side_streams(e);
     for (auto &g : e->groups) {
         const Tuning &t = e->tuning[g.L];
         g.runs_off = m.size();
@@ -889,11 +908,58 @@ void timed_launch(pa_engine *e, int kind, F &&launch)
 
 const uint32_t *meta(pa_engine *e, uint64_t off) { return e->d_meta + off; }
 
-void launch_group_sweep(pa_engine *e, const SweepGroup &g, uint32_t c)
+void launch_group_sweep(pa_engine *e, const SweepGroup &g, uint32_t c, cudaStream_t s)
 {
     const Tuning &t = e->tuning[g.L];
     launch_sweep(e->P, meta(e, g.runs_off), meta(e, g.tile_map_off[c]), (uint32_t)g.runs.size(), g.n_tiles[c],
-                 t.candidates[c], g.any_glass, g.theta_max, e->stream);
+                 t.candidates[c], g.any_glass, g.theta_max, s);
+}
+
+// The sweeps of every lattice size.  They touch different runs, and one size's launch is often
+// too short to fill the GPU (a server's size is one run or two) or ends in a partial wave, so they
+// are spread over the engine's stream and side streams, largest first, forked from and joined to
+// the engine's stream by events; what follows on it waits for all of them.  Profiling launches
+// one after another, for the events around each.
+void enqueue_sweeps(pa_engine *e)
+{
+    const size_t n_side = e->profiling || e->groups.size() < 2 ? 0 : std::min(e->groups.size() - 1, e->side.size());
+    if (n_side == 0) {
+        for (auto &g : e->groups)
+            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, e->tuning[g.L].pick, e->stream); });
+        return;
+    }
+    cudaEventRecord(e->fork, e->stream);
+    for (size_t k = 0; k < n_side; ++k) cudaStreamWaitEvent(e->side[k].stream, e->fork, 0);
+    size_t at = 0;
+    for (uint32_t gi : e->sweep_order) {
+        const SweepGroup &g = e->groups[gi];
+        launch_group_sweep(e, g, e->tuning[g.L].pick, at == 0 ? e->stream : e->side[at - 1].stream);
+        at = at == n_side ? 0 : at + 1;
+    }
+    e->launches += e->groups.size();
+    for (size_t k = 0; k < n_side; ++k) {
+        cudaEventRecord(e->side[k].join, e->side[k].stream);
+        cudaStreamWaitEvent(e->stream, e->side[k].join, 0);
+    }
+}
+
+// Side streams for engines with more than one lattice size, created while no capture is running;
+// without them (creation failed) the sweeps stay on the engine's stream.
+void make_side_streams(pa_engine *e)
+{
+    if (e->groups.size() < 2 || !e->side.empty() || e->side_failed) return;
+    bool ok = cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming) == cudaSuccess;
+    for (uint32_t k = 0; ok && k < SIDE_STREAMS; ++k) {
+        pa_engine::Side x{};
+        ok = cudaStreamCreateWithFlags(&x.stream, cudaStreamNonBlocking) == cudaSuccess;
+        if (ok && cudaEventCreateWithFlags(&x.join, cudaEventDisableTiming) != cudaSuccess) {
+            cudaStreamDestroy(x.stream);
+            ok = false;
+        }
+        if (ok) e->side.push_back(x);
+    }
+    if (!ok) (void)cudaGetLastError();
+    e->side_failed = e->side.empty();
 }
 
 // beta_0 draws of the pending runs (Sec. II.B step (i)) and their step-0 measurement.
@@ -982,7 +1048,7 @@ void enqueue_tick(pa_engine *e)
     const uint32_t *act = meta(e, e->big_off);
     const uint32_t na = (uint32_t)e->big.size();
     enqueue_resample(e);
-    for (auto &g : e->groups) timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, e->tuning[g.L].pick); });
+    enqueue_sweeps(e);
     enqueue_dos_sample(e);
     if (!e->q_runs.empty())
         timed_launch(e, PA_K_OVERLAP, [&] {
@@ -1015,13 +1081,13 @@ pa_status enqueue_tuning_tick(pa_engine *e)
     for (auto &g : e->groups) {
         Tuning &t = e->tuning[g.L];
         if (t.tuned) {
-            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, t.pick); });
+            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, t.pick, e->stream); });
             continue;
         }
         bool live = false;  // a run of this size still has a temperature to go
         for (uint32_t r : g.runs) live |= e->rh[r].steps_done + 1 < e->rh[r].d.n_beta;
         if (!live) {
-            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, t.pick); });
+            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, t.pick, e->stream); });
             continue;
         }
         const uint32_t nc = (uint32_t)t.candidates.size();
@@ -1030,7 +1096,7 @@ pa_status enqueue_tuning_tick(pa_engine *e)
         PA_CUDA(cudaEventCreate(&x.a));
         PA_CUDA(cudaEventCreate(&x.b));
         PA_CUDA(cudaEventRecord(x.a, e->stream));
-        launch_group_sweep(e, g, c);
+        launch_group_sweep(e, g, c, e->stream);
         PA_CUDA(cudaEventRecord(x.b, e->stream));
         e->launches += 1;
         timing.push_back(x);
@@ -1249,6 +1315,11 @@ pa_status pa_destroy(pa_engine *e)
         cudaEventDestroy(t.b);
     }
     for (auto ev : e->ev_free) cudaEventDestroy(ev);
+    for (auto &x : e->side) {
+        cudaEventDestroy(x.join);
+        cudaStreamDestroy(x.stream);
+    }
+    if (e->fork) cudaEventDestroy(e->fork);
     if (e->own_stream && e->stream) cudaStreamDestroy(e->stream);
     delete e;
     return PA_OK;
@@ -1528,7 +1599,7 @@ pa_status pa_calibrate_philox(uint32_t wide, uint32_t reps, void *cuda_stream, d
 static cudaError_t copy_out(void *host, const void *dev, size_t bytes, cudaStream_t s)
 {
     volatile char *p = static_cast<volatile char *>(host);
-    if (bytes >= (64u << 10))
+    if (bytes >= (1u << 20))
         for (size_t o = 0; o < bytes; o += 4096) p[o] = 0;
     if (bytes) p[bytes - 1] = 0;
     return cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, s);
