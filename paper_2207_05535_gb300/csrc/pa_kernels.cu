@@ -3900,6 +3900,7 @@ static int small_fit(uint32_t L, int any_glass, const SmallShape &sh)
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t cfg = small_launch_config(1, sh, 0, at);
     int fit = 0;
+    if (sh.cs > 8) cudaFuncSetAttribute(small_kernel(L, any_glass, sh.variant), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (cudaOccupancyMaxActiveClusters(&fit, small_kernel(L, any_glass, sh.variant), &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         fit = 0;
@@ -4017,13 +4018,6 @@ cudaError_t prepare_kernels()
                                                            (int)SMALL_PRE_BYTES);
                 if (e != cudaSuccess) return e;
             }
-    for (uint32_t L : {8u, 16u, 32u})
-        for (int sg = 0; sg < 2; ++sg)
-            for (uint32_t v = 0; v <= (L == 32 ? 2u : 4u); ++v) {
-                const cudaError_t e =
-                    cudaFuncSetAttribute(small_kernel(L, sg, v), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-                if (e != cudaSuccess) return e;
-            }
     cudaError_t e = cudaFuncSetAttribute(sweep_kernel<false, 1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          200 * 1024);
     if (e == cudaSuccess)
@@ -4031,23 +4025,6 @@ cudaError_t prepare_kernels()
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(resample_multinomial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  multinomial_smem(RESAMPLE_STAGE_MAX, MULTI_LEVELS));
-    for (void *k : {(void *)sweep_pow2_kernel<true, 1024, 2, 2, false, true, 512, 1>,
-                    (void *)sweep_pow2_kernel<true, 1024, 2, 2, false, false, 512, 1>,
-                    (void *)sweep_pow2_kernel<false, 1024, 2, 2, false, true, 512, 1>,
-                    (void *)sweep_pow2_kernel<false, 1024, 2, 2, false, false, 512, 1>,
-                    (void *)sweep_pow2_kernel<true, 16, 1, 2, true, true, 256, 2>,
-                    (void *)sweep_pow2_kernel<true, 16, 1, 2, true, false, 256, 2>,
-                    (void *)sweep_pow2_kernel<false, 16, 1, 2, true, true, 256, 2>,
-                    (void *)sweep_pow2_kernel<false, 16, 1, 2, true, false, 256, 2>})  // 144 and 52 KB
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-    for (void *k : {(void *)sweep_compact_kernel<true, 1024, 1, false, 1>,
-                    (void *)sweep_compact_kernel<false, 1024, 1, false, 1>,
-                    (void *)sweep_compact_kernel<true, 256, 3, true, 2>, (void *)sweep_compact_kernel<false, 256, 3, true, 2>,
-                    (void *)sweep_compact_kernel<true, 256, 3, false, 2>, (void *)sweep_compact_kernel<false, 256, 3, false, 2>,
-                    (void *)sweep_compact_kernel<true, 512, 2, true, 2>, (void *)sweep_compact_kernel<false, 512, 2, true, 2>,
-                    (void *)sweep_compact_kernel<true, 512, 2, false, 2>, (void *)sweep_compact_kernel<false, 512, 2, false, 2>})
-        if (e == cudaSuccess)  // geometry and bond masks of up to 1009 words, child parts of up to 512
-            e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 112 * 1024);
     if (e == cudaSuccess)  // Wang pairing with R_cap up to 8192: 144 KB
         e = cudaFuncSetAttribute(wang_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     return e;
@@ -4124,6 +4101,14 @@ SweepCfg sweep_fast_config(uint32_t L, uint32_t WPT, uint32_t NR, uint32_t block
     return c;
 }
 
+// Kernels of a lattice size whose shapes take more than 48 KB of dynamic shared memory.
+static void allow_smem(std::initializer_list<void *> kernels, uint32_t bytes)
+{
+    for (void *k : kernels)
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+            (void)cudaGetLastError();  // the launch reports it
+}
+
 std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
 {
     std::vector<SweepCfg> v;
@@ -4138,6 +4123,10 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
             v.push_back(sweep_fast_config(L, 1, 1, 256, TH));  // L = 8, 16: 1902, 1868
             v.push_back(sweep_fast_config(L, 1, 1, 128, TH));  // 1901, 1868
         } else if (L == 32) {  // a table of 16 KB; two children without it: 1850
+            allow_smem({(void *)sweep_pow2_kernel<true, 16, 1, 2, true, true, 256, 2>,
+                        (void *)sweep_pow2_kernel<true, 16, 1, 2, true, false, 256, 2>,
+                        (void *)sweep_pow2_kernel<false, 16, 1, 2, true, true, 256, 2>,
+                        (void *)sweep_pow2_kernel<false, 16, 1, 2, true, false, 256, 2>}, 64 * 1024);
             v.push_back(sweep_fast_config(L, 1, 2, 256, 8));  // 1875
             v.push_back(sweep_fast_config(L, 1, 1, 128, 8));  // 1794
         } else if (L == 64) {  // a table of two half-sweeps: 1616; four children: 1825
@@ -4147,6 +4136,10 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
             v.push_back(sweep_fast_config(L, 1, 2, 256, 0));  // 1854
             v.push_back(sweep_fast_config(L, 1, 1, 256, 0));  // 1789
         } else {  // L = 256: 4 words of one child by 256 threads: 1664
+            allow_smem({(void *)sweep_pow2_kernel<true, 1024, 2, 2, false, true, 512, 1>,
+                        (void *)sweep_pow2_kernel<true, 1024, 2, 2, false, false, 512, 1>,
+                        (void *)sweep_pow2_kernel<false, 1024, 2, 2, false, true, 512, 1>,
+                        (void *)sweep_pow2_kernel<false, 1024, 2, 2, false, false, 512, 1>}, 160 * 1024);
             v.push_back(sweep_fast_config(L, 2, 2, 512, 0));   // 1781
             v.push_back(sweep_fast_config(L, 1, 1, 1024, 0));  // 1648
         }
@@ -4186,6 +4179,19 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
         // Updates/ns (40 runs, 4e8 spins, theta = 10) of 256 threads with one child each, 256 and 512
         // with two: L = 6 816, 356, 347; L = 10 1170, 1083, 1039; L = 30 1415, 1488, 1404; L = 46 1374,
         // 1451, 1468; L = 100 1305, 1374, 1380.
+        if (CW > 256)  // geometry and bond masks of up to 1009 words
+            allow_smem({(void *)sweep_compact_kernel<true, 1024, 1, false, 1>,
+                        (void *)sweep_compact_kernel<false, 1024, 1, false, 1>}, 112 * 1024);
+        else if (Lh < 32)  // two children per thread: child parts
+            allow_smem({(void *)sweep_compact_kernel<true, 256, 3, true, 2>,
+                        (void *)sweep_compact_kernel<false, 256, 3, true, 2>,
+                        (void *)sweep_compact_kernel<true, 512, 2, true, 2>,
+                        (void *)sweep_compact_kernel<false, 512, 2, true, 2>}, 112 * 1024);
+        else
+            allow_smem({(void *)sweep_compact_kernel<true, 256, 3, false, 2>,
+                        (void *)sweep_compact_kernel<false, 256, 3, false, 2>,
+                        (void *)sweep_compact_kernel<true, 512, 2, false, 2>,
+                        (void *)sweep_compact_kernel<false, 512, 2, false, 2>}, 112 * 1024);
         if (CW <= 4) {
             shape(256, 1);
             shape(256, 2);
