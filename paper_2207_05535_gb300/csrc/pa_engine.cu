@@ -1012,7 +1012,7 @@ void enqueue_resample(pa_engine *e)
             launch_resample_nearest(e->P, meta(e, e->near_off), (uint32_t)e->near_runs.size(), e->near_maxcap,
                                     e->stream);
         });
-        e->launches += resample_nearest_launches(e->near_maxcap) - 1;
+        e->launches += resample_nearest_launches((uint32_t)e->near_runs.size(), e->near_maxcap) - 1;
     }
     if (!e->multi_runs.empty())
         timed_launch(e, PA_K_RESAMPLE, [&] {

@@ -28,6 +28,7 @@
 //                        per-CTA family statistics
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 #include <vector>
 
@@ -79,6 +80,22 @@ __host__ __device__ inline uint32_t run_ctas(uint32_t R_cap)
 {
     const uint32_t c = (R_cap + CTA_REPLICAS - 1) / CTA_REPLICAS;
     return c < 1 ? 1 : (c > MAX_RUN_CTAS ? MAX_RUN_CTAS : c);
+}
+
+// CTAs per run, for the largest of a launch's n_runs populations, of the nearest-integer
+// resampling and the measurement: run_ctas, or more where the launch leaves SMs idle.  A CTA takes
+// about 7 us and 1 us per 1000 replicas, and splitting a population 4 us for the second resampling
+// launch; with two CTAs per SM, 304 run at once.  The split is taken where that predicts a gain of 15 %.
+// One run of R = 16000: resampling 24.0 -> 16.9 us, measurement 23.8 -> 19.7; of R = 64000: 32.1 ->
+// 16.6, 28.1 -> 22.4; 48 of R = 50000: 43.8 -> 34.8, 38.1 -> 32.0.  A launch that fills the GPU
+// gains nothing: 200 runs of R = 20000 take 44 and 43 us with 2 CTAs each, 45 and 43 with 3.
+inline uint32_t split_ctas(uint32_t n_runs, uint32_t max_Rcap)
+{
+    const uint32_t least = run_ctas(max_Rcap);
+    if (max_Rcap <= 4096 || n_runs == 0) return least;
+    auto us = [&](uint32_t nc) { return 7.0 + 1e-3 * max_Rcap / nc + (nc > 1 ? 4.0 : 0.0); };
+    const uint32_t most = (uint32_t)std::min<uint64_t>({304 / n_runs, MAX_RUN_CTAS, (max_Rcap + 2047ull) / 2048});
+    return most > least && us(most) < 0.85 * us(least) ? most : least;
 }
 
 struct Pool {
@@ -193,10 +210,14 @@ void launch_init_population(const Pool &P, const uint32_t *tile_off, const uint3
 void launch_resample_multinomial(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap,
                                  uint32_t max_N, cudaStream_t s);
 // Nearest-integer resampling (PA_NEAREST) from the tables the measurement of
-// the previous step prepared, run_ctas(R_cap) CTAs per run, in
-// resample_nearest_launches(max_Rcap) kernel launches (one when every
-// population fits one CTA).
+// the previous step prepared, split_ctas CTAs per run, in
+// resample_nearest_launches(n_runs, max_Rcap) kernel launches (one when every
+// population takes one CTA).
 inline uint32_t resample_nearest_launches(uint32_t max_Rcap) { return run_ctas(max_Rcap) == 1 ? 1u : 2u; }
+inline uint32_t resample_nearest_launches(uint32_t n_runs, uint32_t max_Rcap)
+{
+    return split_ctas(n_runs, max_Rcap) == 1 ? 1u : 2u;
+}
 void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap, cudaStream_t s);
 // Launch shapes to try for lattice size L (first = default); one entry unless
 // the bit-sliced kernel applies.
@@ -205,7 +226,7 @@ void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *til
                   uint32_t n_tiles, const SweepCfg &cfg, int any_glass, uint32_t theta_max, cudaStream_t s);
 void launch_overlap(const Pool &P, const uint32_t *q_runs, uint32_t n_q_runs, uint32_t max_Rcap, int init,
                     cudaStream_t s);
-// run_ctas(R_cap) CTAs per run (at most run_ctas(max_Rcap)); also prepares the
+// split_ctas CTAs per run (fewer for the smaller populations); also prepares the
 // next nearest-integer resampling of each run.
 void launch_measure(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t max_Rcap, uint32_t max_N, int init,
                     cudaStream_t s);

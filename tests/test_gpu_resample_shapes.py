@@ -65,3 +65,11 @@ def test_wang_large_families(R):
     b = np.array([0.0, 0.3, 0.9, 1.2, 1.4])
     _against_oracle([W.RunDesc(8, W.EA_PMJ, R, 1, b, seed=7, run_id=k, disorder_id=k, overlap=W.Q_WANG)
                      for k in range(6)])
+
+
+# one or a few large populations, split over more CTAs than many of them would be, with a
+# population too small to split beside them
+@pytest.mark.parametrize("sizes", [[4096], [4097], [9001], [20000, 3], [40000, 17000, 60]])
+def test_split_populations(sizes):
+    b = W.schedule(0.6, 4)
+    _against_oracle([W.RunDesc(6, W.EA_PMJ if k else W.FERRO, R, 1, b, seed=8, run_id=k) for k, R in enumerate(sizes)])
