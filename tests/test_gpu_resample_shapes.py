@@ -73,3 +73,33 @@ def test_wang_large_families(R):
 def test_split_populations(sizes):
     b = W.schedule(0.6, 4)
     _against_oracle([W.RunDesc(6, W.EA_PMJ if k else W.FERRO, R, 1, b, seed=8, run_id=k) for k, R in enumerate(sizes)])
+
+
+# weighted overlap distributions: more runs than a CTA stages at once, histograms that end inside a
+# piece, runs without pairs at some steps; 1e-12 relative, as every weighted average
+@pytest.mark.parametrize("M,L", [(1, 8), (7, 12), (256, 8), (300, 10), (513, 4)])
+def test_weighted_overlap_distributions(M, L):
+    rng = np.random.default_rng(M)
+    N, n = L * L, 5
+    rec = np.zeros((M, n), dtype=_lib.RECORD_DTYPE)
+    rec["beta"] = np.linspace(0.0, 0.4, n)
+    rec["lnQ"] = rng.normal(0.3, 0.05, (M, n))
+    rec["minus_betaF"] = N * np.log(2.0) + np.cumsum(rec["lnQ"], axis=1)
+    rec["R"], rec["R_target"], rec["N"] = rng.integers(40, 60, (M, n)), 50, N
+    R = rec["R"].astype(np.int64)
+    rec["sumE"], rec["sumE2"], rec["sumAbsM"], rec["sumM2"] = -20 * R, 500 * R, 6 * R, 60 * R
+    for f, v in (("sumE3", 9000), ("sumE4", 400000), ("sumAbsM3", 700), ("sumM4", 9000)):
+        rec[f][..., 0] = v * R
+    rec["n_q"] = rng.integers(0, 30, (M, n))
+    rec["n_q_pair"] = rng.integers(0, 2, (M, n)) * 25
+    rec["n_q_wang"] = rec["R"]
+    qs = [rng.integers(0, 1000, (M, n, N + 1)).astype(np.uint32) for _ in range(3)]
+    for q, f in zip(qs, ("n_q", "n_q_pair", "n_q_wang")):
+        q[rec[f] == 0] = 0
+    g = _lib.pa_weighted_average(rec, N, 0, qs[0], qs[1], qh_wang=qs[2])
+    one = _lib.pa_weighted_average(rec, N, 0, None, qs[1])
+    o = O.weighted_average(rec, N, 0, qs[0], qs[1], qh_wang=qs[2])
+    for a, b in zip(g[1:], o[1:]):
+        assert np.allclose(a, b, rtol=1e-12, atol=0)
+    assert one[1] is None and np.array_equal(one[2], g[2])
+    assert np.allclose(g[0]["W_minus_betaF"], o[0]["W_minus_betaF"], rtol=1e-12, atol=0)
