@@ -175,8 +175,8 @@ pa_status pa_create(const pa_run_desc *runs, uint32_t n_runs, void *cuda_stream,
 /* pa_create with options (bit flags):
  *   PA_CREATE_GENERIC_SWEEP keeps every lattice size on the general byte-plane
  *     sweep kernel instead of the bit-sliced kernels (rows tiling 32-bit words
- *     when L/2 is a power of two, otherwise rows repacked without padding or
- *     padded rows, whichever the autotuner finds faster); all give identical
+ *     when L/2 is a power of two, otherwise rows repacked without padding;
+ *     padded rows at L = 12, where they are faster); all give identical
  *     results, and the option exists to check that;
  *   PA_CREATE_NO_AUTOTUNE skips timing the bit-sliced kernels' launch shapes on
  *     the first anneal steps and uses the default shape;

@@ -159,7 +159,8 @@ inline uint32_t plane_words_of(uint32_t L) { return (L * row_pitch(L) + 31) / 32
 // (N + 1), then a tail used by one kernel at a time: the multinomial member
 // list (R_cap u32), or the per-CTA replica totals of the resampling
 // (MAX_RUN_CTAS u32), or the measurement's per-CTA family statistics
-// (MEASURE_PART_WORDS each).
+// (MEASURE_PART_WORDS each; a CTA of split_ctas' splits has more than 1365
+// replicas, whose member words are far more than its statistics).
 constexpr uint64_t MEASURE_PART_WORDS = 4;
 __host__ __device__ inline uint64_t scr_hist_words(uint32_t N) { return (uint64_t(N) + 2) / 2; }
 __host__ __device__ inline uint64_t scr_mhist_off(uint32_t N) { return scr_hist_words(N); }
@@ -212,7 +213,7 @@ void launch_resample_multinomial(const Pool &P, const uint32_t *runs, uint32_t n
 // Nearest-integer resampling (PA_NEAREST) from the tables the measurement of
 // the previous step prepared, split_ctas CTAs per run, in
 // resample_nearest_launches(n_runs, max_Rcap) kernel launches (one when every
-// population takes one CTA).
+// population takes one CTA).  Of a full launch: resample_nearest_launches(max_Rcap).
 inline uint32_t resample_nearest_launches(uint32_t max_Rcap) { return run_ctas(max_Rcap) == 1 ? 1u : 2u; }
 inline uint32_t resample_nearest_launches(uint32_t n_runs, uint32_t max_Rcap)
 {
