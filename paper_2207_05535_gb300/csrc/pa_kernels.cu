@@ -2248,11 +2248,12 @@ __global__ void __launch_bounds__(256) overlap_kernel(Pool P, const uint32_t *q_
 // Independent pairings from permutations (Sec. III.D, Wang et al., with the
 // random search pattern sigma).  One CTA per run, everything in shared memory:
 //   1. pi and sigma: replica indices in ascending order of per-replica 64-bit
-//      Philox keys whose low 13 bits are replaced by the index (bitonic sort);
+//      Philox keys whose low 13 bits are replaced by the index (counting sort);
 //   2. warp 0 visits positions k = sigma_0, sigma_1, ...; where replica k and
 //      pi_k share a family it tests the positions sigma_{i+1}, sigma_{i+2}, ...
 //      (mod R) 32 at a time with a ballot and swaps pi_k with the first pi_p
-//      outside k's family whose position p is outside pi_k's family.  A swap
+//      outside k's family whose position p is outside pi_k's family, the whole
+//      block searching on once a few rounds found none.  A swap
 //      fixes both positions and breaks no other, so one pass in sigma order
 //      equals the serial algorithm; a search that exhausts its R - 1 positions
 //      skips the measurement at this step;
@@ -2343,8 +2344,12 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
     // 32 positions at a time.  Once a family nears R / 2 a search goes through most of the
     // permutation, and there are up to R / 2 of them; so after WARP_TRIES
     // rounds the block's 32 warps take the rest at once, the smallest l found being the one the warp
-    // would have reached.  The warps meet at barrier 1 only, twice per search.
-    auto meet = [&] { asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory"); };
+    // would have reached.  The warps meet at barrier 1 only, twice per search; bar.sync wants a
+    // warp's lanes together, and they leave a search at different times.
+    auto meet = [&] {
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
+    };
     auto block_search = [&] {
         const uint32_t i0 = s_i0, fk = s_fk, fpk = s_fpk;
         for (uint32_t l = s_l0 + tid; l < R; l += nt) {
@@ -2406,7 +2411,6 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
                         s_fpk = fpk;
                         s_found = 0xFFFFFFFFu;
                     }
-                    __syncwarp();
                     meet();
                     block_search();
                     meet();
@@ -2435,7 +2439,6 @@ __global__ void __launch_bounds__(1024) wang_kernel(Pool P, const uint32_t *runs
             s_swaps = swaps;
             s_l0 = 0;
         }
-        __syncwarp();
         meet();
     }
     __syncthreads();
