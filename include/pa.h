@@ -400,6 +400,21 @@ uint64_t pa_launch_count(const pa_engine *e);
 pa_status pa_sweep_shape(const pa_engine *e, uint32_t group, uint32_t *L, uint32_t *words_per_thread,
                          uint32_t *block, uint32_t *tuned);
 
+/* Which of the lattice size's launch shapes that is: its number among the
+ * candidates (the same for every engine), how many there are, the children
+ * each thread sweeps, and the consecutive tiles of replicas one CTA works
+ * through at the group's present runs. */
+pa_status pa_sweep_candidate(const pa_engine *e, uint32_t group, uint32_t *candidate, uint32_t *n_candidates,
+                             uint32_t *children_per_thread, uint32_t *tiles_per_cta);
+
+/* Fix the launch shape of lattice size L in this engine to one of its
+ * candidates, in place of timing them (PA_SWEEP_SHAPE_AUTO: back to the
+ * engine's own choice), from the next anneal step on: to compare the shapes,
+ * whose results are identical.  PA_ERR_INVALID_ARG for an L out of range or a
+ * candidate that L does not have. */
+#define PA_SWEEP_SHAPE_AUTO 0xFFFFFFFFu
+pa_status pa_set_sweep_shape(pa_engine *e, uint32_t L, uint32_t candidate);
+
 /* Number of lattice sizes whose sweep launch shape is still being chosen: the
  * first anneal steps after a size appears run each candidate shape on the
  * step's real sweep (one warm-up step, then two steps per candidate, timed)

@@ -64,7 +64,8 @@ EXPORTS = ["pa_create", "pa_create_ex", "pa_pool_sizes", "pa_server_create", "pa
            "pa_checkpoint", "pa_restore",
            "pa_weighted_average_runs", "pa_weighted_average", "pa_weighted_average_noalloc", "pa_launch_count", "pa_set_profiling",
            "pa_step_records", "pa_set_allocator", "pa_tuning_pending",
-           "pa_kernel_times", "pa_transfer_bytes", "pa_calibrate_philox", "pa_sweep_shape", "pa_destroy", "pa_status_string"]
+           "pa_kernel_times", "pa_transfer_bytes", "pa_calibrate_philox", "pa_sweep_shape", "pa_sweep_candidate",
+           "pa_set_sweep_shape", "pa_destroy", "pa_status_string"]
 KERNEL_KINDS = ["resample", "sweep", "overlap", "measure", "init", "wavg", "small"]
 
 # pa_alloc_fn / pa_free_fn (include/pa.h)
@@ -115,6 +116,8 @@ def load(path: str = LIB_PATH):
         lib.pa_launch_count.argtypes = [vp]
         lib.pa_launch_count.restype = C.c_uint64
         lib.pa_sweep_shape.argtypes = [vp, u32, P(u32), P(u32), P(u32), P(u32)]
+        lib.pa_sweep_candidate.argtypes = [vp, u32, P(u32), P(u32), P(u32), P(u32)]
+        lib.pa_set_sweep_shape.argtypes = [vp, u32, u32]
         lib.pa_set_profiling.argtypes = [vp, C.c_int]
         lib.pa_kernel_times.argtypes = [vp, P(C.c_double), P(C.c_uint64)]
         lib.pa_transfer_bytes.argtypes = [vp, P(C.c_uint64), P(C.c_uint64)]
@@ -378,6 +381,23 @@ def pa_sweep_shapes(h):
             return out
         out.append(tuple(int(x.value) for x in v))
         g += 1
+
+
+def pa_sweep_candidates(h):
+    """[(candidate, number of candidates, children per thread, tiles per CTA)], groups as in pa_sweep_shapes."""
+    out, lib = [], load()
+    while True:
+        v = [C.c_uint32() for _ in range(4)]
+        if lib.pa_sweep_candidate(h, len(out), *[C.byref(x) for x in v]) != PA_OK:
+            return out
+        out.append(tuple(int(x.value) for x in v))
+
+
+PA_SWEEP_SHAPE_AUTO = 0xFFFFFFFF
+
+
+def pa_set_sweep_shape(h, L, candidate=PA_SWEEP_SHAPE_AUTO):
+    _check(load().pa_set_sweep_shape(h, L, candidate), "pa_set_sweep_shape")
 
 
 def pa_set_profiling(h, on=True):

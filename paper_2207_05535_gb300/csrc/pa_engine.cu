@@ -244,6 +244,7 @@ struct pa_engine {
     std::vector<uint32_t> big;         // the other resident runs (per-stage kernels)
     uint64_t big_off = 0;
     std::map<uint32_t, Tuning> tuning;  // per lattice size
+    std::map<uint32_t, uint32_t> fixed_shape;  // pa_set_sweep_shape: lattice size -> candidate
     struct Side {
         cudaStream_t stream;
         cudaEvent_t join;
@@ -908,6 +909,19 @@ void timed_launch(pa_engine *e, int kind, F &&launch)
 
 const uint32_t *meta(pa_engine *e, uint64_t off) { return e->d_meta + off; }
 
+// The launch shape of a group's sweeps: fixed by the caller, or the tuner's; shape_chosen is false
+// while the tuner is still timing.
+uint32_t shape_of(const pa_engine *e, const SweepGroup &g)
+{
+    auto it = e->fixed_shape.find(g.L);
+    return it != e->fixed_shape.end() ? it->second : e->tuning.at(g.L).pick;
+}
+
+bool shape_chosen(const pa_engine *e, const SweepGroup &g)
+{
+    return e->fixed_shape.count(g.L) || e->tuning.at(g.L).tuned;
+}
+
 void launch_group_sweep(pa_engine *e, const SweepGroup &g, uint32_t c, cudaStream_t s)
 {
     const Tuning &t = e->tuning[g.L];
@@ -925,7 +939,7 @@ void enqueue_sweeps(pa_engine *e)
     const size_t n_side = e->profiling || e->groups.size() < 2 ? 0 : std::min(e->groups.size() - 1, e->side.size());
     if (n_side == 0) {
         for (auto &g : e->groups)
-            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, e->tuning[g.L].pick, e->stream); });
+            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, shape_of(e, g), e->stream); });
         return;
     }
     cudaEventRecord(e->fork, e->stream);
@@ -933,7 +947,7 @@ void enqueue_sweeps(pa_engine *e)
     size_t at = 0;
     for (uint32_t gi : e->sweep_order) {
         const SweepGroup &g = e->groups[gi];
-        launch_group_sweep(e, g, e->tuning[g.L].pick, at == 0 ? e->stream : e->side[at - 1].stream);
+        launch_group_sweep(e, g, shape_of(e, g), at == 0 ? e->stream : e->side[at - 1].stream);
         at = at == n_side ? 0 : at + 1;
     }
     e->launches += e->groups.size();
@@ -1080,8 +1094,8 @@ pa_status enqueue_tuning_tick(pa_engine *e)
     std::vector<Timing> timing;
     for (auto &g : e->groups) {
         Tuning &t = e->tuning[g.L];
-        if (t.tuned) {
-            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, t.pick, e->stream); });
+        if (shape_chosen(e, g)) {
+            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, shape_of(e, g), e->stream); });
             continue;
         }
         bool live = false;  // a run of this size still has a temperature to go
@@ -1459,7 +1473,7 @@ pa_status pa_anneal_step(pa_engine *e, uint32_t n_steps, int use_graph)
     if (n_steps == 0 || e->active.empty()) return PA_OK;
     for (;;) {  // eager tuning steps while a lattice size's sweep shape is not chosen yet
         bool untuned = false;
-        for (auto &g : e->groups) untuned |= !e->tuning[g.L].tuned;
+        for (auto &g : e->groups) untuned |= !shape_chosen(e, g);
         if (!untuned) break;
         PA_TRY(enqueue_tuning_tick(e));
         advance_host_steps(e, 1);
@@ -1506,7 +1520,7 @@ pa_status pa_tuning_pending(const pa_engine *e, uint32_t *n)
 {
     if (!e || !n) return PA_ERR_INVALID_ARG;
     uint32_t k = 0;
-    for (const auto &g : e->groups) k += e->tuning.at(g.L).tuned ? 0u : 1u;
+    for (const auto &g : e->groups) k += shape_chosen(e, g) ? 0u : 1u;
     *n = k;
     return PA_OK;
 }
@@ -1517,11 +1531,40 @@ pa_status pa_sweep_shape(const pa_engine *e, uint32_t group, uint32_t *L, uint32
     if (!e || group >= e->groups.size() || !L || !words_per_thread || !block || !tuned) return PA_ERR_INVALID_ARG;
     const SweepGroup &g = e->groups[group];
     const Tuning &t = e->tuning.at(g.L);
-    const SweepCfg &c = t.candidates[t.pick];
+    const SweepCfg &c = t.candidates[shape_of(e, g)];
     *L = g.L;
     *words_per_thread = c.fast ? c.WPT : 0;
     *block = c.block;
-    *tuned = (t.tuned && t.candidates.size() > 1) ? 1u : 0u;
+    *tuned = (t.tuned && t.candidates.size() > 1 && !e->fixed_shape.count(g.L)) ? 1u : 0u;
+    return PA_OK;
+}
+
+pa_status pa_sweep_candidate(const pa_engine *e, uint32_t group, uint32_t *candidate, uint32_t *n_candidates,
+                             uint32_t *children_per_thread, uint32_t *tiles_per_cta)
+{
+    if (!e || group >= e->groups.size() || !candidate || !n_candidates || !children_per_thread || !tiles_per_cta)
+        return PA_ERR_INVALID_ARG;
+    const SweepGroup &g = e->groups[group];
+    const Tuning &t = e->tuning.at(g.L);
+    const uint32_t c = shape_of(e, g);
+    *candidate = c;
+    *n_candidates = (uint32_t)t.candidates.size();
+    *children_per_thread = std::max(t.candidates[c].NR, 1u);
+    *tiles_per_cta = sweep_tiles_per_cta(t.candidates[c], g.n_tiles[c], g.theta_max);
+    return PA_OK;
+}
+
+pa_status pa_set_sweep_shape(pa_engine *e, uint32_t L, uint32_t candidate)
+{
+    if (!e || L < 4 || L > 256 || (L & 1u)) return PA_ERR_INVALID_ARG;
+    if (candidate == PA_SWEEP_SHAPE_AUTO) {
+        e->fixed_shape.erase(L);
+    } else {
+        if (candidate >= sweep_candidates(L, (e->flags & PA_CREATE_GENERIC_SWEEP) ? 0 : 1).size())
+            return PA_ERR_INVALID_ARG;
+        e->fixed_shape[L] = candidate;
+    }
+    e->dirty = true;  // a captured step holds the shape it was captured with
     return PA_OK;
 }
 

@@ -223,6 +223,8 @@ void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_run
 // Launch shapes to try for lattice size L (first = default); one entry unless
 // the bit-sliced kernel applies.
 std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast);
+// Consecutive tiles one CTA of launch_sweep works through.
+uint32_t sweep_tiles_per_cta(const SweepCfg &cfg, uint32_t n_tiles, uint32_t theta_max);
 void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *tile_off, uint32_t n_group_runs,
                   uint32_t n_tiles, const SweepCfg &cfg, int any_glass, uint32_t theta_max, cudaStream_t s);
 void launch_overlap(const Pool &P, const uint32_t *q_runs, uint32_t n_q_runs, uint32_t max_Rcap, int init,

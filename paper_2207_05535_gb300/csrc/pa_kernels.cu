@@ -4279,20 +4279,27 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
     return v;
 }
 
+// With few sweeps per launch, finding the run, its thresholds, keys and table are a third of a tile's
+// time, and one CTA pays them once for K tiles (theta = 1, 40 runs of 1.6e6 replicas in all: L = 16
+// 1077 -> 1219 updates/ns, L = 64 1042 -> 1342, L = 256 1358 -> 1441).  At theta = 10 they are 3 %
+// and the loop over tiles costs the power-of-two kernel as much in registers (L = 16: 1877 one tile,
+// 1818 four), so it is compiled both ways and theta > 4 takes one tile.  K leaves at least 4 (compact
+// rows: 16) CTAs per SM slot, for a last wave that is short beside the launch.
+static bool sweep_many(const SweepCfg &cfg, uint32_t theta_max) { return cfg.fast == 1 && theta_max <= 4; }
+
+uint32_t sweep_tiles_per_cta(const SweepCfg &cfg, uint32_t n_tiles, uint32_t theta_max)
+{
+    if (sweep_many(cfg, theta_max)) return std::min(8u, std::max(1u, n_tiles / (152 * 4 * 4)));
+    if (cfg.fast == 3) return std::min(4u, std::max(1u, n_tiles / (152 * 2 * 16)));
+    return 1;
+}
+
 void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *tile_off, uint32_t n_group_runs,
                   uint32_t n_tiles, const SweepCfg &shape, int any_glass, uint32_t theta_max, cudaStream_t s)
 {
     SweepCfg cfg = shape;
-    // Consecutive tiles per CTA.  With few sweeps per launch, finding the run, its thresholds, keys
-    // and table are a third of a tile's time, and one CTA pays them once for K tiles (theta = 1,
-    // 40 runs of 1.6e6 replicas in all: L = 16 1077 -> 1219 updates/ns, L = 64 1042 -> 1342, L = 256
-    // 1358 -> 1441).  At theta = 10 they are 3 % and the loop over tiles costs the power-of-two
-    // kernel as much in registers (L = 16: 1877 one tile, 1818 four), so it is compiled both ways
-    // and theta > 4 takes one tile.  K leaves at least 4 (compact rows: 16) CTAs per SM slot, for
-    // a last wave that is short beside the launch.
-    const bool many = cfg.fast == 1 && theta_max <= 4;
-    if (many) cfg.K = std::min(8u, std::max(1u, n_tiles / (152 * 4 * 4)));
-    if (cfg.fast == 3) cfg.K = std::min(4u, std::max(1u, n_tiles / (152 * 2 * 16)));
+    const bool many = sweep_many(cfg, theta_max);
+    cfg.K = sweep_tiles_per_cta(cfg, n_tiles, theta_max);
     const dim3 grid((n_tiles + cfg.K - 1) / cfg.K);
 #define PA_SWEEP_FAST_(SG, HW, WPT, NR, TAB, MANY, MAXT, MINB)                                                        \
     sweep_pow2_kernel<SG, HW, WPT, NR, TAB, MANY, MAXT, MINB><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, \
