@@ -699,6 +699,12 @@ constexpr uint32_t FEW_REPLICAS = 1024;
 constexpr uint32_t COUNTS_SMEM_LEVELS = 2048;  // level tables staged in shared memory (L <= 45)
 constexpr uint32_t COUNTS_BATCH = 4;           // replicas per thread in flight
 constexpr uint32_t PARENT_BATCH = 8;           // rows of 32 copy numbers a warp loads at once
+// A replica with more copies than this has its row's children written by the whole warp: written by
+// its own lane, a step that leaves few families is a chain of one store after another, and three times
+// slower again in the split kernel than fused (L = 32, dbeta = 0.08, the first steps of a quench: one run of
+// R = 9000 48 us in one CTA, 104 split, 19 now; 20 of R = 24000 600 -> 48).  At dbeta = 0.01 few rows
+// have one: 16.7 -> 15.4 us for either split population.
+constexpr uint32_t PARENT_OWN_COPIES = 8;
 
 struct RunChunk {
     uint32_t lo, hi;  // this CTA's replicas
@@ -769,10 +775,23 @@ __device__ __forceinline__ void parents_pass(const Pool &P, uint32_t run, const 
                 const uint32_t y = __shfl_up_sync(FULL, x, o);
                 if ((int)lane >= o) x += y;
             }
-            const uint32_t o = carry + x - r;
-            for (uint32_t c = 0; c < r; ++c)
-                if (o + c < rd.R_cap) parent[o + c] = j;
-            carry += __shfl_sync(FULL, x, 31);
+            const uint32_t all = __shfl_sync(FULL, x, 31);
+            if (__any_sync(FULL, r > PARENT_OWN_COPIES)) {
+                // 32 children at a time, each lane finding its parent among the row's scan
+                const uint32_t n = carry < rd.R_cap ? min(all, rd.R_cap - carry) : 0u;
+                for (uint32_t k0 = 0; k0 < n; k0 += 32) {
+                    const uint32_t k = k0 + lane;
+                    uint32_t src = 0;  // replicas of the row whose copies end at or before child k
+#pragma unroll
+                    for (uint32_t step = 16; step; step >>= 1)
+                        if (__shfl_sync(FULL, x, src + step - 1) <= k) src += step;
+                    if (k < n) parent[carry + k] = b0 + 32 * q + src;
+                }
+            } else {
+                const uint32_t o = carry + x - r, n = o < rd.R_cap ? min(r, rd.R_cap - o) : 0u;
+                for (uint32_t c = 0; c < n; ++c) parent[o + c] = j;
+            }
+            carry += all;
         }
     }
     if (first_cta && tid == 0) {
