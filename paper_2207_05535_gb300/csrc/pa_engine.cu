@@ -253,7 +253,11 @@ struct pa_engine {
     cudaEvent_t fork = nullptr;
     bool side_failed = false;
     std::vector<uint32_t> sweep_order;  // indices of `groups`, most spins to update first
-    uint32_t max_Rcap_active = 0, max_N_active = 0, max_pw = 1;
+    uint32_t max_Rcap_active = 0, max_pw = 1;
+    struct Largest {  // of the runs of a launch
+        uint32_t Rcap = 0, N = 0;
+    } big_max, init_max;
+    uint32_t multi_maxN = 0;
     // execution
     uint64_t launches = 0;
     cudaGraph_t graph = nullptr;
@@ -734,22 +738,23 @@ pa_status rebuild(pa_engine *e)
     m.insert(m.end(), e->big.begin(), e->big.end());
     e->q_runs.clear();
     e->max_Rcap_active = 0;
-    e->max_N_active = 0;
     for (uint32_t s : e->active) {
         if (e->rd[s].overlap) e->q_runs.push_back(s);  // small runs have none
         e->max_Rcap_active = std::max(e->max_Rcap_active, e->rd[s].R_cap);
-        e->max_N_active = std::max(e->max_N_active, e->rd[s].N);
     }
     e->q_off = m.size();
     m.insert(m.end(), e->q_runs.begin(), e->q_runs.end());
     e->near_runs.clear();
     e->multi_runs.clear();
-    e->near_maxcap = e->multi_maxcap = 0;
+    e->near_maxcap = e->multi_maxcap = e->multi_maxN = 0;
+    e->big_max = {};
     for (uint32_t s : e->big) {
         const bool multi = e->rd[s].resample == PA_MULTINOMIAL;
         (multi ? e->multi_runs : e->near_runs).push_back(s);
         uint32_t &cap = multi ? e->multi_maxcap : e->near_maxcap;
         cap = std::max(cap, e->rd[s].R_cap);
+        if (multi) e->multi_maxN = std::max(e->multi_maxN, e->rd[s].N);
+        e->big_max = {std::max(e->big_max.Rcap, e->rd[s].R_cap), std::max(e->big_max.N, e->rd[s].N)};
     }
     e->near_off = m.size();
     m.insert(m.end(), e->near_runs.begin(), e->near_runs.end());
@@ -830,7 +835,9 @@ pa_status rebuild(pa_engine *e)
     e->init_tiles_off = m.size();
     uint64_t acc = 0;
     m.push_back(0u);
+    e->init_max = {};
     for (uint32_t s : e->pending) {  // 4 replicas per CTA; none for theta = PA_THETA_INF runs
+        e->init_max = {std::max(e->init_max.Rcap, e->rd[s].R_cap), std::max(e->init_max.N, e->rd[s].N)};
         acc += e->rd[s].theta == PA_THETA_INF ? 0u : (e->rd[s].R + 3) / 4;
         if (acc > 0x7fffffffull) return PA_ERR_INVALID_ARG;
         m.push_back((uint32_t)acc);
@@ -1000,7 +1007,7 @@ pa_status enqueue_pending(pa_engine *e)
             launch_wang(e->P, meta(e, e->init_wang_off), e->init_wang_n, e->init_wang_maxcap, 1, e->stream);
         });
     timed_launch(e, PA_K_MEASURE,
-                 [&] { launch_measure(e->P, runs, e->init_n, e->max_Rcap_active, e->max_N_active, 1, e->stream); });
+                 [&] { launch_measure(e->P, runs, e->init_n, e->init_max.Rcap, e->init_max.N, 1, e->stream); });
     e->pending.clear();
     e->dirty = true;  // the pending list is consumed
     PA_CUDA(cudaGetLastError());
@@ -1031,7 +1038,7 @@ void enqueue_resample(pa_engine *e)
     if (!e->multi_runs.empty())
         timed_launch(e, PA_K_RESAMPLE, [&] {
             launch_resample_multinomial(e->P, meta(e, e->multi_off), (uint32_t)e->multi_runs.size(),
-                                        e->multi_maxcap, e->max_N_active, e->stream);
+                                        e->multi_maxcap, e->multi_maxN, e->stream);
         });
 }
 
@@ -1069,7 +1076,7 @@ void enqueue_tick(pa_engine *e)
             launch_overlap(e->P, meta(e, e->q_off), (uint32_t)e->q_runs.size(), e->max_Rcap_active, 0, e->stream);
         });
     enqueue_wang(e);
-    timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->max_Rcap_active, e->max_N_active, 0, e->stream); });
+    timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->big_max.Rcap, e->big_max.N, 0, e->stream); });
 }
 
 // One eager step of tuning.  A lattice size whose sweep shape is not chosen yet
@@ -1121,7 +1128,7 @@ pa_status enqueue_tuning_tick(pa_engine *e)
             launch_overlap(e->P, meta(e, e->q_off), (uint32_t)e->q_runs.size(), e->max_Rcap_active, 0, e->stream);
         });
     enqueue_wang(e);
-    if (na) timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->max_Rcap_active, e->max_N_active, 0, e->stream); });
+    if (na) timed_launch(e, PA_K_MEASURE, [&] { launch_measure(e->P, act, na, e->big_max.Rcap, e->big_max.N, 0, e->stream); });
     PA_CUDA(cudaGetLastError());
     if (timing.empty()) return PA_OK;
     PA_CUDA(cudaStreamSynchronize(e->stream));

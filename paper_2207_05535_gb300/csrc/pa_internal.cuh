@@ -98,6 +98,26 @@ inline uint32_t split_ctas(uint32_t n_runs, uint32_t max_Rcap)
     return most > least && us(most) < 0.85 * us(least) ? most : least;
 }
 
+// Threads per CTA of the measurement and of the nearest-integer resampling, for the largest
+// population and lattice of a launch.  A run of few replicas is a chain of dependent steps that more
+// threads do not shorten, and with 128 threads eight runs share an SM instead of two: 2048 runs of R = 100, L = 16:
+// measurement 89 -> 37 us a step, resampling 36 -> 15 us.  But the measurement also clears, adds
+// and scans N + 1 levels, which 512 threads do faster until their CTAs, two per SM, no longer run at
+// once.  Measurement with 128 against 512 threads, R = 50 to 150: L = 20 14.9 / 15.2 us (152 runs),
+// L = 32 17.7 / 17.0 (100), 18.4 / 19.6 (200), L = 64 30.9 / 21.7 (152), 33.8 / 26.0 (304), 35.4 / 41.9
+// (400), L = 128 98 / 50 (304), 107 / 120 (700), L = 256 342 / 135 (304), 349 / 239 (400).  Resampling,
+// which scans only the occupied levels: R = 100 8.2 / 8.6, R = 700 10.4 / 9.4 (one run), 12.4 / 15.2 (400).
+constexpr uint32_t FEW_REPLICAS = 1024;  // capacity: R of about 740
+inline uint32_t measure_threads(uint32_t n_runs, uint32_t max_Rcap, uint32_t max_N)
+{
+    const uint32_t at_once = max_N <= 400 ? 0u : max_N <= 1024 ? 152u : max_N <= 4096 ? 304u : max_N <= 16384 ? 608u : ~0u;
+    return max_Rcap <= FEW_REPLICAS && n_runs > at_once ? 128u : 512u;
+}
+inline uint32_t resample_threads(uint32_t n_runs, uint32_t max_Rcap)
+{
+    return max_Rcap <= FEW_REPLICAS / 2 || (max_Rcap <= FEW_REPLICAS && n_runs > 152) ? 128u : 512u;
+}
+
 struct Pool {
     const RunDev *runs;
     RunState *st;

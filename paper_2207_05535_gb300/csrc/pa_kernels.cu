@@ -690,12 +690,7 @@ __global__ void __launch_bounds__(MULTI_THREADS) resample_multinomial_kernel(Poo
 //   resample_counts_kernel   r_j of every replica and each CTA's total
 //   resample_parents_kernel  offsets (earlier CTAs' totals plus a scan inside
 //                            the CTA) and the parent map
-constexpr uint32_t RESAMPLE_THREADS = 512;
-// Launches whose populations all have at most this many replicas resample and measure with 128
-// threads per run: a run's time is a chain of dependent steps that more threads do not shorten,
-// and four times the runs share an SM (2048 runs of R = 100, L = 16: measurement
-// 89 -> 37 us a step, resampling 36 -> 15 us).
-constexpr uint32_t FEW_REPLICAS = 1024;
+constexpr uint32_t RESAMPLE_THREADS = 512;  // the largest of resample_threads
 constexpr uint32_t COUNTS_SMEM_LEVELS = 2048;  // level tables staged in shared memory (L <= 45)
 constexpr uint32_t COUNTS_BATCH = 4;           // replicas per thread in flight
 constexpr uint32_t PARENT_BATCH = 8;           // rows of 32 copy numbers a warp loads at once
@@ -2746,7 +2741,7 @@ struct Moments {
 // level floor(tau) and the draw threshold ceil(frac 2^32).  It leaves the
 // histograms cleared.
 #ifndef PA_MEASURE_THREADS
-#define PA_MEASURE_THREADS 512
+#define PA_MEASURE_THREADS 512  // the largest of measure_threads
 #endif
 #ifndef PA_MEASURE_MIN_BLOCKS
 #define PA_MEASURE_MIN_BLOCKS 2  // two CTAs per SM: at most 64 registers
@@ -4125,8 +4120,7 @@ void launch_resample_nearest(const Pool &P, const uint32_t *runs, uint32_t n_run
     const dim3 grid(n_runs, split_ctas(n_runs, max_Rcap));
     const uint32_t per_cta = (max_Rcap + grid.y - 1) / grid.y;
     if (grid.y == 1) {  // every population in one CTA: one launch
-        resample_counts_kernel<true>
-            <<<grid, max_Rcap <= FEW_REPLICAS ? 128 : RESAMPLE_THREADS, 0, s>>>(P, runs, per_cta);
+        resample_counts_kernel<true><<<grid, resample_threads(n_runs, max_Rcap), 0, s>>>(P, runs, per_cta);
         return;
     }
     resample_counts_kernel<false><<<grid, RESAMPLE_THREADS, 0, s>>>(P, runs, per_cta);
@@ -4392,7 +4386,7 @@ void launch_measure(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32
 {
     if (n_runs == 0) return;
     const uint32_t bins = std::min(max_N + 1, MEASURE_SMEM_BINS);
-    const uint32_t threads = max_Rcap <= FEW_REPLICAS ? 128 : PA_MEASURE_THREADS;
+    const uint32_t threads = measure_threads(n_runs, max_Rcap, max_N);
     const uint32_t nc = split_ctas(n_runs, max_Rcap), per_cta = (max_Rcap + nc - 1) / nc;
     measure_kernel<<<dim3(n_runs, nc), threads, 2 * bins * sizeof(uint32_t), s>>>(P, runs, init, bins, per_cta);
 }

@@ -1,0 +1,49 @@
+"""The rules that choose launch shapes, compiled from the engine's header: what
+they pick on both sides of their lines, and that the scratch they imply exists."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2207_05535_gb300 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA_INCLUDE = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build.nvcc()))), "include")
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    """Evaluate an expression of pa_internal.cuh for each tuple of arguments."""
+    tmp = tmp_path_factory.mktemp("rules")
+
+    def run(expr, names, rows):
+        src, exe = tmp / "r.cpp", tmp / "r"
+        args = ", ".join(f"unsigned {n}" for n in names)
+        calls = "".join(f"  f({', '.join(str(v) + 'u' for v in r)});\n" for r in rows)
+        src.write_text(f"""#include <cstdio>
+#include <cuda_runtime.h>
+#include "pa_internal.cuh"
+static void f({args}) {{ std::printf("%llu\\n", (unsigned long long)({expr})); }}
+int main() {{
+{calls}  return 0;
+}}
+""")
+        subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I",
+                        os.path.join(ROOT, "paper_2207_05535_gb300", "csrc"), "-I", CUDA_INCLUDE, str(src), "-o",
+                        str(exe)], check=True)
+        out = subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.split()
+        return [int(v) for v in out]
+
+    return run
+
+
+def test_few_threads_only_where_the_levels_allow(rule):
+    """128 threads per run scan a large lattice's levels slower than 512, while those fit the GPU at once."""
+    rows = {(1, 100, 64): 128, (1, 1024, 256): 128, (1, 1025, 256): 512, (100, 300, 1024): 512, (153, 300, 1024): 128,
+            (1, 300, 4096): 512, (304, 300, 4096): 512, (305, 300, 4096): 128, (304, 300, 16384): 512,
+            (609, 300, 16384): 128, (100000, 300, 65536): 512}
+    got = rule("pa::measure_threads(n, cap, N)", ("n", "cap", "N"), list(rows))
+    assert got == list(rows.values())
+    rows = {(1, 244): 128, (1, 512): 128, (1, 972): 512, (152, 972): 512, (153, 972): 128, (2048, 1025): 512}
+    got = rule("pa::resample_threads(n, cap)", ("n", "cap"), list(rows))
+    assert got == list(rows.values())
