@@ -179,7 +179,7 @@ pa_status pa_create(const pa_run_desc *runs, uint32_t n_runs, void *cuda_stream,
  *     padded rows at L = 12, where they are faster); all give identical
  *     results, and the option exists to check that;
  *   PA_CREATE_NO_AUTOTUNE skips timing the bit-sliced kernels' launch shapes on
- *     the first anneal steps and uses the default shape;
+ *     the first anneal steps and uses the default shape of the load;
  *   PA_CREATE_SEPARATE_KERNELS keeps small runs on the per-stage kernels.
  * Without it, a small run (L = 8, 16 or 32, nearest-integer resampling, no
  * overlaps, R_cap <= 8192) is annealed by one launch per step when its lattice
@@ -193,8 +193,10 @@ pa_status pa_create(const pa_run_desc *runs, uint32_t n_runs, void *cuda_stream,
  * per-stage kernels.
  * Without it, the first anneal steps of a lattice size time every candidate shape
  * on the steps' real sweeps (pa_tuning_pending) and keep the fastest; the
- * choice is shared with every later engine of the process on the same device,
- * which then skips the timing for that size.
+ * choice holds for the lattice size, for how far its resident runs fill the
+ * GPU (three classes) and for schedules of few or many sweeps (theta <= 4 for
+ * all of them, or not), and is shared with every later engine of the process
+ * on the same device, which then skips the timing for these.
  * Results never depend on the launch shape. */
 enum { PA_CREATE_GENERIC_SWEEP = 1, PA_CREATE_NO_AUTOTUNE = 2, PA_CREATE_SEPARATE_KERNELS = 4 };
 pa_status pa_create_ex(const pa_run_desc *runs, uint32_t n_runs, void *cuda_stream, uint32_t flags,
@@ -416,7 +418,8 @@ pa_status pa_sweep_candidate(const pa_engine *e, uint32_t group, uint32_t *candi
 pa_status pa_set_sweep_shape(pa_engine *e, uint32_t L, uint32_t candidate);
 
 /* Number of lattice sizes whose sweep launch shape is still being chosen: the
- * first anneal steps after a size appears run each candidate shape on the
+ * first anneal steps after a size appears, or its resident runs fill the GPU
+ * to another degree than any timed before, run each candidate shape on the
  * step's real sweep (one warm-up step, then two steps per candidate, timed)
  * eagerly, before graph replay takes over.  Host bookkeeping; no
  * synchronisation. */

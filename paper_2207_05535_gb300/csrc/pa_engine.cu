@@ -84,26 +84,35 @@ struct FreeList {
     }
 };
 
+// What the fastest launch shape of a sweep depends on: lattice size, how far its runs fill the GPU,
+// and few sweeps per launch or many.  The couplings do not change the order (L = 16, 30 and 64 timed
+// at every load).
+struct ShapeKey {
+    uint32_t L = 0;
+    SweepLoad load = LOAD_FEW;
+    bool few = false;
+    bool operator<(const ShapeKey &o) const { return std::tie(L, load, few) < std::tie(o.L, o.load, o.few); }
+};
+
 struct Tuning {
-    std::vector<SweepCfg> candidates;
+    std::vector<uint32_t> tried;  // the lattice size's shapes that this load times
     uint32_t pick = 0;
     bool tuned = false;
-    float ms = 0.f;
     uint32_t round = 0;       // tuning steps taken so far
-    std::vector<float> best;  // per candidate: its fastest timed step (ms), 0 = not timed yet
+    std::vector<float> best;  // per shape tried: its fastest timed step (ms), 0 = not timed yet
 };
 
 // Launch shapes chosen by timing are shared by every engine of the process on the
-// same device: a new engine reuses the choice for a lattice size instead of timing
-// the candidates again.  Key: (device, L, bit-sliced kernels allowed).
+// same device: a new engine reuses the choice for a lattice size, load and kind of schedule
+// instead of timing the candidates again.  Key: (device, bit-sliced kernels allowed, ShapeKey).
 std::mutex g_tune_mu;
-std::map<std::tuple<int, uint32_t, int>, uint32_t> g_tuned;
+std::map<std::tuple<int, int, ShapeKey>, uint32_t> g_tuned;
 
-std::tuple<int, uint32_t, int> tune_key(uint32_t L, uint32_t flags)
+std::tuple<int, int, ShapeKey> tune_key(const ShapeKey &k, uint32_t flags)
 {
     int dev = 0;
     cudaGetDevice(&dev);
-    return std::make_tuple(dev, L, (flags & PA_CREATE_GENERIC_SWEEP) ? 0 : 1);
+    return std::make_tuple(dev, (flags & PA_CREATE_GENERIC_SWEEP) ? 0 : 1, k);
 }
 
 // Device allocator: cudaMalloc / cudaFree unless the caller installed callbacks
@@ -167,6 +176,7 @@ constexpr uint32_t SIDE_STREAMS = 3;  // beside the engine's own
 
 struct SweepGroup {  // runs of one lattice size among the resident runs
     uint32_t L = 0;
+    ShapeKey key;
     int any_glass = 0;
     uint32_t theta_max = 0;
     double updates = 0;  // per temperature
@@ -243,7 +253,8 @@ struct pa_engine {
     std::vector<SmallGroup> small;     // runs on the one-launch-per-step path
     std::vector<uint32_t> big;         // the other resident runs (per-stage kernels)
     uint64_t big_off = 0;
-    std::map<uint32_t, Tuning> tuning;  // per lattice size
+    std::map<uint32_t, std::vector<SweepCfg>> shapes;  // per lattice size: its candidates
+    std::map<ShapeKey, Tuning> tuning;
     std::map<uint32_t, uint32_t> fixed_shape;  // pa_set_sweep_shape: lattice size -> candidate
     struct Side {
         cudaStream_t stream;
@@ -685,6 +696,38 @@ pa_status admit(pa_engine *e, const pa_run_desc *runs, uint32_t n, uint32_t *slo
 
 void make_side_streams(pa_engine *e);
 
+// The candidate launch shapes of lattice size L.
+const std::vector<SweepCfg> &shapes_of(pa_engine *e, uint32_t L)
+{
+    auto it = e->shapes.find(L);
+    if (it == e->shapes.end())
+        it = e->shapes.emplace(L, sweep_candidates(L, (e->flags & PA_CREATE_GENERIC_SWEEP) ? 0 : 1)).first;
+    return it->second;
+}
+
+// The group's key, and its tuning state from an earlier resident set, an earlier engine, or new.
+void choose_shape(pa_engine *e, SweepGroup &g, const std::vector<SweepCfg> &shapes)
+{
+    uint64_t ctas = 0;
+    for (uint32_t s : g.runs) ctas += ((uint64_t)e->rd[s].R + shapes[0].RPC - 1) / shapes[0].RPC;
+    g.key = ShapeKey{g.L, sweep_load(ctas), few_sweeps(g.theta_max)};
+    if (e->tuning.count(g.key)) return;
+    Tuning t;
+    for (uint32_t c = 0; c < shapes.size(); ++c)
+        if (shapes[c].loads >> g.key.load & 1u) t.tried.push_back(c);
+    t.pick = default_shape(shapes, g.key.load);
+    t.tuned = t.tried.size() < 2 || (e->flags & PA_CREATE_NO_AUTOTUNE);
+    if (!t.tuned) {
+        std::lock_guard<std::mutex> lock(g_tune_mu);
+        auto c = g_tuned.find(tune_key(g.key, e->flags));
+        if (c != g_tuned.end() && c->second < shapes.size()) {
+            t.pick = c->second;
+            t.tuned = true;
+        }
+    }
+    e->tuning[g.key] = t;
+}
+
 // Rebuild the device lists (resident runs, overlap runs, per-size work lists,
 // the pending-draw list) after the resident set changed.
 pa_status rebuild(pa_engine *e)
@@ -786,20 +829,6 @@ pa_status rebuild(pa_engine *e)
             SweepGroup g;
             g.L = L;
             e->groups.push_back(g);
-            if (!e->tuning.count(L)) {
-                Tuning t;
-                t.candidates = sweep_candidates(L, (e->flags & PA_CREATE_GENERIC_SWEEP) ? 0 : 1);
-                t.tuned = t.candidates.size() < 2 || (e->flags & PA_CREATE_NO_AUTOTUNE);
-                if (!t.tuned) {
-                    std::lock_guard<std::mutex> lock(g_tune_mu);
-                    auto c = g_tuned.find(tune_key(L, e->flags));
-                    if (c != g_tuned.end() && c->second < t.candidates.size()) {
-                        t.pick = c->second;
-                        t.tuned = true;
-                    }
-                }
-                e->tuning[L] = t;
-            }
         }
         SweepGroup &g = e->groups[it->second];
         g.runs.push_back(s);
@@ -813,10 +842,11 @@ pa_status rebuild(pa_engine *e)
                      [&](uint32_t a, uint32_t b) { return e->groups[a].updates > e->groups[b].updates; });
     make_side_streams(e);
     for (auto &g : e->groups) {
-        const Tuning &t = e->tuning[g.L];
+        const std::vector<SweepCfg> &shapes = shapes_of(e, g.L);
+        choose_shape(e, g, shapes);
         g.runs_off = m.size();
         m.insert(m.end(), g.runs.begin(), g.runs.end());
-        for (const SweepCfg &c : t.candidates) {
+        for (const SweepCfg &c : shapes) {
             g.tile_map_off.push_back(m.size());
             uint64_t acc = 0;
             m.push_back(0u);
@@ -921,19 +951,18 @@ const uint32_t *meta(pa_engine *e, uint64_t off) { return e->d_meta + off; }
 uint32_t shape_of(const pa_engine *e, const SweepGroup &g)
 {
     auto it = e->fixed_shape.find(g.L);
-    return it != e->fixed_shape.end() ? it->second : e->tuning.at(g.L).pick;
+    return it != e->fixed_shape.end() ? it->second : e->tuning.at(g.key).pick;
 }
 
 bool shape_chosen(const pa_engine *e, const SweepGroup &g)
 {
-    return e->fixed_shape.count(g.L) || e->tuning.at(g.L).tuned;
+    return e->fixed_shape.count(g.L) || e->tuning.at(g.key).tuned;
 }
 
 void launch_group_sweep(pa_engine *e, const SweepGroup &g, uint32_t c, cudaStream_t s)
 {
-    const Tuning &t = e->tuning[g.L];
     launch_sweep(e->P, meta(e, g.runs_off), meta(e, g.tile_map_off[c]), (uint32_t)g.runs.size(), g.n_tiles[c],
-                 t.candidates[c], g.any_glass, g.theta_max, s);
+                 shapes_of(e, g.L)[c], g.any_glass, g.theta_max, s);
 }
 
 // The sweeps of every lattice size.  They touch different runs, and one size's launch is often
@@ -1095,12 +1124,11 @@ pa_status enqueue_tuning_tick(pa_engine *e)
     enqueue_resample(e);
     struct Timing {
         SweepGroup *g;
-        uint32_t c;
+        uint32_t q;  // index in the shapes tried
         cudaEvent_t a, b;
     };
     std::vector<Timing> timing;
     for (auto &g : e->groups) {
-        Tuning &t = e->tuning[g.L];
         if (shape_chosen(e, g)) {
             timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, shape_of(e, g), e->stream); });
             continue;
@@ -1108,16 +1136,16 @@ pa_status enqueue_tuning_tick(pa_engine *e)
         bool live = false;  // a run of this size still has a temperature to go
         for (uint32_t r : g.runs) live |= e->rh[r].steps_done + 1 < e->rh[r].d.n_beta;
         if (!live) {
-            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, t.pick, e->stream); });
+            timed_launch(e, PA_K_SWEEP, [&] { launch_group_sweep(e, g, shape_of(e, g), e->stream); });
             continue;
         }
-        const uint32_t nc = (uint32_t)t.candidates.size();
-        const uint32_t c = t.round == 0 ? 0u : (t.round - 1) % nc;
-        Timing x{&g, c, nullptr, nullptr};
+        const Tuning &t = e->tuning.at(g.key);
+        const uint32_t q = t.round == 0 ? 0u : (t.round - 1) % (uint32_t)t.tried.size();
+        Timing x{&g, q, nullptr, nullptr};
         PA_CUDA(cudaEventCreate(&x.a));
         PA_CUDA(cudaEventCreate(&x.b));
         PA_CUDA(cudaEventRecord(x.a, e->stream));
-        launch_group_sweep(e, g, c, e->stream);
+        launch_group_sweep(e, g, t.round == 0 ? t.pick : t.tried[q], e->stream);
         PA_CUDA(cudaEventRecord(x.b, e->stream));
         e->launches += 1;
         timing.push_back(x);
@@ -1133,23 +1161,23 @@ pa_status enqueue_tuning_tick(pa_engine *e)
     if (timing.empty()) return PA_OK;
     PA_CUDA(cudaStreamSynchronize(e->stream));
     for (auto &x : timing) {
-        Tuning &t = e->tuning[x.g->L];
-        const uint32_t nc = (uint32_t)t.candidates.size();
+        Tuning &t = e->tuning.at(x.g->key);
+        const uint32_t nc = (uint32_t)t.tried.size();
         float ms = 0.f;
         PA_CUDA(cudaEventElapsedTime(&ms, x.a, x.b));
         cudaEventDestroy(x.a);
         cudaEventDestroy(x.b);
         if (t.best.size() != nc) t.best.assign(nc, 0.f);
-        if (t.round > 0 && (t.best[x.c] == 0.f || ms < t.best[x.c])) t.best[x.c] = ms;
+        if (t.round > 0 && (t.best[x.q] == 0.f || ms < t.best[x.q])) t.best[x.q] = ms;
         t.round += 1;
         if (t.round == 1 + 2 * nc) {  // every candidate timed on two steps
-            t.pick = 0;
-            for (uint32_t c = 1; c < nc; ++c)
-                if (t.best[c] < t.best[t.pick]) t.pick = c;
+            uint32_t fastest = 0;
+            for (uint32_t q = 1; q < nc; ++q)
+                if (t.best[q] < t.best[fastest]) fastest = q;
+            t.pick = t.tried[fastest];
             t.tuned = true;
-            t.ms = t.best[t.pick];
             std::lock_guard<std::mutex> lock(g_tune_mu);
-            g_tuned[tune_key(x.g->L, e->flags)] = t.pick;
+            g_tuned[tune_key(x.g->key, e->flags)] = t.pick;
         }
     }
     return PA_OK;
@@ -1537,12 +1565,12 @@ pa_status pa_sweep_shape(const pa_engine *e, uint32_t group, uint32_t *L, uint32
 {
     if (!e || group >= e->groups.size() || !L || !words_per_thread || !block || !tuned) return PA_ERR_INVALID_ARG;
     const SweepGroup &g = e->groups[group];
-    const Tuning &t = e->tuning.at(g.L);
-    const SweepCfg &c = t.candidates[shape_of(e, g)];
+    const Tuning &t = e->tuning.at(g.key);
+    const SweepCfg &c = e->shapes.at(g.L)[shape_of(e, g)];
     *L = g.L;
     *words_per_thread = c.fast ? c.WPT : 0;
     *block = c.block;
-    *tuned = (t.tuned && t.candidates.size() > 1 && !e->fixed_shape.count(g.L)) ? 1u : 0u;
+    *tuned = (t.tuned && t.tried.size() > 1 && !e->fixed_shape.count(g.L)) ? 1u : 0u;
     return PA_OK;
 }
 
@@ -1552,12 +1580,12 @@ pa_status pa_sweep_candidate(const pa_engine *e, uint32_t group, uint32_t *candi
     if (!e || group >= e->groups.size() || !candidate || !n_candidates || !children_per_thread || !tiles_per_cta)
         return PA_ERR_INVALID_ARG;
     const SweepGroup &g = e->groups[group];
-    const Tuning &t = e->tuning.at(g.L);
+    const std::vector<SweepCfg> &shapes = e->shapes.at(g.L);
     const uint32_t c = shape_of(e, g);
     *candidate = c;
-    *n_candidates = (uint32_t)t.candidates.size();
-    *children_per_thread = std::max(t.candidates[c].NR, 1u);
-    *tiles_per_cta = sweep_tiles_per_cta(t.candidates[c], g.n_tiles[c], g.theta_max);
+    *n_candidates = (uint32_t)shapes.size();
+    *children_per_thread = std::max(shapes[c].NR, 1u);
+    *tiles_per_cta = sweep_tiles_per_cta(shapes[c], g.n_tiles[c], g.theta_max);
     return PA_OK;
 }
 
@@ -1567,7 +1595,7 @@ pa_status pa_set_sweep_shape(pa_engine *e, uint32_t L, uint32_t candidate)
     if (candidate == PA_SWEEP_SHAPE_AUTO) {
         e->fixed_shape.erase(L);
     } else {
-        if (candidate >= sweep_candidates(L, (e->flags & PA_CREATE_GENERIC_SWEEP) ? 0 : 1).size())
+        if (candidate >= shapes_of(e, L).size())
             return PA_ERR_INVALID_ARG;
         e->fixed_shape[L] = candidate;
     }

@@ -106,7 +106,7 @@ inline uint32_t split_ctas(uint32_t n_runs, uint32_t max_Rcap)
 // once.  Measurement with 128 against 512 threads, R = 50 to 150: L = 20 14.9 / 15.2 us (152 runs),
 // L = 32 17.7 / 17.0 (100), 18.4 / 19.6 (200), L = 64 30.9 / 21.7 (152), 33.8 / 26.0 (304), 35.4 / 41.9
 // (400), L = 128 98 / 50 (304), 107 / 120 (700), L = 256 342 / 135 (304), 349 / 239 (400).  Resampling,
-// which scans only the occupied levels: R = 100 8.2 / 8.6, R = 700 10.4 / 9.4 (one run), 12.4 / 15.2 (400).
+// which scans only the occupied levels: R = 100 8.2 / 8.5 (one run), 8.3 / 12.6 (400), R = 700 10.0 / 8.6, 11.3 / 14.6.
 constexpr uint32_t FEW_REPLICAS = 1024;  // capacity: R of about 740
 inline uint32_t measure_threads(uint32_t n_runs, uint32_t max_Rcap, uint32_t max_N)
 {
@@ -155,7 +155,29 @@ struct SweepCfg {
     uint32_t TH;     // half-sweeps of shared Philox parts held in shared memory (0: none)
     uint32_t K;      // consecutive tiles one CTA works through (set by launch_sweep)
     uint32_t Lh, pw; // compact rows: L/2 and words of a stored plane
+    uint32_t loads;  // the loads (bits 1 << SweepLoad) at which the tuner times it
 };
+
+// How far the sweeps of a lattice size fill the GPU, from the CTAs that its first launch shape takes: up
+// to two per SM, a few waves of them, or more.  Below two per SM a launch lasts as long as one CTA,
+// so one child per thread and small blocks win; from eight per SM on it is the throughput, two
+// children and large blocks; between them whole waves decide (theta = 10, us a launch, one / two children): L = 30
+// 100 CTAs 28 / 48, 190 59 / 74, 750 172 / 166, 1500 336 / 319; L = 64 200 28 / 33, 800 82 / 87, 1600 158 / 153,
+// 13000 1167 / 1124; L = 256 50 64 / 114, 200 181 / 223, 400 356 / 332, 1600 1290 / 1203.
+enum SweepLoad : uint32_t { LOAD_FEW = 0, LOAD_SOME = 1, LOAD_FULL = 2, LOAD_ANY = 7 /* mask */ };
+inline SweepLoad sweep_load(uint64_t ctas) { return ctas < 304 ? LOAD_FEW : ctas < 1216 ? LOAD_SOME : LOAD_FULL; }
+// Few sweeps per launch: kernels of their own for the power-of-two sizes (launch_sweep).
+inline bool few_sweeps(uint32_t theta_max) { return theta_max <= 4; }
+// The shape before (or without) timing: the first one, and of a load that leaves SMs idle the one
+// that spreads the replicas over the most CTAs.
+inline uint32_t default_shape(const std::vector<SweepCfg> &shapes, SweepLoad load)
+{
+    uint32_t pick = 0;
+    if (load == LOAD_FEW)
+        for (uint32_t c = 1; c < shapes.size(); ++c)
+            if (shapes[c].RPC < shapes[pick].RPC) pick = c;
+    return pick;
+}
 
 // Row pitch of a colour plane: L/2 when that is a power of two; else the
 // smallest power of two >= L/2 that makes L * pitch a multiple of 32 (rows then

@@ -4144,6 +4144,7 @@ SweepCfg sweep_fast_config(uint32_t L, uint32_t WPT, uint32_t NR, uint32_t block
     c.G = 8 * HW;
     c.PS = 0;
     c.TH = TH;
+    c.loads = LOAD_ANY;
     c.smem = TH * c.G * 16 + (WPT * NR > 1 ? c.RPC * c.G * 8 : 0) + c.RPC * 2 * HW * 4 + 8 * c.RPC;
     return c;
 }
@@ -4162,9 +4163,9 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
     const uint32_t N = L * L;
     const bool pow2 = L >= 8 && L <= 256 && (L & (L - 1)) == 0;
     if (pow2 && allow_fast) {
-        // Updates/ns of each shape (40 ferromagnet runs, 4e8 spins, theta = 10); the tuner picks.  The
-        // second one of L >= 32 takes one child per thread, for populations too small to fill the
-        // GPU with two.
+        // Updates/ns of each shape (40 ferromagnet runs, 4e8 spins, theta = 10); the tuner picks, for each
+        // load.  The second one of L >= 32 takes one child per thread, for populations too small to
+        // fill the GPU with two (SweepLoad).
         if (L <= 16) {  // tables of 5 and 10 KB; two children per thread: 1501, 1865
             const uint32_t TH = L == 8 ? 40 : 20;
             v.push_back(sweep_fast_config(L, 1, 1, 256, TH));  // L = 8, 16: 1902, 1868
@@ -4196,9 +4197,10 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
     if (allow_fast && CW <= 1024) {  // compact rows
         // The replicas of a CTA of at most `target` threads that leave the fewest lanes idle in
         // whole groups of four warps (one per SM sub-partition).
-        auto shape = [&](uint32_t target, uint32_t NR) {
+        auto shape = [&](uint32_t target, uint32_t NR, uint32_t loads = LOAD_ANY) {
             SweepCfg c{};
             c.K = 1;
+            c.loads = loads;
             c.fast = 3;
             c.WPT = 1;
             c.TPR = CW;
@@ -4225,7 +4227,9 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
         };
         // Updates/ns (40 runs, 4e8 spins, theta = 10) of 256 threads with one child each, 256 and 512
         // with two: L = 6 816, 356, 347; L = 10 1170, 1083, 1039; L = 30 1415, 1488, 1404; L = 46 1374,
-        // 1451, 1468; L = 100 1305, 1374, 1380.
+        // 1451, 1468; L = 100 1305, 1374, 1380.  128 threads with one child
+        // each are faster wherever SMs are idle (R = 100, theta = 10: L = 10, 30, 62 28 -> 22 us), and for planes of
+        // up to 4 words at every load (1.6e6 replicas: L = 6 749 -> 725 us).
         if (CW > 256)  // geometry and bond masks of up to 1009 words
             allow_smem({(void *)sweep_compact_kernel<true, 1024, 1, false, 1>,
                         (void *)sweep_compact_kernel<false, 1024, 1, false, 1>}, 112 * 1024);
@@ -4239,16 +4243,18 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
                         (void *)sweep_compact_kernel<false, 256, 3, false, 2>,
                         (void *)sweep_compact_kernel<true, 512, 2, false, 2>,
                         (void *)sweep_compact_kernel<false, 512, 2, false, 2>}, 112 * 1024);
+        constexpr uint32_t few = 1u << LOAD_FEW, more = LOAD_ANY & ~few;
         if (CW <= 4) {
             shape(256, 1);
-            shape(256, 2);
+            shape(256, 2, more);
         } else if (CW <= 256) {
             shape(256, 2);
-            shape(512, 2);
+            shape(512, 2, more);
             shape(256, 1);
         } else {
             shape(CW, 1);
         }
+        if (CW <= 128) shape(128, 1, CW <= 4 ? LOAD_ANY : few);
     }
     // Padded rows draw only the 6 Philox groups that a word of 4 rows holds at L = 12, where the
     // compact planes end in a word three quarters empty: 1218 against 1138 updates/ns there; at
@@ -4258,6 +4264,7 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
             SweepCfg c{};
             const uint32_t HW = L * Pt / 32;
             c.K = 1;
+            c.loads = LOAD_ANY;
             c.fast = 2;
             c.WPT = 1;
             c.TPR = HW;
@@ -4272,6 +4279,7 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
     if (!v.empty()) return v;
     SweepCfg c{};
     c.K = 1;
+    c.loads = LOAD_ANY;
     c.fast = 0;
     c.WPT = 1;
     c.G = (N + 7) / 8;
@@ -4298,7 +4306,7 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
 // and the loop over tiles costs the power-of-two kernel as much in registers (L = 16: 1877 one tile,
 // 1818 four), so it is compiled both ways and theta > 4 takes one tile.  K leaves at least 4 (compact
 // rows: 16) CTAs per SM slot, for a last wave that is short beside the launch.
-static bool sweep_many(const SweepCfg &cfg, uint32_t theta_max) { return cfg.fast == 1 && theta_max <= 4; }
+static bool sweep_many(const SweepCfg &cfg, uint32_t theta_max) { return cfg.fast == 1 && few_sweeps(theta_max); }
 
 uint32_t sweep_tiles_per_cta(const SweepCfg &cfg, uint32_t n_tiles, uint32_t theta_max)
 {
