@@ -221,6 +221,7 @@ inline uint64_t scratch_words(uint32_t N, uint32_t R_cap)
 // Small populations annealed by one launch per step (anneal_small_kernel): one
 // thread-block cluster per run, cluster size small_cluster().
 constexpr uint32_t SMALL_MAX_RCAP = 8192;
+constexpr uint32_t SMALL_MAX_CTAS = 16;  // largest cluster (above 8 by the non-portable opt-in)
 inline bool small_eligible(const RunDev &x)
 {
     return (x.L == 8 || x.L == 16 || x.L == 32) && x.theta != PA_THETA_INF && x.resample == PA_NEAREST &&
@@ -308,6 +309,30 @@ void launch_unpack_spins(const uint32_t *words, const RunDev &rd, uint32_t t0, u
 struct SmallShape {
     uint32_t cs, block, variant, H, smem;
 };
+// The largest clusters to try.  More than 8 CTAs (the non-portable sizes, at most one such cluster per GPC) shorten
+// the sweeps and lengthen the chain of cluster barriers, so they pay where the sweeps last longer.
+// One temperature per launch, 8 against 16 CTAs (us per temperature, theta = 10; threads that 8 CTAs
+// sweep with): L = 16 R = 400 (461) 34.6 / 28.1 for one run, 35.0 / 37.6 for nine; R = 500 (568) 42.8 / 31.7,
+// 43.7 / 36.6; R = 1000 (1095) 63.3 / 45.2, 66.5 / 66.6; L = 8 R = 400 20.5 / 20.3, 22.2 / 23.6; R = 500 24.5 / 21.0, 24.7 / 22.5.
+inline uint32_t small_largest_cluster(uint32_t L, uint32_t n_runs, uint32_t threads_of_8)
+{
+    return L != 32 && threads_of_8 > (n_runs <= 8 ? 384u : 512u) ? SMALL_MAX_CTAS : 8u;
+}
+// Several temperatures per launch, where the draws overlap CTA 0's measurement: the line is the sweeps' work
+// per thread, theta times the warps of a CTA of 8 times a thread's draws (a word of L = 8 is drawn by 4
+// lanes, one of L = 16 by one).  8 / 16 CTAs, one run, by theta: L = 16 R = 500 (352 threads) 12.2 / 13.3 at 3, 13.6 /
+// 13.4 at 4, 28.1 / 20.9 at 10; R = 700 (448) 12.3 / 13.2 at 2, 13.9 / 13.5 at 3, 35.5 / 21.2 at 10; L = 8 R = 500 12.3 / 13.1
+// at 10, 20.8 / 15.9 at 20; R = 700 12.6 / 13.2 at 8, 14.7 / 13.5 at 10.  Above 512 threads 16 CTAs at every theta
+// (L = 8 R = 1200 12.5 / 12.4 at 2, 23.8 / 14.2 at 10; L = 16 R = 1000 13.4 / 13.9, 44.7 / 28.2).  Eight or nine runs leave no
+// room for 16 CTAs each (L = 16, theta = 10: R = 500 28.0 / 29.4, R = 600 35.3 / 29.4), five do; up to 384 threads the
+// line is a little higher (L = 16 R = 300 at 5, 224 threads: 12.4 / 13.1).
+inline uint32_t small_largest_cluster_ahead(uint32_t L, uint32_t n_runs, uint32_t threads_of_8, uint32_t theta_max)
+{
+    const uint32_t block = (threads_of_8 + 31) / 32 * 32;
+    if (n_runs > 5 && threads_of_8 <= 384) return 8;
+    const uint32_t line = threads_of_8 <= 384 ? 5000 : 4300;
+    return block > 512 || (uint64_t)theta_max * block * (L * L / 64) > line ? SMALL_MAX_CTAS : 8u;
+}
 SmallShape small_shape(uint32_t L, int any_glass, uint32_t n_runs, uint32_t R_max, uint32_t R_cap_max);
 SmallShape small_shape_ahead(uint32_t L, int any_glass, uint32_t n_runs, uint32_t R_max, uint32_t theta_max);
 void launch_anneal_small(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t L, const SmallShape &sh,

@@ -3351,7 +3351,6 @@ __global__ void __launch_bounds__(WAVG_Q_THREADS)
 // path, so a run can move between the two paths at any step.
 // --------------------------------------------------------------------------
 constexpr uint32_t SMALL_MAX_N = 1024;  // L <= 32
-constexpr uint32_t SMALL_MAX_CTAS = 16;  // largest cluster (above 8 by the non-portable opt-in)
 
 // HW: words of a colour plane (L = 8: 1, 16: 4, 32: 16); LPW lanes per word; NT the
 // largest block (a multiple of 32, at least 128) and MINB the CTAs per SM it is
@@ -3963,13 +3962,6 @@ static uint32_t isqrt_u32(uint32_t R)
     return q;
 }
 
-// The largest cluster to try, from the threads that 8 CTAs would sweep with: more than 8 CTAs
-// (the non-portable sizes) pay where those are bound by their throughput, not by the chain of a
-// temperature's steps.  Per temperature, 8 against 16 CTAs: L = 16, R = 1000 (628 threads) 45.3
-// against 28.6 us; L = 16, R = 500 (324 threads) 28.8 against 29.7; L = 8, R = 500 (328) 12.7
-// against 13.4.
-static uint32_t small_largest_cluster(uint32_t threads_of_8) { return threads_of_8 > 384 ? SMALL_MAX_CTAS : 8u; }
-
 // Launch shapes of the small-run kernel for n runs of lattice size L.  A run's
 // steps are a chain of cluster barriers, so a run whose CTAs share SMs with
 // another run's is slower by the sharing, and the launch lasts as long as its
@@ -3984,7 +3976,7 @@ SmallShape small_shape(uint32_t L, int any_glass, uint32_t n_runs, uint32_t R_ma
     const uint32_t hw = L * L / 64;
     const uint32_t lpr = hw * (L == 8 ? SMALL_LPW_L8 : L == 16 ? SMALL_LPW_L16 : SMALL_LPW_L32);
     const uint32_t R_est = R_max + 3 * isqrt_u32(R_max) + 1;
-    for (uint32_t cs = L == 32 ? 8 : small_largest_cluster((R_est + 7) / 8 * lpr); cs >= 1; --cs) {
+    for (uint32_t cs = small_largest_cluster(L, n_runs, (R_est + 7) / 8 * lpr); cs >= 1; --cs) {
         if (cs > 1 && cs * n_runs > SMS) continue;  // cannot have an SM per CTA
         const uint32_t chunk = (R_est + cs - 1) / cs;
         uint32_t block = (chunk * lpr + 31) / 32 * 32;
@@ -4015,7 +4007,7 @@ SmallShape small_shape_ahead(uint32_t L, int any_glass, uint32_t n_runs, uint32_
     if ((L != 8 && L != 16) || theta_max == 0) return none;
     const uint32_t hw = L * L / 64, lpr4 = 4;
     const uint32_t R_est = R_max + 3 * isqrt_u32(R_max) + 1;
-    for (uint32_t cs = small_largest_cluster((R_est + 6) / 7 * lpr4); cs >= 2; --cs) {
+    for (uint32_t cs = small_largest_cluster_ahead(L, n_runs, (R_est + 6) / 7 * lpr4, theta_max); cs >= 2; --cs) {
         if (cs * n_runs > SMS) continue;
         const uint32_t Wc = (R_est + cs - 2) / (cs - 1);
         uint32_t block = (Wc * lpr4 + 31) / 32 * 32;

@@ -47,3 +47,15 @@ def test_few_threads_only_where_the_levels_allow(rule):
     rows = {(1, 244): 128, (1, 512): 128, (1, 972): 512, (152, 972): 512, (153, 972): 128, (2048, 1025): 512}
     got = rule("pa::resample_threads(n, cap)", ("n", "cap"), list(rows))
     assert got == list(rows.values())
+
+
+def test_clusters_grow_only_with_the_sweeps_work(rule):
+    """16 CTAs lengthen a temperature's chain: few sweeps stay on 8 (theta = 2, R = 700 12.3 us against 13.2)."""
+    names = ("L", "n", "t", "th")
+    # threads that 8 CTAs take for R = 300, 500, 700, 1000 at L = 16 and 8: 4 lanes per replica
+    rows = {(16, 1, 448, 2): 8, (16, 5, 448, 1): 8, (16, 1, 448, 3): 16, (16, 1, 352, 3): 8, (16, 1, 352, 4): 16,
+            (16, 8, 328, 10): 8, (16, 1, 204, 5): 8, (16, 1, 204, 10): 16, (16, 9, 388, 4): 16, (16, 1, 628, 1): 16, (8, 1, 328, 10): 8, (8, 1, 328, 20): 16,
+            (8, 1, 447, 8): 8, (8, 1, 447, 10): 16, (8, 20, 328, 10): 8, (16, 1, 0, 1 << 22): 8}
+    assert rule("pa::small_largest_cluster_ahead(L, n, t, th)", names, list(rows)) == list(rows.values())
+    rows = {(16, 1, 384): 8, (16, 1, 385): 16, (16, 9, 461): 8, (16, 9, 568): 16, (32, 1, 9999): 8}
+    assert rule("pa::small_largest_cluster(L, n, t)", names[:3], list(rows)) == list(rows.values())
