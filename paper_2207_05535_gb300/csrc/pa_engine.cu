@@ -170,6 +170,7 @@ struct SmallGroup {  // small runs of one lattice size, annealed by anneal_small
     uint32_t R_max = 0, R_cap_max = 0, theta_max = 0;
     SmallShape shape = {1, 512, 0, 0, 0};  // one temperature per launch
     SmallShape ahead = {0, 0, 0, 0, 0};     // several temperatures per launch (cs = 0: none)
+    bool several_only = false;              // single temperatures go per stage: its runs are among `big` too
 };
 
 constexpr uint32_t SIDE_STREAMS = 3;  // beside the engine's own
@@ -251,7 +252,8 @@ struct pa_engine {
     uint32_t inf_maxR = 0, init_inf_n = 0, init_inf_maxR = 0;
     std::vector<SweepGroup> groups;
     std::vector<SmallGroup> small;     // runs on the one-launch-per-step path
-    std::vector<uint32_t> big;         // the other resident runs (per-stage kernels)
+    std::vector<uint32_t> big;         // the runs on the per-stage kernels
+    bool all_small = false;            // every resident run is in `small`
     uint64_t big_off = 0;
     std::map<uint32_t, std::vector<SweepCfg>> shapes;  // per lattice size: its candidates
     std::map<ShapeKey, Tuning> tuning;
@@ -741,9 +743,11 @@ pa_status rebuild(pa_engine *e)
     e->small.clear();
     e->big.clear();
     const bool fuse = !(e->flags & (PA_CREATE_SEPARATE_KERNELS | PA_CREATE_GENERIC_SWEEP));
+    e->all_small = true;
     for (uint32_t s : e->active) {
         const RunDev &x = e->rd[s];
         if (!fuse || !small_eligible(x)) {
+            e->all_small = false;
             e->big.push_back(s);
             continue;
         }
@@ -769,10 +773,13 @@ pa_status rebuild(pa_engine *e)
         g.shape = small_shape(g.L, g.any_glass, (uint32_t)g.runs.size(), g.R_max, g.R_cap_max);
         g.ahead = small_shape_ahead(g.L, g.any_glass, (uint32_t)g.runs.size(), g.R_max, g.theta_max);
         if (g.shape.variant == 0 && g.ahead.cs == 0) {
+            e->all_small = false;
             e->big.insert(e->big.end(), g.runs.begin(), g.runs.end());
             e->small.erase(e->small.begin() + k);
             continue;
         }
+        g.several_only = g.shape.variant == 0 && small_steps_per_stage(g.L, g.R_max, g.theta_max);
+        if (g.several_only) e->big.insert(e->big.end(), g.runs.begin(), g.runs.end());
         g.runs_off = m.size();
         m.insert(m.end(), g.runs.begin(), g.runs.end());
         ++k;
@@ -1080,15 +1087,18 @@ void enqueue_dos_sample(pa_engine *e)
     });
 }
 
-// n_steps temperatures of every small run, one launch per lattice size.
+// n_steps temperatures of every small run, one launch per lattice size (of one temperature, the runs
+// that the per-stage kernels do not step).
 void enqueue_small(pa_engine *e, uint32_t n_steps)
 {
-    for (auto &g : e->small)
+    for (auto &g : e->small) {
+        if (n_steps == 1 && g.several_only) continue;
         timed_launch(e, PA_K_SMALL, [&] {
             launch_anneal_small(e->P, meta(e, g.runs_off), (uint32_t)g.runs.size(), g.L,
                                 n_steps > 1 && g.ahead.cs ? g.ahead : g.shape, g.any_glass,
                                 n_steps, e->stream);
         });
+    }
 }
 
 void enqueue_tick(pa_engine *e)
@@ -1506,6 +1516,13 @@ pa_status pa_anneal_step(pa_engine *e, uint32_t n_steps, int use_graph)
     for (uint32_t s : e->active) left = std::max(left, e->rh[s].d.n_beta - 1 - e->rh[s].steps_done);
     n_steps = std::min(n_steps, left);
     if (n_steps == 0 || e->active.empty()) return PA_OK;
+    // every run on the small path: n temperatures in one launch per lattice size
+    if (e->all_small && (n_steps > 1 || e->big.empty())) {
+        enqueue_small(e, n_steps);
+        PA_CUDA(cudaGetLastError());
+        advance_host_steps(e, n_steps);
+        return PA_OK;
+    }
     for (;;) {  // eager tuning steps while a lattice size's sweep shape is not chosen yet
         bool untuned = false;
         for (auto &g : e->groups) untuned |= !shape_chosen(e, g);
@@ -1513,12 +1530,6 @@ pa_status pa_anneal_step(pa_engine *e, uint32_t n_steps, int use_graph)
         PA_TRY(enqueue_tuning_tick(e));
         advance_host_steps(e, 1);
         if (--n_steps == 0) return PA_OK;
-    }
-    if (e->big.empty()) {  // every run on the small path: n temperatures in one launch per lattice size
-        enqueue_small(e, n_steps);
-        PA_CUDA(cudaGetLastError());
-        advance_host_steps(e, n_steps);
-        return PA_OK;
     }
     if (use_graph && !e->profiling) {
         if (!e->graph_exec) {

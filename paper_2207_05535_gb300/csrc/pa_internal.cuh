@@ -333,6 +333,14 @@ inline uint32_t small_largest_cluster_ahead(uint32_t L, uint32_t n_runs, uint32_
     const uint32_t line = threads_of_8 <= 384 ? 5000 : 4300;
     return block > 512 || (uint64_t)theta_max * block * (L * L / 64) > line ? SMALL_MAX_CTAS : 8u;
 }
+// A run whose populations fit a cluster only when several temperatures are drawn ahead takes a single
+// temperature per launch in several tiles per CTA, which the per-stage kernels beat from this work
+// on (us per temperature, cluster / per stage: L = 16 R = 1500 theta = 2 34.6 / 35.7, theta = 10 85.8 / 46; L = 8 R = 1500 24.4 /
+// 33.2, 43.0 / 40.5; R = 2000 27.9 / 34.2, 53.1 / 41.6).
+inline bool small_steps_per_stage(uint32_t L, uint32_t R_max, uint32_t theta_max)
+{
+    return (uint64_t)theta_max * R_max * L * L > 800000;
+}
 SmallShape small_shape(uint32_t L, int any_glass, uint32_t n_runs, uint32_t R_max, uint32_t R_cap_max);
 SmallShape small_shape_ahead(uint32_t L, int any_glass, uint32_t n_runs, uint32_t R_max, uint32_t theta_max);
 void launch_anneal_small(const Pool &P, const uint32_t *runs, uint32_t n_runs, uint32_t L, const SmallShape &sh,

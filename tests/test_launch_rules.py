@@ -59,3 +59,5 @@ def test_clusters_grow_only_with_the_sweeps_work(rule):
     assert rule("pa::small_largest_cluster_ahead(L, n, t, th)", names, list(rows)) == list(rows.values())
     rows = {(16, 1, 384): 8, (16, 1, 385): 16, (16, 9, 461): 8, (16, 9, 568): 16, (32, 1, 9999): 8}
     assert rule("pa::small_largest_cluster(L, n, t)", names[:3], list(rows)) == list(rows.values())
+    rows = {(16, 1500, 2): 0, (16, 1500, 10): 1, (8, 1500, 2): 0, (8, 1500, 10): 1, (8, 2000, 10): 1, (8, 2000, 1 << 22): 1}
+    assert rule("pa::small_steps_per_stage(L, R, th)", ("L", "R", "th"), list(rows)) == list(rows.values())
