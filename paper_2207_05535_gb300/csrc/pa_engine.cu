@@ -1742,6 +1742,11 @@ pa_status pa_measure(pa_engine *e, uint32_t run, uint32_t step, pa_step_record *
     return sync_read(e);
 }
 
+// Up to this many sites are unpacked on the host, without a launch and the clearing of its staging
+// buffer (us per call, device / host: one replica of L = 16 66 / 57; ten, 2560 sites, 69 / 65; one of L = 64,
+// 4096 sites, 69 / 81).
+static constexpr uint64_t FEW_SITES = 2560;
+
 pa_status pa_population_slice(pa_engine *e, uint32_t run, uint32_t first, uint32_t count, int8_t *host_spins,
                               int32_t *host_E, int32_t *host_M, uint32_t *host_fam, uint32_t *R_out,
                               uint32_t *step_out)
@@ -1756,8 +1761,14 @@ pa_status pa_population_slice(pa_engine *e, uint32_t run, uint32_t first, uint32
     if (R_out) *R_out = R;
     if (step_out) *step_out = st.step;
     const uint32_t lo = std::min(first, R), n = std::min<uint64_t>(count, (uint64_t)R - lo);
+    std::vector<uint32_t> words;  // of a few replicas, unpacked here
     if (host_spins && n && x.theta == PA_THETA_INF) {
         std::memset(host_spins, 0xFF, (size_t)n * x.N);  // not represented: -1 throughout
+    } else if (host_spins && n && (uint64_t)n * x.N <= FEW_SITES) {
+        words.resize((size_t)n * x.wstride);
+        PA_CUDA(cudaMemcpyAsync(words.data(), e->P.spins[b] + x.spin_off + (uint64_t)lo * x.wstride,
+                                sizeof(uint32_t) * words.size(), cudaMemcpyDeviceToHost, e->stream));
+        e->d2h += sizeof(uint32_t) * words.size();
     } else if (host_spins && n) {
         // Unpacked on the device (1000 replicas of L = 16: 0.81 ms with the unpacking on the host,
         // 0.16 ms now), through the run's other spin buffer: the next step's children overwrite it,
@@ -1785,7 +1796,15 @@ pa_status pa_population_slice(pa_engine *e, uint32_t run, uint32_t first, uint32
     if (host_fam && n)
         PA_CUDA(cudaMemcpyAsync(host_fam, e->P.fam[b] + x.rep_off + lo, sizeof(uint32_t) * n,
                                 cudaMemcpyDeviceToHost, e->stream));
-    return sync_read(e);
+    PA_TRY(sync_read(e));
+    if (!words.empty())
+        for (uint32_t j = 0; j < n; ++j)
+            for (uint32_t q = 0; q < x.N; ++q) {
+                const uint32_t xx = q % x.L, y = q / x.L, c = (xx + y) & 1u, pos = y * x.pitch + (xx >> 1);
+                const uint32_t word = words[(size_t)j * x.wstride + c * x.pw + (pos >> 5)];
+                host_spins[(size_t)j * x.N + q] = ((word >> (pos & 31)) & 1u) ? (int8_t)1 : (int8_t)-1;
+            }
+    return PA_OK;
 }
 
 pa_status pa_population(pa_engine *e, uint32_t run, int8_t *host_spins, int32_t *host_E, int32_t *host_M,
