@@ -167,7 +167,11 @@ pa_status pa_set_allocator(pa_alloc_fn alloc, pa_free_fn free_, void *ctx);
 /* Create an engine holding n_runs runs, allocate their device memory, draw the
  * beta_0 = 0 populations (Sec. II.B step (i): uniform states), the couplings
  * (Eq. H_SG) and measure step 0.  cuda_stream: a cudaStream_t to enqueue on,
- * or NULL for a private non-blocking stream.  *out receives the engine.
+ * or NULL for a private non-blocking stream.  An engine whose runs have several
+ * lattice sizes spreads their sweeps over up to three streams of its own beside
+ * it (pa_side_streams), of the same priority; events order them after what was
+ * on cuda_stream before and ahead of what follows on it.  *out receives the
+ * engine.
  * Errors: PA_ERR_INVALID_ARG (descriptor out of range; paired runs must share
  * L, model, disorder_id and n_beta), PA_ERR_OOM, PA_ERR_CUDA. */
 pa_status pa_create(const pa_run_desc *runs, uint32_t n_runs, void *cuda_stream, pa_engine **out);
@@ -428,6 +432,12 @@ pa_status pa_tuning_pending(const pa_engine *e, uint32_t *n);
 /* Kernel classes timed by the profiling mode. */
 enum { PA_K_RESAMPLE = 0, PA_K_SWEEP = 1, PA_K_OVERLAP = 2, PA_K_MEASURE = 3, PA_K_INIT = 4, PA_K_WAVG = 5,
        PA_K_SMALL = 6, PA_K_COUNT = 7 };  /* PA_K_SMALL: the one-launch-per-step path of small runs */
+
+/* The streams (cudaStream_t) the engine has beside its own, for the sweeps of
+ * several lattice sizes: up to cap of them in streams, *n = how many there are.
+ * They live as long as the engine; for inspection, nothing is to be enqueued on
+ * them. */
+pa_status pa_side_streams(const pa_engine *e, void **streams, uint32_t cap, uint32_t *n);
 
 /* Profiling mode: with on != 0 every kernel launch is bracketed by CUDA events
  * on the engine's stream and pa_anneal_step launches eagerly (no graph). */

@@ -65,7 +65,7 @@ EXPORTS = ["pa_create", "pa_create_ex", "pa_pool_sizes", "pa_server_create", "pa
            "pa_weighted_average_runs", "pa_weighted_average", "pa_weighted_average_noalloc", "pa_launch_count", "pa_set_profiling",
            "pa_step_records", "pa_set_allocator", "pa_tuning_pending",
            "pa_kernel_times", "pa_transfer_bytes", "pa_calibrate_philox", "pa_sweep_shape", "pa_sweep_candidate",
-           "pa_set_sweep_shape", "pa_destroy", "pa_status_string"]
+           "pa_set_sweep_shape", "pa_side_streams", "pa_destroy", "pa_status_string"]
 KERNEL_KINDS = ["resample", "sweep", "overlap", "measure", "init", "wavg", "small"]
 
 # pa_alloc_fn / pa_free_fn (include/pa.h)
@@ -118,6 +118,7 @@ def load(path: str = LIB_PATH):
         lib.pa_sweep_shape.argtypes = [vp, u32, P(u32), P(u32), P(u32), P(u32)]
         lib.pa_sweep_candidate.argtypes = [vp, u32, P(u32), P(u32), P(u32), P(u32)]
         lib.pa_set_sweep_shape.argtypes = [vp, u32, u32]
+        lib.pa_side_streams.argtypes = [vp, P(vp), u32, P(u32)]
         lib.pa_set_profiling.argtypes = [vp, C.c_int]
         lib.pa_kernel_times.argtypes = [vp, P(C.c_double), P(C.c_uint64)]
         lib.pa_transfer_bytes.argtypes = [vp, P(C.c_uint64), P(C.c_uint64)]
@@ -398,6 +399,15 @@ PA_SWEEP_SHAPE_AUTO = 0xFFFFFFFF
 
 def pa_set_sweep_shape(h, L, candidate=PA_SWEEP_SHAPE_AUTO):
     _check(load().pa_set_sweep_shape(h, L, candidate), "pa_set_sweep_shape")
+
+
+def pa_side_streams(h):
+    """Handles of the streams beside the engine's own."""
+    n = C.c_uint32()
+    _check(load().pa_side_streams(h, None, 0, C.byref(n)), "pa_side_streams")
+    buf = (C.c_void_p * max(n.value, 1))()
+    _check(load().pa_side_streams(h, buf, n.value, C.byref(n)), "pa_side_streams")
+    return [buf[k] for k in range(n.value)]
 
 
 def pa_set_profiling(h, on=True):

@@ -1000,15 +1000,18 @@ void enqueue_sweeps(pa_engine *e)
     }
 }
 
-// Side streams for engines with more than one lattice size, created while no capture is running;
-// without them (creation failed) the sweeps stay on the engine's stream.
+// Side streams for engines with more than one lattice size, at the priority of the engine's stream,
+// created while no capture is running; without them (creation failed) the sweeps stay on the engine's
+// stream.
 void make_side_streams(pa_engine *e)
 {
     if (e->groups.size() < 2 || !e->side.empty() || e->side_failed) return;
-    bool ok = cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming) == cudaSuccess;
+    int priority = 0;
+    bool ok = cudaStreamGetPriority(e->stream, &priority) == cudaSuccess &&
+              cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming) == cudaSuccess;
     for (uint32_t k = 0; ok && k < SIDE_STREAMS; ++k) {
         pa_engine::Side x{};
-        ok = cudaStreamCreateWithFlags(&x.stream, cudaStreamNonBlocking) == cudaSuccess;
+        ok = cudaStreamCreateWithPriority(&x.stream, cudaStreamNonBlocking, priority) == cudaSuccess;
         if (ok && cudaEventCreateWithFlags(&x.join, cudaEventDisableTiming) != cudaSuccess) {
             cudaStreamDestroy(x.stream);
             ok = false;
@@ -1611,6 +1614,14 @@ pa_status pa_set_sweep_shape(pa_engine *e, uint32_t L, uint32_t candidate)
         e->fixed_shape[L] = candidate;
     }
     e->dirty = true;  // a captured step holds the shape it was captured with
+    return PA_OK;
+}
+
+pa_status pa_side_streams(const pa_engine *e, void **streams, uint32_t cap, uint32_t *n)
+{
+    if (!e || !n || (cap && !streams)) return PA_ERR_INVALID_ARG;
+    for (uint32_t k = 0; k < cap && k < e->side.size(); ++k) streams[k] = e->side[k].stream;
+    *n = (uint32_t)e->side.size();
     return PA_OK;
 }
 
