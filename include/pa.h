@@ -13,6 +13,7 @@
  *  - Every call returns a pa_status; nothing else crosses the ABI on error.
  *  - Pointers named host_* or documented as "host" are host memory owned by
  *    the caller; the engine copies what it needs and keeps no reference.
+ *    Result buffers are writable and as large as stated, pageable or pinned.
  *  - The engine owns all device memory it allocates (from cudaMalloc, or from
  *    the allocator installed by pa_set_allocator) and frees it in
  *    pa_destroy.  Work is enqueued asynchronously on the engine's CUDA stream;

@@ -33,6 +33,7 @@
 #include <utility>
 #include <vector>
 
+#include "pa_copy_out.h"
 #include "pa_internal.cuh"
 
 using namespace pa;
@@ -1690,24 +1691,6 @@ pa_status pa_calibrate_philox(uint32_t wide, uint32_t reps, void *cuda_stream, d
     if (err) return cuda_fail(err, "pa_calibrate_philox");
     *calls_per_s = best;
     return PA_OK;
-}
-
-// Enqueues the copy of a result into the caller's memory, whose pages are first touched from the
-// host (they are overwritten anyway), while the device still works on the result.  A copy into
-// pages that have never been touched takes their faults one by one from the device: 20.8 MB into
-// fresh pages 17 ms, 0.8 ms with the touching (0.13 ms into pages in use).  Only pageable memory is
-// touched: pinned pages are there already, and a pointer that the host cannot write is left to
-// the copy to refuse.
-static cudaError_t copy_out(void *host, const void *dev, size_t bytes, cudaStream_t s)
-{
-    cudaPointerAttributes at{};
-    if (bytes >= (1u << 20) && cudaPointerGetAttributes(&at, host) == cudaSuccess &&
-        at.type == cudaMemoryTypeUnregistered) {
-        volatile char *p = static_cast<volatile char *>(host);
-        for (size_t o = 0; o < bytes; o += 4096) p[o] = 0;
-        p[bytes - 1] = 0;
-    }
-    return cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, s);
 }
 
 pa_status pa_records(pa_engine *e, uint32_t run, pa_step_record *host_out, uint32_t *host_qhist,
