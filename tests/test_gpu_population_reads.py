@@ -30,3 +30,48 @@ def test_slices_on_both_sides_of_the_line(L, n):
             assert R == len(s) and len(p) == got
             for a, b in ((p, s), (e, E), (m, M), (f, fam)):
                 assert np.array_equal(a, b[first:first + got])
+
+
+# Reads of the whole population go through the buffer that the next step's children take, in up to eight
+# pieces: the anneal goes on as if nothing had been read
+@pytest.mark.parametrize("flags", [SEPARATE, 0, 1])
+@pytest.mark.parametrize("L,R", [(6, 500), (8, 700), (16, 900), (30, 300), (64, 90), (128, 40)])
+def test_whole_reads_leave_the_anneal_alone(L, R, flags):
+    with _engine(L, R, flags) as eng, _engine(L, R, flags) as other:
+        for n in (1, 2, 1, 3):
+            eng.step(n)
+            other.step(n)
+            s, E, M, fam, _ = eng.population(0)
+            assert np.array_equal(s.sum(axis=1, dtype=np.int64), M)
+            cut = eng.checkpoint(0)
+            assert cut == other.checkpoint(0)
+        eng.run_to_end()
+        other.run_to_end()
+        assert np.array_equal(eng.records(0), other.records(0))
+        for a, b in zip(eng.population(0), other.population(0)):
+            assert np.array_equal(a, b)
+
+
+# results of 1 MB and more: into fresh pages, into pages that hold something, into pinned memory
+def test_large_results_into_pageable_and_pinned_memory():
+    import ctypes as C
+
+    import torch
+
+    L, R, temps = 32, 3000, 40
+    N = L * L
+    descs = [W.RunDesc(L, W.EA_PMJ, R, 1, W.schedule(0.8, temps), seed=37, run_id=k, disorder_id=0,
+                       overlap=W.Q_SHIFT | W.Q_PAIR, paired=1 - k) for k in range(2)]
+    with _lib.Engine(descs) as eng:
+        eng.run_to_end()
+        rec, qa, qb = eng.records(0, qhist=True)
+        assert qa.nbytes < 1 << 20 and np.array_equal(qa.sum(axis=1), rec["n_q"])
+        s, E, M, fam, _ = eng.population(0)
+        assert s.nbytes > 1 << 20
+        cap = eng.runs[0].R_cap
+        R_i, step = C.c_uint32(), C.c_uint32()
+        for buf in (np.empty((cap, N), np.int8), np.full((cap, N), 9, np.int8),
+                    torch.full((cap, N), 9, dtype=torch.int8).pin_memory().numpy()):
+            _lib._check(_lib.load().pa_population(eng.h, 0, _lib._p(buf, C.c_int8), None, None, None, C.byref(R_i),
+                                                  C.byref(step)), "pa_population")
+            assert R_i.value == len(s) and np.array_equal(buf[:len(s)], s)
