@@ -31,10 +31,13 @@ inline void populate_pages(void *p, size_t bytes)
 // there already.
 inline cudaError_t copy_out(void *host, const void *dev, size_t bytes, cudaStream_t s)
 {
-    cudaPointerAttributes at{};
-    if (bytes >= (1u << 20) && cudaPointerGetAttributes(&at, host) == cudaSuccess &&
-        at.type == cudaMemoryTypeUnregistered)
-        populate_pages(host, bytes);
+    if (bytes >= (1u << 20)) {
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, host) != cudaSuccess)
+            (void)cudaGetLastError();  // of this query alone: the copy says what is wrong with the pointer
+        else if (at.type == cudaMemoryTypeUnregistered)
+            populate_pages(host, bytes);
+    }
     return cudaMemcpyAsync(host, dev, bytes, cudaMemcpyDeviceToHost, s);
 }
 

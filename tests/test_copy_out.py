@@ -86,6 +86,10 @@ CASES = {
     "pinned": """char *p = map(n, PROT_READ | PROT_WRITE); fake_type = cudaMemoryTypeHost;
     pa::copy_out(p, nullptr, n, nullptr);
     CHECK(resident(p, n) == 0 && fake_copied == n);""",
+    # a query that fails leaves no error behind for the next check of unrelated work
+    "query_fails": """char *p = map(n, PROT_READ | PROT_WRITE); fake_attr = cudaErrorUnknown;
+    CHECK(pa::copy_out(p, nullptr, n, nullptr) == cudaSuccess && fake_copied == n && resident(p, n) == 0);
+    CHECK(cudaGetLastError() == cudaSuccess);""",
     "small": """char *p = map(n, PROT_READ | PROT_WRITE);
     pa::copy_out(p, nullptr, (1u << 20) - 1, nullptr);
     CHECK(resident(p, n) == 0);""",
