@@ -33,7 +33,6 @@
 #include <utility>
 #include <vector>
 
-#include "pa_copy_out.h"
 #include "pa_internal.cuh"
 
 using namespace pa;

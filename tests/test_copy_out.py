@@ -5,12 +5,15 @@ import subprocess
 
 import pytest
 
-CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2207_05535_gb300", "csrc")
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC, INCLUDE = os.path.join(ROOT, "paper_2207_05535_gb300", "csrc"), os.path.join(ROOT, "include")
 
 FAKE = r"""
 #pragma once
 #include <cstddef>
 #include <cstring>
+#define __host__
+#define __device__
 enum cudaError_t { cudaSuccess = 0, cudaErrorInvalidValue = 1, cudaErrorUnknown = 999 };
 enum cudaMemoryType { cudaMemoryTypeUnregistered = 0, cudaMemoryTypeHost = 1, cudaMemoryTypeManaged = 3 };
 enum cudaMemcpyKind { cudaMemcpyDeviceToHost = 2 };
@@ -42,7 +45,8 @@ MAIN = r"""
 #include <cstdio>
 #include <vector>
 #include <sys/mman.h>
-#include "pa_copy_out.h"
+#include <cuda_runtime.h>
+#include "pa_internal.cuh"
 static size_t resident(void *p, size_t n)
 {
     const size_t page = (size_t)sysconf(_SC_PAGESIZE);
@@ -100,7 +104,7 @@ def _run(tmp_path, body):
     (tmp_path / "cuda_runtime.h").write_text(FAKE)
     src, exe = tmp_path / "t.cpp", tmp_path / "t"
     src.write_text(MAIN.replace("@", body))
-    subprocess.run(["g++", "-std=c++17", "-I", str(tmp_path), "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    subprocess.run(["g++", "-std=c++17", "-I", str(tmp_path), "-I", CSRC, "-I", INCLUDE, str(src), "-o", str(exe)], check=True)
     res = subprocess.run([str(exe)], capture_output=True, text=True)
     assert res.returncode == 0, (res.returncode, res.stdout)
 
