@@ -205,8 +205,9 @@ inline uint32_t plane_words_of(uint32_t L) { return (L * row_pitch(L) + 31) / 32
 // (N + 1), then a tail used by one kernel at a time: the multinomial member
 // list (R_cap u32), or the per-CTA replica totals of the resampling
 // (MAX_RUN_CTAS u32), or the measurement's per-CTA family statistics
-// (MEASURE_PART_WORDS each; a CTA of split_ctas' splits has more than 1365
-// replicas, whose member words are far more than its statistics).
+// (MEASURE_PART_WORDS each; split_ctas cuts pieces of more than 1365 slots, so a
+// run on nc CTAs, whatever the launch's largest population, has more than 1365
+// (nc - 1) slots, whose member words are far more than the statistics).
 constexpr uint64_t MEASURE_PART_WORDS = 4;
 __host__ __device__ inline uint64_t scr_hist_words(uint32_t N) { return (uint64_t(N) + 2) / 2; }
 __host__ __device__ inline uint64_t scr_mhist_off(uint32_t N) { return scr_hist_words(N); }

@@ -61,3 +61,44 @@ def test_clusters_grow_only_with_the_sweeps_work(rule):
     assert rule("pa::small_largest_cluster(L, n, t)", names[:3], list(rows)) == list(rows.values())
     rows = {(16, 1500, 2): 0, (16, 1500, 10): 1, (8, 1500, 2): 0, (8, 1500, 10): 1, (8, 2000, 10): 1, (8, 2000, 1 << 22): 1}
     assert rule("pa::small_steps_per_stage(L, R, th)", ("L", "R", "th"), list(rows)) == list(rows.values())
+
+
+def test_scratch_holds_every_split(tmp_path):
+    """The CTAs that a run gets in a launch of any others: its scratch tail holds their totals and family statistics."""
+    prog, exe = tmp_path / "s.cpp", tmp_path / "s"
+    prog.write_text(r"""
+#include <cstdio>
+#include <cuda_runtime.h>
+#include "pa_internal.cuh"
+int main()
+{
+    const unsigned caps[] = {1, 64, 500, 1024, 1365, 1366, 1367, 2048, 2731, 4096, 4097, 5632, 8192, 9824, 16384, 16385,
+                             24576, 40000, 65536, 100000, 311296, 1000000, 5000000, 4200000000u};
+    const unsigned runs[] = {1, 2, 3, 5, 9, 10, 16, 19, 38, 76, 77, 101, 152, 153, 304, 305, 4096};
+    unsigned widest = 0;
+    for (unsigned n : runs)
+        for (unsigned most : caps) {
+            const unsigned grid = pa::split_ctas(n, most), per_cta = (most + grid - 1) / grid;
+            if (grid < 1 || grid > pa::MAX_RUN_CTAS) return 1;
+            if (pa::resample_nearest_launches(n, most) != (grid == 1 ? 1u : 2u)) return 2;
+            for (unsigned cap : caps) {
+                if (cap > most) continue;
+                const unsigned need = (unsigned)(((unsigned long long)cap + per_cta - 1) / per_cta);  // as the kernels
+                const unsigned nc = need < grid ? need : grid;
+                if (nc > widest) widest = nc;
+                if (nc > 1 && cap <= 1365ull * (nc - 1)) return 3;
+                for (unsigned N : {16u, 256u, 65536u}) {
+                    const unsigned long long tail = pa::scratch_words(N, cap) - pa::scr_tail_off(N);
+                    if (tail < pa::MEASURE_PART_WORDS * nc || 2 * tail < nc) return 4;
+                }
+            }
+        }
+    std::printf("%u\n", widest);
+    return 0;
+}
+""")
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I",
+                    os.path.join(ROOT, "paper_2207_05535_gb300", "csrc"), "-I", CUDA_INCLUDE, str(prog), "-o", str(exe)],
+                   check=True)
+    res = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert res.returncode == 0 and int(res.stdout) > 32
