@@ -179,7 +179,7 @@ inline uint32_t default_shape(const std::vector<SweepCfg> &shapes, SweepLoad loa
     uint32_t pick = 0;
     if (load == LOAD_FEW)
         for (uint32_t c = 1; c < shapes.size(); ++c)
-            if (shapes[c].RPC < shapes[pick].RPC) pick = c;
+            if (shapes[c].RPC <= shapes[pick].RPC) pick = c;  // of two alike the later: L = 12's padded rows
     return pick;
 }
 

@@ -61,9 +61,6 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
-#ifndef PA_PACK_MODE
-#define PA_PACK_MODE 0  // packing of the comparison bits: 0 compare + predicated or (integer ALU), 1 shifted adds
-#endif
 constexpr uint32_t SMEM_BINS = 4096;
 
 __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
@@ -98,12 +95,6 @@ __device__ __forceinline__ void or_if_below(uint32_t &acc, uint32_t u, uint32_t 
 __device__ __forceinline__ void pack_group(uint32_t &B1, uint32_t &B2, const uint4 &u, uint32_t g, uint32_t t1,
                                            uint32_t t2)
 {
-#if PA_PACK_MODE == 1
-    B1 += ((uint32_t)(u.x < t1) << (4 * g)) + ((uint32_t)(u.y < t1) << (4 * g + 1)) +
-          ((uint32_t)(u.z < t1) << (4 * g + 2)) + ((uint32_t)(u.w < t1) << (4 * g + 3));
-    B2 += ((uint32_t)(u.x < t2) << (4 * g)) + ((uint32_t)(u.y < t2) << (4 * g + 1)) +
-          ((uint32_t)(u.z < t2) << (4 * g + 2)) + ((uint32_t)(u.w < t2) << (4 * g + 3));
-#else
     or_if_below(B1, u.x, t1, 1u << (4 * g));
     or_if_below(B1, u.y, t1, 2u << (4 * g));
     or_if_below(B1, u.z, t1, 4u << (4 * g));
@@ -112,7 +103,6 @@ __device__ __forceinline__ void pack_group(uint32_t &B1, uint32_t &B2, const uin
     or_if_below(B2, u.y, t2, 2u << (4 * g));
     or_if_below(B2, u.z, t2, 4u << (4 * g));
     or_if_below(B2, u.w, t2, 8u << (4 * g));
-#endif
 }
 
 __device__ __forceinline__ uint32_t pick(const uint4 &u, uint32_t q)
@@ -1536,28 +1526,22 @@ __global__ void __launch_bounds__(MAXT, MINB) sweep_pow2_kernel(Pool P, const ui
 }
 
 // --------------------------------------------------------------------------
-// Bit-sliced sweep with padded rows, used for L = 12 (Sec. V.A.1): rows of a
-// colour plane are padded to a pitch P in {8, 16, 32} with L P a multiple of 32,
-// so rows tile 32-bit words exactly as in the power-of-two kernel; padding bits are masked out of every flip
-// and popcount and stay 0.  Each thread owns one plane word (32 / P rows); its
-// sites are the compact sublattice indices [kb, kb + (32 / P) L/2), drawn from
-// the same Philox counters as every other path (the groups at either end of
-// the range are shared with the neighbouring words and drawn by both), and
-// each comparison bit is placed at its padded position.
+// Bit-sliced sweep with padded rows, for L = 12 (Sec. V.A.1), where the compact planes below end in a
+// word three quarters empty: rows of 6 sites at a pitch of 8 bits, so that 4 rows fill a word and a
+// plane 3 words; padding bits are masked out of every flip and popcount and stay 0.  Each thread owns
+// one plane word; its 24 sites are the compact sublattice indices 24 w .. 24 w + 23, six whole Philox
+// groups of the same counters as every other path, and each row's comparison bits are placed at
+// their padded position.  Bound by Philox like the other sweeps, three CTAs of 256 threads per SM (two
+// or one: slower).  1.6e6 replicas, theta = 10: 1411 updates/ns against 1135 with compact rows, and
+// against 1219 when the kernel was written for every pitch, with the groups of a word counted at run time.
 // --------------------------------------------------------------------------
-// Compact sites of one padded plane word: RW rows of Lh sites with RW * pitch = 32 and
-// Lh <= pitch, i.e. at most 32 sites, starting anywhere in a Philox group: <= 9 groups.
-constexpr uint32_t PAD_MAX_GROUPS = 9;
-
-#ifndef PA_PAD_MIN_BLOCKS
-#define PA_PAD_MIN_BLOCKS 3  // caps registers at 85: 3 CTAs of 256 threads per SM (measured best of 1, 2, 3)
-#endif
-
-
-template <bool SG, uint32_t PT>  // PT: the row pitch of the runs' lattice size (8, 16 or 32)
-__global__ void __launch_bounds__(256, PA_PAD_MIN_BLOCKS) sweep_pad_kernel(Pool P, const uint32_t *group_runs, const uint32_t *tile_off,
-                                                        uint32_t n_group_runs, SweepCfg cfg)
+template <bool SG>
+__global__ void __launch_bounds__(256, 3) sweep_pad_kernel(Pool P, const uint32_t *group_runs, const uint32_t *tile_off,
+                                                           uint32_t n_group_runs, SweepCfg cfg)
 {
+    constexpr uint32_t Lh = 6, Pt = 8, RW = 32 / Pt, HW = 3, N = 144, NG = RW * Lh / 4;
+    constexpr uint32_t LOW = 0x01010101u, HIGH = LOW << (Lh - 1), EVEN = 0x00FF00FFu;  // a row's first, last site; even rows
+    constexpr uint32_t ROWMASK = (1u << Lh) - 1u, VMASK = LOW * ROWMASK;
     extern __shared__ __align__(16) uint32_t smw[];
     const uint32_t slot = locate_slot(tile_off, n_group_runs, blockIdx.x);
     const uint32_t run = group_runs[slot];
@@ -1570,9 +1554,6 @@ __global__ void __launch_bounds__(256, PA_PAD_MIN_BLOCKS) sweep_pad_kernel(Pool 
     const uint32_t tile0 = (blockIdx.x - tile_off[slot]) * cfg.RPC;
     if (tile0 >= Rn) return;  // uniform over the CTA
 
-    const uint32_t HW = cfg.TPR;  // words per plane = threads per replica
-    constexpr uint32_t Pt = PT;
-    const uint32_t Lh = rd.Lh, N = rd.N;
     const uint32_t rloc = threadIdx.x / HW, w = threadIdx.x - rloc * HW;
     const uint32_t child = tile0 + rloc;
     const bool active = child < Rn;
@@ -1598,18 +1579,7 @@ __global__ void __launch_bounds__(256, PA_PAD_MIN_BLOCKS) sweep_pad_kernel(Pool 
 #pragma unroll
             for (int d = 0; d < 4; ++d) J[c][d] = Jp[(c * 4 + d) * HW + w];
     }
-    // word geometry
-    constexpr bool sub = Pt < 32;  // several rows per word
-    constexpr uint32_t RW = sub ? 32 / Pt : 1u;
-    const uint32_t y0 = w * RW;
-    const uint32_t wp = (w + HW - 1) % HW, wn = (w + 1) % HW;
-    constexpr uint32_t LOW = !sub ? 1u : Pt == 4 ? 0x11111111u : Pt == 8 ? 0x01010101u : 0x00010001u;
-    const uint32_t HIGH = LOW << (Lh - 1);
-    constexpr uint32_t EVEN = Pt == 4 ? 0x0F0F0F0Fu : Pt == 8 ? 0x00FF00FFu : 0x0000FFFFu;  // rows 0, 2, ... (sub)
-    const uint32_t VMASK = LOW * ((1u << Lh) - 1u);                                      // Lh < 32 here
-    const uint32_t kb = y0 * Lh, kend = kb + RW * Lh;                                     // compact sites of the word
-    const uint32_t g0 = kb >> 2, off = kb & 3u, ng = (kend - 4 * g0 + 3) / 4;          // Philox groups (<= 9)
-    const uint32_t ROWMASK = (1u << Lh) - 1u;
+    const uint32_t wp = w == 0 ? HW - 1 : w - 1, wn = w == HW - 1 ? 0 : w + 1;
 
     const unsigned long long T1 = P.thr[rd.thr_off + 2 * i], T2 = P.thr[rd.thr_off + 2 * i + 1];
     const uint32_t t1 = T1 > 0xFFFFFFFFull ? 0xFFFFFFFFu : (uint32_t)T1;
@@ -1627,15 +1597,9 @@ __global__ void __launch_bounds__(256, PA_PAD_MIN_BLOCKS) sweep_pad_kernel(Pool 
         same = o;
         const uint32_t rl = ((o << 1) & ~LOW) | ((o >> (Lh - 1)) & LOW);   // xp <- xp - 1 in the row
         const uint32_t rr = ((o >> 1) & ~HIGH) | ((o << (Lh - 1)) & HIGH); // xp <- xp + 1 in the row
-        if (sub) {
-            up = __funnelshift_l(O[wp], o, Pt);  // row above: position - P
-            dn = __funnelshift_r(o, O[wn], Pt);  // row below: position + P
-            rot = c == 0 ? ((rl & EVEN) | (rr & ~EVEN)) : ((rr & EVEN) | (rl & ~EVEN));
-        } else {
-            up = O[wp];
-            dn = O[wn];
-            rot = ((c + y0) & 1u) == 0 ? rl : rr;
-        }
+        up = __funnelshift_l(O[wp], o, Pt);  // row above: position - P
+        dn = __funnelshift_r(o, O[wn], Pt);  // row below: position + P
+        rot = c == 0 ? ((rl & EVEN) | (rr & ~EVEN)) : ((rr & EVEN) | (rl & ~EVEN));
     };
 
     for (uint32_t t = 0; t < rd.theta; ++t) {
@@ -1650,48 +1614,14 @@ __global__ void __launch_bounds__(256, PA_PAD_MIN_BLOCKS) sweep_pad_kernel(Pool 
                 const uint32_t a = x1 ^ x2, b = x1 & x2, e = x3 ^ x4, f = x3 & x4;
                 const uint32_t c0 = a ^ e, ge2 = b | f | (a & e);
                 const uint32_t ctr3 = (TAG_SWEEP << 24) | (t << 1) | c;
-                // comparison bits of the word's compact sites kb..kend-1, in compact order from
-                // bit `off` of C1 / C2 (the Philox groups of 4 start at kb & ~3) ...
-#if PA_PACK_MODE == 1
-                unsigned long long C1 = 0, C2 = 0;
+                uint32_t C1 = 0, C2 = 0, B1 = 0, B2 = 0;  // comparison bits in compact order, then padded
 #pragma unroll
-                for (uint32_t q = 0; q < PAD_MAX_GROUPS; ++q) {
-                    if (q < ng) {
-                        const uint4 u = philox_rk<false>(g0 + q, child, ctr3, hi1_0, lo1_0, K);
-                        C1 |= (unsigned long long)((uint32_t)(u.x < t1) | ((uint32_t)(u.y < t1) << 1) |
-                                                   ((uint32_t)(u.z < t1) << 2) | ((uint32_t)(u.w < t1) << 3))
-                              << (4 * q);
-                        C2 |= (unsigned long long)((uint32_t)(u.x < t2) | ((uint32_t)(u.y < t2) << 1) |
-                                                   ((uint32_t)(u.z < t2) << 2) | ((uint32_t)(u.w < t2) << 3))
-                              << (4 * q);
-                    }
-                }
-#else
-                // groups 0..7 fill the low words, group 8 the high words (positions 32..35)
-                uint32_t C1l = 0, C2l = 0, C1h = 0, C2h = 0;
+                for (uint32_t q = 0; q < NG; ++q)
+                    pack_group(C1, C2, philox_rk<false>(NG * w + q, child, ctr3, hi1_0, lo1_0, K), q, t1, t2);
 #pragma unroll
-                for (uint32_t q = 0; q < PAD_MAX_GROUPS - 1; ++q) {
-                    if (q < ng) {
-                        const uint4 u = philox_rk<false>(g0 + q, child, ctr3, hi1_0, lo1_0, K);
-                        pack_group(C1l, C2l, u, q, t1, t2);
-                    }
-                }
-                if (ng == PAD_MAX_GROUPS) {
-                    const uint4 u = philox_rk<false>(g0 + PAD_MAX_GROUPS - 1, child, ctr3, hi1_0, lo1_0, K);
-                    pack_group(C1h, C2h, u, 0, t1, t2);
-                }
-                const unsigned long long C1 = ((unsigned long long)C1h << 32) | C1l;
-                const unsigned long long C2 = ((unsigned long long)C2h << 32) | C2l;
-#endif
-                // ... then each row's Lh bits moved to its padded position r * Pt
-                uint32_t B1 = 0, B2 = 0;
-#pragma unroll
-                for (uint32_t r = 0; r < 8; ++r) {
-                    if (r < RW) {
-                        const uint32_t sh = off + r * Lh;
-                        B1 |= ((uint32_t)(C1 >> sh) & ROWMASK) << (r * Pt);
-                        B2 |= ((uint32_t)(C2 >> sh) & ROWMASK) << (r * Pt);
-                    }
+                for (uint32_t r = 0; r < RW; ++r) {
+                    B1 |= ((C1 >> (r * Lh)) & ROWMASK) << (r * Pt);
+                    B2 |= ((C2 >> (r * Lh)) & ROWMASK) << (r * Pt);
                 }
                 const uint32_t flip = (ge2 | (c0 & (B1 | all1)) | B2 | all2) & VMASK;
                 own[c] = S ^ flip;
@@ -4248,9 +4178,8 @@ std::vector<SweepCfg> sweep_candidates(uint32_t L, int allow_fast)
         }
         if (CW <= 128) shape(128, 1, CW <= 4 ? LOAD_ANY : few);
     }
-    // Padded rows draw only the 6 Philox groups that a word of 4 rows holds at L = 12, where the
-    // compact planes end in a word three quarters empty: 1218 against 1138 updates/ns there; at
-    // every other size tried (6 to 62) the compact rows are 10 to 55 % faster.
+    // Padded rows: 1411 against 1135 updates/ns at L = 12; at every other size tried (6 to 62) the compact
+    // rows are 10 to 55 % faster.
     if (allow_fast && L == 12) {
         for (uint32_t target : {128u, 256u}) {
             SweepCfg c{};
@@ -4343,9 +4272,9 @@ void launch_sweep(const Pool &P, const uint32_t *group_runs, const uint32_t *til
         else
             PA_SWEEP_COMPACT(1024, 1, false, 1);
 #undef PA_SWEEP_COMPACT
-    } else if (cfg.fast == 2) {  // padded rows of pitch 8
-        any_glass ? sweep_pad_kernel<true, 8><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg)
-                  : sweep_pad_kernel<false, 8><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg);
+    } else if (cfg.fast == 2) {  // padded rows, L = 12
+        any_glass ? sweep_pad_kernel<true><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg)
+                  : sweep_pad_kernel<false><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg);
     } else if (!cfg.fast && cfg.G <= cfg.TPR && cfg.block <= 512)
         sweep_kernel<true, 512><<<grid, cfg.block, cfg.smem, s>>>(P, group_runs, tile_off, n_group_runs, cfg);
     else if (!cfg.fast)
