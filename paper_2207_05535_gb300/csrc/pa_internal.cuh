@@ -90,9 +90,9 @@ __host__ __device__ inline uint32_t run_ctas(uint32_t R_cap)
 // resampling and the measurement: run_ctas, or more where the launch leaves SMs idle.  A CTA takes
 // about 7 us and 1 us per 1000 replicas, and splitting a population 4 us for the second resampling
 // launch; with two CTAs per SM, 304 run at once.  The split is taken where that predicts a gain of 15 %.
-// One run of R = 16000: resampling 24.0 -> 16.9 us, measurement 23.8 -> 19.7; of R = 64000: 32.1 ->
-// 16.6, 28.1 -> 22.4; 48 of R = 50000: 43.8 -> 34.8, 38.1 -> 32.0.  A launch that fills the GPU
-// gains nothing: 200 runs of R = 20000 take 44 and 43 us with 2 CTAs each, 45 and 43 with 3.
+// One run of R = 16000: resampling 20.8 -> 15.8 us, measurement 21.8 -> 17.5; of R = 64000: 27.0 -> 15.9, 26.0 -> 21.0;
+// 48 of R = 50000: 37 -> 29, 36 -> 30; 100 of R = 9000 19.0 -> 19.8, 21.9 -> 21.6.  A launch that fills the GPU gains
+// nothing: 200 runs of R = 20000 take 42 and 42 us with 2 CTAs each.
 inline uint32_t split_ctas(uint32_t n_runs, uint32_t max_Rcap)
 {
     const uint32_t least = run_ctas(max_Rcap);
@@ -224,7 +224,7 @@ inline uint64_t scratch_words(uint32_t N, uint32_t R_cap)
 }
 
 // Small populations annealed by one launch per step (anneal_small_kernel): one
-// thread-block cluster per run, cluster size small_cluster().
+// thread-block cluster per run (small_shape, small_shape_ahead).
 constexpr uint32_t SMALL_MAX_RCAP = 8192;
 constexpr uint32_t SMALL_MAX_CTAS = 16;  // largest cluster (above 8 by the non-portable opt-in)
 inline bool small_eligible(const RunDev &x)

@@ -686,9 +686,9 @@ constexpr uint32_t COUNTS_BATCH = 4;           // replicas per thread in flight
 constexpr uint32_t PARENT_BATCH = 8;           // rows of 32 copy numbers a warp loads at once
 // A replica with more copies than this has its row's children written by the whole warp: written by
 // its own lane, a step that leaves few families is a chain of one store after another, and three times
-// slower again in the split kernel than fused (L = 32, dbeta = 0.08, the first steps of a quench: one run of
-// R = 9000 48 us in one CTA, 104 split, 19 now; 20 of R = 24000 600 -> 48).  At dbeta = 0.01 few rows
-// have one: 16.7 -> 15.4 us for either split population.
+// slower again in the split kernel than fused (L = 32, dbeta = 0.08, the first steps of a quench: five runs of
+// R = 9000 75 us in one CTA each, 224 split, 34 now; 20 of R = 24000 600 -> 71).  At dbeta = 0.01 few rows have
+// one.
 constexpr uint32_t PARENT_OWN_COPIES = 8;
 
 struct RunChunk {
@@ -859,7 +859,10 @@ __global__ void __launch_bounds__(RESAMPLE_THREADS, 2) resample_counts_kernel(Po
         reinterpret_cast<uint32_t *>(P.scratch + rd.scr_off + scr_tail_off(rd.N))[blockIdx.y] = sum;
 }
 
-__global__ void __launch_bounds__(RESAMPLE_THREADS) resample_parents_kernel(Pool P, const uint32_t *runs, uint32_t per_cta)
+// Three CTAs per SM (40 registers, a few of them spilled): with 56 registers and two, the 400 CTAs of 200 runs of R = 20000
+// take a second, nearly empty wave (both resampling launches 45.8 us, 41.7 with three), while a quench's steps
+// are faster (26 against 34 us in the case above).
+__global__ void __launch_bounds__(RESAMPLE_THREADS, 3) resample_parents_kernel(Pool P, const uint32_t *runs, uint32_t per_cta)
 {
     __shared__ uint32_t sh_u[RESAMPLE_THREADS / 32];
     __shared__ uint32_t sh_off, sh_total;
