@@ -193,7 +193,8 @@ pa_status pa_create(const pa_run_desc *runs, uint32_t n_runs, void *cuda_stream,
  * measures it (when every resident run is
  * small, pa_anneal_step(n) is one launch per lattice size for all n steps, and
  * at L = 8 and 16 the cluster draws each next temperature's random numbers
- * while it measures the current one).
+ * while it measures the current one; larger populations fit a cluster only so,
+ * and their single steps take the per-stage kernels where those are faster).
  * Both paths give identical results; PA_CREATE_GENERIC_SWEEP implies the
  * per-stage kernels.
  * Without it, the first anneal steps of a lattice size time every candidate shape

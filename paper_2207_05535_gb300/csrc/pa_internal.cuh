@@ -86,13 +86,13 @@ __host__ __device__ inline uint32_t run_ctas(uint32_t R_cap)
     return c < 1 ? 1 : (c > MAX_RUN_CTAS ? MAX_RUN_CTAS : c);
 }
 
-// CTAs per run, for the largest of a launch's n_runs populations, of the nearest-integer
-// resampling and the measurement: run_ctas, or more where the launch leaves SMs idle.  A CTA takes
-// about 7 us and 1 us per 1000 replicas, and splitting a population 4 us for the second resampling
-// launch; with two CTAs per SM, 304 run at once.  The split is taken where that predicts a gain of 15 %.
-// One run of R = 16000: resampling 20.8 -> 15.8 us, measurement 21.8 -> 17.5; of R = 64000: 27.0 -> 15.9, 26.0 -> 21.0;
-// 48 of R = 50000: 37 -> 29, 36 -> 30; 100 of R = 9000 19.0 -> 19.8, 21.9 -> 21.6.  A launch that fills the GPU gains
-// nothing: 200 runs of R = 20000 take 42 and 42 us with 2 CTAs each.
+// CTAs per run, for the largest of a launch's n_runs populations, of the nearest-integer resampling
+// and the measurement: run_ctas, or more where the launch leaves SMs idle.  A CTA takes about 7 us and
+// 1 us per 1000 replicas, and splitting a population 4 us for the second resampling launch; with two
+// CTAs per SM, 304 run at once.  The split is taken where that predicts a gain of 15 %. One run of R =
+// 16000: resampling 20.8 -> 15.8 us, measurement 21.8 -> 17.5; of R = 64000: 27.0 -> 15.9, 26.0 ->
+// 21.0; 48 of R = 50000: 37 -> 29, 36 -> 30; 100 of R = 9000 19.0 -> 19.8, 21.9 -> 21.6.  A launch
+// that fills the GPU gains nothing: 200 runs of R = 20000 take 42 and 42 us with 2 CTAs each.
 inline uint32_t split_ctas(uint32_t n_runs, uint32_t max_Rcap)
 {
     const uint32_t least = run_ctas(max_Rcap);
@@ -102,15 +102,16 @@ inline uint32_t split_ctas(uint32_t n_runs, uint32_t max_Rcap)
     return most > least && us(most) < 0.85 * us(least) ? most : least;
 }
 
-// Threads per CTA of the measurement and of the nearest-integer resampling, for the largest
-// population and lattice of a launch.  A run of few replicas is a chain of dependent steps that more
-// threads do not shorten, and with 128 threads eight runs share an SM instead of two: 2048 runs of R = 100, L = 16:
-// measurement 89 -> 37 us a step, resampling 36 -> 15 us.  But the measurement also clears, adds
+// Threads per CTA of the measurement and of the nearest-integer resampling, for the largest population
+// and lattice of a launch.  A run of few replicas is a chain of dependent steps that more threads do
+// not shorten, and with 128 threads eight runs share an SM instead of two: 2048 runs of R = 100, L =
+// 16: measurement 89 -> 37 us a step, resampling 36 -> 15 us.  But the measurement also clears, adds
 // and scans N + 1 levels, which 512 threads do faster until their CTAs, two per SM, no longer run at
-// once.  Measurement with 128 against 512 threads, R = 50 to 150: L = 20 14.9 / 15.2 us (152 runs),
-// L = 32 17.7 / 17.0 (100), 18.4 / 19.6 (200), L = 64 30.9 / 21.7 (152), 33.8 / 26.0 (304), 35.4 / 41.9
-// (400), L = 128 98 / 50 (304), 107 / 120 (700), L = 256 342 / 135 (304), 349 / 239 (400).  Resampling,
-// which scans only the occupied levels: R = 100 8.2 / 8.5 (one run), 8.3 / 12.6 (400), R = 700 10.0 / 8.6, 11.3 / 14.6.
+// once.  Measurement with 128 against 512 threads, R = 50 to 150: L = 20 14.9 / 15.2 us (152 runs), L
+// = 32 17.7 / 17.0 (100), 18.4 / 19.6 (200), L = 64 30.9 / 21.7 (152), 33.8 / 26.0 (304), 35.4 / 41.9
+// (400), L = 128 98 / 50 (304), 107 / 120 (700), L = 256 342 / 135 (304), 349 / 239 (400).
+// Resampling, which scans only the occupied levels: R = 100 8.2 / 8.5 (one run), 8.3 / 12.6 (400), R =
+// 700 10.0 / 8.6, 11.3 / 14.6.
 constexpr uint32_t FEW_REPLICAS = 1024;  // capacity: R of about 740
 inline uint32_t measure_threads(uint32_t n_runs, uint32_t max_Rcap, uint32_t max_N)
 {
@@ -162,12 +163,13 @@ struct SweepCfg {
     uint32_t loads;  // the loads (bits 1 << SweepLoad) at which the tuner times it
 };
 
-// How far the sweeps of a lattice size fill the GPU, from the CTAs that its first launch shape takes: up
-// to two per SM, a few waves of them, or more.  Below two per SM a launch lasts as long as one CTA,
+// How far the sweeps of a lattice size fill the GPU, from the CTAs that its first launch shape takes:
+// up to two per SM, a few waves of them, or more.  Below two per SM a launch lasts as long as one CTA,
 // so one child per thread and small blocks win; from eight per SM on it is the throughput, two
-// children and large blocks; between them whole waves decide (theta = 10, us a launch, one / two children): L = 30
-// 100 CTAs 28 / 48, 190 59 / 74, 750 172 / 166, 1500 336 / 319; L = 64 200 28 / 33, 800 82 / 87, 1600 158 / 153,
-// 13000 1167 / 1124; L = 256 50 64 / 114, 200 181 / 223, 400 356 / 332, 1600 1290 / 1203.
+// children and large blocks; between them whole waves decide (theta = 10, us a launch, one / two
+// children): L = 30 100 CTAs 28 / 48, 190 59 / 74, 750 172 / 166, 1500 336 / 319; L = 64 200 28 / 33,
+// 800 82 / 87, 1600 158 / 153, 13000 1167 / 1124; L = 256 50 64 / 114, 200 181 / 223, 400 356 / 332,
+// 1600 1290 / 1203.
 enum SweepLoad : uint32_t { LOAD_FEW = 0, LOAD_SOME = 1, LOAD_FULL = 2, LOAD_ANY = 7 /* mask */ };
 inline SweepLoad sweep_load(uint64_t ctas) { return ctas < 304 ? LOAD_FEW : ctas < 1216 ? LOAD_SOME : LOAD_FULL; }
 // Few sweeps per launch: kernels of their own for the power-of-two sizes (launch_sweep).
@@ -314,23 +316,25 @@ void launch_unpack_spins(const uint32_t *words, const RunDev &rd, uint32_t t0, u
 struct SmallShape {
     uint32_t cs, block, variant, H, smem;
 };
-// The largest clusters to try.  More than 8 CTAs (the non-portable sizes, at most one such cluster per GPC) shorten
-// the sweeps and lengthen the chain of cluster barriers, so they pay where the sweeps last longer.
-// One temperature per launch, 8 against 16 CTAs (us per temperature, theta = 10; threads that 8 CTAs
-// sweep with): L = 16 R = 400 (461) 34.6 / 28.1 for one run, 35.0 / 37.6 for nine; R = 500 (568) 42.8 / 31.7,
-// 43.7 / 36.6; R = 1000 (1095) 63.3 / 45.2, 66.5 / 66.6; L = 8 R = 400 20.5 / 20.3, 22.2 / 23.6; R = 500 24.5 / 21.0, 24.7 / 22.5.
+// The largest clusters to try.  More than 8 CTAs (the non-portable sizes, at most one such cluster per
+// GPC) shorten the sweeps and lengthen the chain of cluster barriers, so they pay where the sweeps
+// last longer. One temperature per launch, 8 against 16 CTAs (us per temperature, theta = 10; threads
+// that 8 CTAs sweep with): L = 16 R = 400 (461) 34.6 / 28.1 for one run, 35.0 / 37.6 for nine; R = 500
+// (568) 42.8 / 31.7, 43.7 / 36.6; R = 1000 (1095) 63.3 / 45.2, 66.5 / 66.6; L = 8 R = 400 20.5 / 20.3,
+// 22.2 / 23.6; R = 500 24.5 / 21.0, 24.7 / 22.5.
 inline uint32_t small_largest_cluster(uint32_t L, uint32_t n_runs, uint32_t threads_of_8)
 {
     return L != 32 && threads_of_8 > (n_runs <= 8 ? 384u : 512u) ? SMALL_MAX_CTAS : 8u;
 }
-// Several temperatures per launch, where the draws overlap CTA 0's measurement: the line is the sweeps' work
-// per thread, theta times the warps of a CTA of 8 times a thread's draws (a word of L = 8 is drawn by 4
-// lanes, one of L = 16 by one).  8 / 16 CTAs, one run, by theta: L = 16 R = 500 (352 threads) 12.2 / 13.3 at 3, 13.6 /
-// 13.4 at 4, 28.1 / 20.9 at 10; R = 700 (448) 12.3 / 13.2 at 2, 13.9 / 13.5 at 3, 35.5 / 21.2 at 10; L = 8 R = 500 12.3 / 13.1
-// at 10, 20.8 / 15.9 at 20; R = 700 12.6 / 13.2 at 8, 14.7 / 13.5 at 10.  Above 512 threads 16 CTAs at every theta
-// (L = 8 R = 1200 12.5 / 12.4 at 2, 23.8 / 14.2 at 10; L = 16 R = 1000 13.4 / 13.9, 44.7 / 28.2).  Eight or nine runs leave no
-// room for 16 CTAs each (L = 16, theta = 10: R = 500 28.0 / 29.4, R = 600 35.3 / 29.4), five do; up to 384 threads the
-// line is a little higher (L = 16 R = 300 at 5, 224 threads: 12.4 / 13.1).
+// Several temperatures per launch, where the draws overlap CTA 0's measurement: the line is the
+// sweeps' work per thread, theta times the warps of a CTA of 8 times a thread's draws (a word of L = 8
+// is drawn by 4 lanes, one of L = 16 by one).  8 / 16 CTAs, one run, by theta: L = 16 R = 500 (352
+// threads) 12.2 / 13.3 at 3, 13.6 / 13.4 at 4, 28.1 / 20.9 at 10; R = 700 (448) 12.3 / 13.2 at 2, 13.9
+// / 13.5 at 3, 35.5 / 21.2 at 10; L = 8 R = 500 12.3 / 13.1 at 10, 20.8 / 15.9 at 20; R = 700 12.6 /
+// 13.2 at 8, 14.7 / 13.5 at 10.  Above 512 threads 16 CTAs at every theta (L = 8 R = 1200 12.5 / 12.4
+// at 2, 23.8 / 14.2 at 10; L = 16 R = 1000 13.4 / 13.9, 44.7 / 28.2).  Eight or nine runs leave no
+// room for 16 CTAs each (L = 16, theta = 10: R = 500 28.0 / 29.4, R = 600 35.3 / 29.4), five do; up to
+// 384 threads the line is a little higher (L = 16 R = 300 at 5, 224 threads: 12.4 / 13.1).
 inline uint32_t small_largest_cluster_ahead(uint32_t L, uint32_t n_runs, uint32_t threads_of_8, uint32_t theta_max)
 {
     const uint32_t block = (threads_of_8 + 31) / 32 * 32;
@@ -339,9 +343,9 @@ inline uint32_t small_largest_cluster_ahead(uint32_t L, uint32_t n_runs, uint32_
     return block > 512 || (uint64_t)theta_max * block * (L * L / 64) > line ? SMALL_MAX_CTAS : 8u;
 }
 // A run whose populations fit a cluster only when several temperatures are drawn ahead takes a single
-// temperature per launch in several tiles per CTA, which the per-stage kernels beat from this work
-// on (us per temperature, cluster / per stage: L = 16 R = 1500 theta = 2 34.6 / 35.7, theta = 10 85.8 / 46; L = 8 R = 1500 24.4 /
-// 33.2, 43.0 / 40.5; R = 2000 27.9 / 34.2, 53.1 / 41.6).
+// temperature per launch in several tiles per CTA, which the per-stage kernels beat from this work on
+// (us per temperature, cluster / per stage: L = 16 R = 1500 theta = 2 34.6 / 35.7, theta = 10 85.8 /
+// 46; L = 8 R = 1500 24.4 / 33.2, 43.0 / 40.5; R = 2000 27.9 / 34.2, 53.1 / 41.6).
 inline bool small_steps_per_stage(uint32_t L, uint32_t R_max, uint32_t theta_max)
 {
     return (uint64_t)theta_max * R_max * L * L > 800000;

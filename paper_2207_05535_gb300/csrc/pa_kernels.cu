@@ -859,9 +859,9 @@ __global__ void __launch_bounds__(RESAMPLE_THREADS, 2) resample_counts_kernel(Po
         reinterpret_cast<uint32_t *>(P.scratch + rd.scr_off + scr_tail_off(rd.N))[blockIdx.y] = sum;
 }
 
-// Three CTAs per SM (40 registers, a few of them spilled): with 56 registers and two, the 400 CTAs of 200 runs of R = 20000
-// take a second, nearly empty wave (both resampling launches 45.8 us, 41.7 with three), while a quench's steps
-// are faster (26 against 34 us in the case above).
+// Three CTAs per SM (40 registers, a few of them spilled): with 56 registers and two, the 400 CTAs of
+// 200 runs of R = 20000 take a second, nearly empty wave (both resampling launches 45.8 us, 41.7 with
+// three), while a quench's steps are faster (26 against 34 us in the case above).
 __global__ void __launch_bounds__(RESAMPLE_THREADS, 3) resample_parents_kernel(Pool P, const uint32_t *runs, uint32_t per_cta)
 {
     __shared__ uint32_t sh_u[RESAMPLE_THREADS / 32];
