@@ -131,7 +131,7 @@ def test_spread_sweeps_keep_the_order_of_the_callers_stream():
         eng.sync()
         for graph in (False, True):
             with torch.cuda.stream(mine):
-                torch.cuda._sleep(20_000_000)  # about 10 ms on the caller's stream ahead of the sweeps
+                torch.cuda._sleep(100_000_000)  # about 50 ms on the caller's stream ahead of the sweeps
             eng.step(2, graph)
             after = torch.cuda.Event()
             after.record(mine)
